@@ -447,12 +447,37 @@ __global__ void __launch_bounds__(256) k_sweep_field_i8(const FieldI8Params fp) 
 
 // ---- Parisi-Rapuano wheels (Sec. 3.3, Eq. 5) ----
 //
-// One thread per (configuration, row) walks the colour-c sites of its row in
-// increasing x, drawing R(k) = I(k) ^ I(k-61), I(k) = I(k-24) + I(k-55), from
-// the row's wheel; k = t L/2 + j for the j-th site.  The ring of 64 words
-// (I(k) at index k mod 64) sits in shared memory for the launch, ring index
-// major so that the threads of a warp, which share k, hit 32 banks.
-constexpr int kWheelBlock = 128;
+// R(k) = I(k) ^ I(k-61), I(k) = I(k-24) + I(k-55), one wheel per
+// (configuration, row, colour); the j-th colour-c site of a row takes k =
+// t L/2 + j.  In memory a wheel is a ring of 64 words, I(k) at k mod 64, ring
+// index major.  A warp owns kWheelRows consecutive rows of one configuration.
+// It lays their last 64 numbers out in order in shared memory and takes the
+// rows' sites in chunks of up to 32: first the chunk's random numbers, then
+// its updates.
+//
+// Random numbers: the shortest lag is 24, so up to 24 consecutive outputs of
+// a wheel depend on earlier ones only; the warp's two halves draw 16 outputs
+// of each of the 16 rows at a time (every read of a step before its writes).
+// R(k) takes the place of I(k-61), which no later output reads.
+//
+// Updates: the chunk's (row, site) pairs are dealt to the lanes with the site
+// fastest, so that the loads of a warp are contiguous along x, two items per
+// thread in flight.  W (L a multiple of 4, no fields): an item is an aligned
+// 4-byte word of the row with two active sites, the bond tests of its bytes
+// made at once on their sign bits; otherwise an item is one site, by bytes.
+//
+// Bound: the wheels' own bytes (61 words read, L/2 written per row and
+// colour), the spins and the couplings, 18.5 B per update at L = 64.  L=64,
+// 256 x 2, heat bath: 378 us per colour pass, 3.3 TB/s of DRAM traffic, long
+// scoreboard stalls; 1661 us with one thread per row (its byte loads were L
+// apart: L1 94 % busy).  By bytes only (no W) 510 us.
+constexpr int kWheelRows = 16;
+constexpr int kWheelWarps = 4;
+constexpr int kWheelChunk = 32;
+// A row's line: one word of padding, I(k0-64) .. I(k0-1), the chunk's I, and
+// one more word so that 16 rows x 2 neighbouring words hit 32 banks.
+constexpr int kWheelLine = 1 + 64 + kWheelChunk + 1;
+constexpr int kWheelUnroll = 2;
 
 struct WheelParams {
   I8Params b;
@@ -463,72 +488,242 @@ struct WheelParams {
   const uint64_t* fthr;  // field models: [K][kFieldClasses]
 };
 
-template <int D, bool FIELD>
-__global__ void __launch_bounds__(kWheelBlock) k_sweep_wheel_i8(const WheelParams wp) {
-  __shared__ uint32_t ring[64 * kWheelBlock];
+struct WheelWarp {
+  uint32_t line[kWheelRows][kWheelLine];  // R of the chunk's j-th site at 4 + j
+  int4 off[kWheelRows];                   // offsets of the rows y+1, y-1, z+1, z-1 from the row
+  uint64_t T[kFieldClasses];
+};
+
+// Words of kWheelUnroll items of one warp's rows: see k_sweep_wheel_i8 (W).
+// Bits 1..7 of a +-1 byte all equal its sign, so the class u = (u2 u1 u0) of a
+// byte can be read off any three of them: bits 3, 4, 5 give 8 u, the byte
+// offset of its threshold.
+template <int D>
+__device__ __forceinline__ void wheel_words(const WheelWarp& w, uint32_t lane, uint32_t nrow, uint32_t rowbase,
+                                            uint32_t L, uint32_t j0, uint32_t cnt, uint32_t colour, bool inv,
+                                            int8_t* sp, const int8_t* J0, const int8_t* J1, const int8_t* J2) {
+  const uint32_t wc = cnt >> 1, items = nrow * wc, rec = 65536u / wc + 1u;
+  for (uint32_t it = lane; it < items; it += 32u * kWheelUnroll) {
+    uint32_t self[kWheelUnroll], cls[kWheelUnroll], at[kWheelUnroll], par[kWheelUnroll];
+    uint2 rr[kWheelUnroll];
+#pragma unroll
+    for (int c = 0; c < kWheelUnroll; ++c) {
+      const uint32_t item = min(it + 32u * (uint32_t)c, items - 1u);  // past the end: repeated, not stored
+      const uint32_t r = (item * rec) >> 16, j = item - r * wc;
+      rr[c] = *(const uint2*)&w.line[r][4u + 2u * j];
+      const int4 o = w.off[r];
+      par[c] = ((uint32_t)o.z ^ colour) & 1u;  // active bytes par, par + 2
+      const uint32_t base = rowbase + r * L, x = 2u * j0 + 4u * j, i = base + x;
+      // the word that holds the neighbour outside this one: the next word's
+      // first byte (par = 1) or the previous word's last
+      const uint32_t adj = par[c] ? (x + 4u == L ? base : i + 4u) : (x == 0u ? base + L - 4u : i - 4u);
+      const uint32_t iym = i + (uint32_t)o.y, izm = i + (uint32_t)(o.w & ~1);
+      auto ld = [](const int8_t* q, uint32_t k) { return *(const uint32_t*)(q + k); };
+      const uint32_t b = ld(sp, i), ba = ld(sp, adj), jx = ld(J0, i), ja = ld(J0, adj);
+      const uint32_t byp = ld(sp, i + (uint32_t)o.x), bym = ld(sp, iym), jy = ld(J1, i), jym = ld(J1, iym);
+      uint32_t bzp = 0, bzm = 0, jz = 0, jzm = 0;
+      if (D == 3) {
+        bzp = ld(sp, i + (uint32_t)(o.z & ~1));
+        bzm = ld(sp, izm);
+        jz = ld(J2, i);
+        jzm = ld(J2, izm);
+      }
+      const uint32_t e0 = b ^ __funnelshift_r(b, ba, 8) ^ jx;
+      const uint32_t e1 = b ^ __funnelshift_l(ba, b, 8) ^ __funnelshift_l(ja, jx, 8);
+      const uint32_t e2 = b ^ byp ^ jy, e3 = b ^ bym ^ jym;
+      const uint32_t sa = e0 ^ e1 ^ e2, ca = (e0 & e1) | (e0 & e2) | (e1 & e2);
+      uint32_t u0, u1, u2;
+      if (D == 3) {
+        const uint32_t e4 = b ^ bzp ^ jz, e5 = b ^ bzm ^ jzm;
+        const uint32_t sb = e3 ^ e4 ^ e5, cb = (e3 & e4) | (e3 & e5) | (e4 & e5), k = sa & sb;
+        u0 = sa ^ sb;
+        u1 = ca ^ cb ^ k;
+        u2 = (ca & cb) | (ca & k) | (cb & k);
+      } else {
+        const uint32_t k = sa & e3;
+        u0 = sa ^ e3;
+        u1 = ca ^ k;
+        u2 = ca & k;
+      }
+      cls[c] = (u0 & 0x08080808u) | (u1 & 0x10101010u) | (u2 & 0x20202020u);
+      self[c] = b;
+      at[c] = i;
+    }
+#pragma unroll
+    for (int c = 0; c < kWheelUnroll; ++c) {
+      if (it + 32u * (uint32_t)c >= items) break;
+      const uint32_t q = cls[c] >> (8u * par[c]);
+      const uint64_t T0 = *(const uint64_t*)((const char*)w.T + (q & 0xFFu));
+      const uint64_t T1 = *(const uint64_t*)((const char*)w.T + ((q >> 16) & 0xFFu));
+      const uint32_t f0 = ((uint64_t)rr[c].x < T0) != inv ? 0xFEu : 0u;
+      const uint32_t f1 = ((uint64_t)rr[c].y < T1) != inv ? 0xFE0000u : 0u;
+      *(uint32_t*)(sp + at[c]) = self[c] ^ ((f0 | f1) << (8u * par[c]));  // +-1 negated: all bits but bit 0
+    }
+  }
+}
+
+template <int D, bool FIELD, bool W>
+__global__ void __launch_bounds__(32 * kWheelWarps, FIELD ? 6 : 8) k_sweep_wheel_i8(const WheelParams wp) {
+  __shared__ __align__(16) WheelWarp sm[kWheelWarps];
   const I8Params& p = wp.b;
+  WheelWarp& w = sm[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31u;
   const uint32_t L = (uint32_t)p.L, h = L / 2u, rows = wp.rows;
-  const uint64_t total = (uint64_t)p.slots * p.S * rows;
   const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
   const uint32_t k0 = tk.lo * h;  // t L/2 mod 2^32; only k mod 64 is used
-  const uint32_t tid = threadIdx.x;
-  for (uint64_t base = (uint64_t)blockIdx.x * kWheelBlock; base < total; base += (uint64_t)gridDim.x * kWheelBlock) {
-    const uint64_t idx = base + tid;
-    const bool active = idx < total;
-    const uint32_t lat = active ? (uint32_t)(idx / rows) : 0u;
-    const uint32_t row = active ? (uint32_t)(idx - (uint64_t)lat * rows) : 0u;
-    uint32_t* wg = wp.wheels + ((size_t)lat * 2 + (size_t)p.colour) * 64 * rows + row;
-    if (active)
-      for (int m = 0; m < 64; ++m) ring[m * kWheelBlock + tid] = wg[(size_t)m * rows];
-    if (active) {
-      const int sigma = (int)(lat / (uint32_t)p.S);
-      const int s = (int)(lat - (uint32_t)sigma * (uint32_t)p.S);
-      const uint32_t y = row % L, z = row / L;  // D = 2: z = 0
-      const uint32_t x0 = (uint32_t)(p.colour ^ (int)(y + z)) & 1u;
-      int8_t* sp = p.spins + (size_t)lat * p.N;
-      const int8_t* Jp = p.J + (size_t)s * D * p.N;
-      const int8_t* xo = FIELD ? wp.occ + (size_t)s * p.N : nullptr;
-      const int tslot = sigma / p.R, a = sigma - tslot * p.R;
-      const int kt = p.temp_of[((size_t)s * p.R + a) * p.K + tslot];
-      // rows of the neighbours along y and z
-      const uint32_t yp = (y + 1u == L ? 0u : y + 1u) + L * z, ym = (y == 0u ? L - 1u : y - 1u) + L * z;
-      const uint32_t zp = y + L * (z + 1u == L ? 0u : z + 1u), zm = y + L * (z == 0u ? L - 1u : z - 1u);
-      for (uint32_t j = 0; j < h; ++j) {
-        const uint32_t k = k0 + j;
-        const uint32_t Ik = ring[((k - 24u) & 63u) * kWheelBlock + tid] + ring[((k - 55u) & 63u) * kWheelBlock + tid];
-        const uint32_t r = Ik ^ ring[((k - 61u) & 63u) * kWheelBlock + tid];
-        ring[(k & 63u) * kWheelBlock + tid] = Ik;
-        const uint32_t x = 2u * j + x0;
-        const uint32_t i = x + L * row;
-        if (FIELD && !xo[i]) continue;
-        const uint32_t xp = (x + 1u == L ? 0u : x + 1u) + L * row;
-        const uint32_t xm = (x == 0u ? L - 1u : x - 1u) + L * row;
-        const uint32_t iyp = x + L * yp, iym = x + L * ym;
-        const int si = sp[i];
-        uint64_t T;
-        if (FIELD) {
-          int phi = Jp[i] * xo[xp] * sp[xp] + Jp[xm] * xo[xm] * sp[xm] + Jp[p.N + i] * xo[iyp] * sp[iyp] +
-                    Jp[p.N + iym] * xo[iym] * sp[iym];
-          if (D == 3) {
-            const uint32_t izp = x + L * zp, izm = x + L * zm;
-            phi += Jp[2u * p.N + i] * xo[izp] * sp[izp] + Jp[2u * p.N + izm] * xo[izm] * sp[izm];
-          }
-          const int v = si * phi;
-          const int f = si * wp.hs[(size_t)s * p.N + i] > 0;
-          T = wp.fthr[(size_t)kt * kFieldClasses + (v + 2 * D) * 2 + f];
-        } else {
-          int u = (Jp[i] * si * sp[xp] < 0) + (Jp[xm] * si * sp[xm] < 0) + (Jp[p.N + i] * si * sp[iyp] < 0) +
-                  (Jp[p.N + iym] * si * sp[iym] < 0);
-          if (D == 3) {
-            const uint32_t izp = x + L * zp, izm = x + L * zm;
-            u += (Jp[2u * p.N + i] * si * sp[izp] < 0) + (Jp[2u * p.N + izm] * si * sp[izm] < 0);
-          }
-          T = p.thr[(size_t)kt * kMaxClasses + u];
-        }
-        const bool less = (uint64_t)r < T;
-        if (less != (p.inv != 0)) sp[i] = (int8_t)(-si);
+  // block -> configuration (block-uniform base pointers) and its warps' rows;
+  // the slots of a sample next to each other, so that its couplings are read
+  // from memory once
+  const uint32_t per_block = kWheelRows * (blockDim.x >> 5);
+  const uint32_t blocks = (rows + per_block - 1u) / per_block;
+  const uint32_t cfg = blockIdx.x / blocks;
+  const uint32_t row0 = (blockIdx.x - cfg * blocks) * per_block + kWheelRows * (threadIdx.x >> 5);
+  if (row0 >= rows) return;  // warps are independent: no block barrier below
+  const uint32_t s = cfg / (uint32_t)p.slots, sigma = cfg - s * (uint32_t)p.slots;
+  const size_t lat = (size_t)sigma * p.S + s;
+  const uint32_t nrow = min((uint32_t)kWheelRows, rows - row0);
+  uint32_t* wg = wp.wheels + (lat * 2 + (size_t)p.colour) * 64 * rows + row0;
+  // 16-byte accesses of 4 rows where every ring line is aligned (nrow is then a multiple of 4 too)
+  const bool quads = (rows & 3u) == 0u;
+  if (quads) {
+    const uint32_t q = 4u * (lane & 3u);
+    if (q < nrow)
+#pragma unroll
+      for (uint32_t e = lane >> 2; e < 64u; e += 8u) {
+        const uint4 v = *(const uint4*)(wg + (size_t)((k0 + e) & 63u) * rows + q);
+        w.line[q][1 + e] = v.x;
+        w.line[q + 1][1 + e] = v.y;
+        w.line[q + 2][1 + e] = v.z;
+        w.line[q + 3][1 + e] = v.w;
       }
-      for (int m = 0; m < 64; ++m) wg[(size_t)m * rows] = ring[m * kWheelBlock + tid];
+  } else if ((lane & 15u) < nrow) {
+    for (uint32_t e = lane >> 4; e < 64u; e += 2u)
+      w.line[lane & 15u][1 + e] = wg[(size_t)((k0 + e) & 63u) * rows + (lane & 15u)];
+  }
+  const int tslot = (int)sigma / p.R, a = (int)sigma - tslot * p.R;
+  const int kt = p.temp_of[((size_t)s * p.R + a) * p.K + tslot];
+  if (FIELD)
+    w.T[lane] = wp.fthr[(size_t)kt * kFieldClasses + lane];
+  else if (lane < (uint32_t)kMaxClasses)
+    w.T[lane] = p.thr[(size_t)kt * kMaxClasses + lane];
+  if (lane < (uint32_t)kWheelRows) {
+    const uint32_t row = row0 + lane, y = row % L, z = row / L;  // D = 2: z = 0
+    const int Li = (int)L, l2 = Li * (Li - 1);
+    int4 o;
+    o.x = y + 1u == L ? -l2 : Li;
+    o.y = y == 0u ? l2 : -Li;
+    o.z = o.w = (int)((y + z) & 1u);
+    if (D == 3) {
+      // the row's parity rides in bit 0 of the z offsets, which are even
+      o.z |= z + 1u == L ? -l2 * Li : Li * Li;
+      o.w |= z == 0u ? l2 * Li : -Li * Li;
+    }
+    w.off[lane] = o;
+  }
+  int8_t* sp = p.spins + lat * p.N;
+  const int8_t* J0 = p.J + (size_t)s * D * p.N;
+  const int8_t* J1 = J0 + p.N;
+  const int8_t* J2 = J1 + p.N;  // D = 3 only
+  const int8_t* xo = FIELD ? wp.occ + (size_t)s * p.N : nullptr;
+  const int8_t* hs = FIELD ? wp.hs + (size_t)s * p.N : nullptr;
+  const uint32_t rowbase = row0 * L;
+  for (uint32_t j0 = 0; j0 < h; j0 += kWheelChunk) {
+    const uint32_t cnt = min((uint32_t)kWheelChunk, h - j0);
+    __syncwarp();
+    const uint32_t r16 = lane & 15u, half = lane >> 4;
+    if (j0 > 0u) {  // the last 64 numbers become the line's head again
+      for (uint32_t e = half; e < 64u; e += 2u) {
+        const uint32_t v = w.line[r16][1 + kWheelChunk + e];
+        __syncwarp();
+        w.line[r16][1 + e] = v;
+        __syncwarp();
+      }
+    }
+    uint32_t* ln = &w.line[r16][1 + half];
+#pragma unroll
+    for (uint32_t b = 0; b < (uint32_t)kWheelChunk; b += 16u) {
+      if (b < cnt) {
+        uint32_t I[8], Rn[8];
+#pragma unroll
+        for (uint32_t i = 0; i < 8u; ++i) {
+          const uint32_t j = b + 2u * i;  // output j + half
+          I[i] = ln[64 - 24 + j] + ln[64 - 55 + j];
+          Rn[i] = I[i] ^ ln[64 - 61 + j];
+        }
+        __syncwarp();
+#pragma unroll
+        for (uint32_t i = 0; i < 8u; ++i) {
+          const uint32_t j = b + 2u * i;
+          ln[64 + j] = I[i];
+          ln[64 - 61 + j] = Rn[i];
+        }
+        __syncwarp();
+      }
+    }
+    if (W) {
+      wheel_words<D>(w, lane, nrow, rowbase, L, j0, cnt, (uint32_t)p.colour, p.inv != 0, sp, J0, J1, J2);
+    } else {
+      // item = r cnt + j; r by a 16-bit reciprocal, exact for item < 512, cnt <= 32
+      const uint32_t items = nrow * cnt, inv = 65536u / cnt + 1u;
+      for (uint32_t it = lane; it < items; it += 32u * kWheelUnroll) {
+        int si[kWheelUnroll], v[kWheelUnroll], f[kWheelUnroll];
+        uint32_t ix[kWheelUnroll], rr[kWheelUnroll];
+        bool live[kWheelUnroll];
+#pragma unroll
+        for (int c = 0; c < kWheelUnroll; ++c) {
+          const uint32_t item = it + 32u * (uint32_t)c;
+          live[c] = item < items;
+          si[c] = v[c] = f[c] = 0;
+          ix[c] = rr[c] = 0;
+          if (!live[c]) continue;
+          const uint32_t r = (item * inv) >> 16, j = item - r * cnt;
+          rr[c] = w.line[r][4u + j];
+          const int4 o = w.off[r];
+          const uint32_t x = 2u * (j0 + j) + (((uint32_t)o.z ^ (uint32_t)p.colour) & 1u);
+          const uint32_t base = rowbase + r * L, i = base + x;
+          const uint32_t ixp = x + 1u == L ? base : i + 1u, ixm = x == 0u ? base + L - 1u : i - 1u;
+          const uint32_t iyp = i + (uint32_t)o.x, iym = i + (uint32_t)o.y;
+          const uint32_t izp = i + (uint32_t)(o.z & ~1), izm = i + (uint32_t)(o.w & ~1);
+          ix[c] = i;
+          const int b = sp[i];
+          si[c] = b;
+          // spins and couplings are +-1, so the bond term s_i s_j J is the XOR of the three
+          const int txp = b ^ sp[ixp] ^ J0[i], txm = b ^ sp[ixm] ^ J0[ixm];
+          const int typ = b ^ sp[iyp] ^ J1[i], tym = b ^ sp[iym] ^ J1[iym];
+          int tzp = 0, tzm = 0;
+          if (D == 3) {
+            tzp = b ^ sp[izp] ^ J2[i];
+            tzm = b ^ sp[izm] ^ J2[izm];
+          }
+          if (FIELD) {
+            live[c] = xo[i] != 0;
+            v[c] = txp * xo[ixp] + txm * xo[ixm] + typ * xo[iyp] + tym * xo[iym];
+            if (D == 3) v[c] += tzp * xo[izp] + tzm * xo[izm];
+            f[c] = b == hs[i];
+          } else {
+            v[c] = txp + txm + typ + tym + tzp + tzm;
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < kWheelUnroll; ++c) {
+          if (!live[c]) continue;
+          const uint64_t T = w.T[FIELD ? (v[c] + 2 * D) * 2 + f[c] : (2 * D - v[c]) >> 1];
+          const bool less = (uint64_t)rr[c] < T;
+          if (less != (p.inv != 0)) sp[ix[c]] = (int8_t)(-si[c]);
+        }
+      }
+    }
+    // the ring positions the chunk changed
+    const uint32_t ks = k0 + j0;
+    if (quads) {
+      const uint32_t q = 4u * (lane & 3u);
+      if (q < nrow)
+        for (uint32_t e = lane >> 2; e < cnt; e += 8u)
+          *(uint4*)(wg + (size_t)((ks + e) & 63u) * rows + q) =
+              make_uint4(w.line[q][65 + e], w.line[q + 1][65 + e], w.line[q + 2][65 + e], w.line[q + 3][65 + e]);
+    } else if ((lane & 15u) < nrow) {
+      for (uint32_t e = lane >> 4; e < cnt; e += 2u)
+        wg[(size_t)((ks + e) & 63u) * rows + (lane & 15u)] = w.line[lane & 15u][65 + e];
     }
   }
 }
@@ -1829,13 +2024,23 @@ cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
   p.t_dev = lat.capturing ? lat.t_dev : nullptr;
   if (lat.rng == IANUS_RNG_WHEEL) {
     const WheelParams wp{p, lat.wheels, lat.rows, lat.hs, lat.occ, lat.fthr};
-    const unsigned wgrid = grid_for((uint64_t)lat.slots * lat.S * lat.rows, kWheelBlock, 152u * 12u);
-    if (lat.field)
-      lat.D == 3 ? k_sweep_wheel_i8<3, true><<<wgrid, kWheelBlock, 0, lat.stream>>>(wp)
-                 : k_sweep_wheel_i8<2, true><<<wgrid, kWheelBlock, 0, lat.stream>>>(wp);
-    else
-      lat.D == 3 ? k_sweep_wheel_i8<3, false><<<wgrid, kWheelBlock, 0, lat.stream>>>(wp)
-                 : k_sweep_wheel_i8<2, false><<<wgrid, kWheelBlock, 0, lat.stream>>>(wp);
+    const uint32_t tiles = (lat.rows + kWheelRows - 1) / kWheelRows;
+    const uint32_t warps = std::min<uint32_t>(tiles, kWheelWarps);
+    const uint64_t wgrid = (uint64_t)lat.slots * lat.S * ((tiles + warps - 1) / warps);
+    if (wgrid > 0x7fffffffull) return cudaErrorInvalidConfiguration;  // beyond any device's memory
+    const bool words = !lat.field && lat.L % 4 == 0;
+    const void* k = lat.field ? (lat.D == 3 ? (const void*)k_sweep_wheel_i8<3, true, false>
+                                            : (const void*)k_sweep_wheel_i8<2, true, false>)
+                    : words   ? (lat.D == 3 ? (const void*)k_sweep_wheel_i8<3, false, true>
+                                            : (const void*)k_sweep_wheel_i8<2, false, true>)
+                              : (lat.D == 3 ? (const void*)k_sweep_wheel_i8<3, false, false>
+                                            : (const void*)k_sweep_wheel_i8<2, false, false>);
+    void* args[] = {(void*)&wp};
+    cudaError_t e = cudaLaunchKernel(k, dim3((unsigned)wgrid), dim3(32 * warps), args, 0, lat.stream);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
     return cudaGetLastError();
   }
   const uint64_t total = (uint64_t)lat.slots * lat.S * p.half;
