@@ -453,7 +453,8 @@ __global__ void __launch_bounds__(256) k_sweep_field_i8(const FieldI8Params fp) 
 // index major.  A warp owns kWheelRows consecutive rows of one configuration.
 // It lays their last 64 numbers out in order in shared memory and takes the
 // rows' sites in chunks of up to 32: first the chunk's random numbers, then
-// its updates.
+// its updates.  Where such warps would be few (fewer than 8 a SM) a warp takes
+// 8 or 4 rows: the pass then lasts as long as one warp's dependent loads.
 //
 // Random numbers: the shortest lag is 24, so up to 24 consecutive outputs of
 // a wheel depend on earlier ones only; the warp's two halves draw 16 outputs
@@ -483,6 +484,7 @@ struct WheelParams {
   I8Params b;
   uint32_t* wheels;      // [slots * S][2][64][rows]
   uint32_t rows;
+  uint32_t per_warp;     // rows of a warp: kWheelRows, or 8 or 4 of them
   const int8_t* hs;      // field models: [S][N], else null
   const int8_t* occ;
   const uint64_t* fthr;  // field models: [K][kFieldClasses]
@@ -574,14 +576,14 @@ __global__ void __launch_bounds__(32 * kWheelWarps, FIELD ? 6 : 8) k_sweep_wheel
   // block -> configuration (block-uniform base pointers) and its warps' rows;
   // the slots of a sample next to each other, so that its couplings are read
   // from memory once
-  const uint32_t per_block = kWheelRows * (blockDim.x >> 5);
+  const uint32_t per_block = wp.per_warp * (blockDim.x >> 5);
   const uint32_t blocks = (rows + per_block - 1u) / per_block;
   const uint32_t cfg = blockIdx.x / blocks;
-  const uint32_t row0 = (blockIdx.x - cfg * blocks) * per_block + kWheelRows * (threadIdx.x >> 5);
+  const uint32_t row0 = (blockIdx.x - cfg * blocks) * per_block + wp.per_warp * (threadIdx.x >> 5);
   if (row0 >= rows) return;  // warps are independent: no block barrier below
   const uint32_t s = cfg / (uint32_t)p.slots, sigma = cfg - s * (uint32_t)p.slots;
   const size_t lat = (size_t)sigma * p.S + s;
-  const uint32_t nrow = min((uint32_t)kWheelRows, rows - row0);
+  const uint32_t nrow = min(wp.per_warp, rows - row0);
   uint32_t* wg = wp.wheels + (lat * 2 + (size_t)p.colour) * 64 * rows + row0;
   // 16-byte accesses of 4 rows where every ring line is aligned (nrow is then a multiple of 4 too)
   const bool quads = (rows & 3u) == 0u;
@@ -597,6 +599,7 @@ __global__ void __launch_bounds__(32 * kWheelWarps, FIELD ? 6 : 8) k_sweep_wheel
         w.line[q + 3][1 + e] = v.w;
       }
   } else if ((lane & 15u) < nrow) {
+#pragma unroll 16
     for (uint32_t e = lane >> 4; e < 64u; e += 2u)
       w.line[lane & 15u][1 + e] = wg[(size_t)((k0 + e) & 63u) * rows + (lane & 15u)];
   }
