@@ -1275,6 +1275,15 @@ __global__ void k_init_sites_i8(int8_t* hs, int8_t* occ, int S, uint32_t N, int 
   }
 }
 
+// A block's part of an accumulator: the whole value when it is the
+// configuration's only block, else added (the accumulators start at zero).
+__device__ __forceinline__ void acc_add(int64_t* a, long long v, uint32_t chunks) {
+  if (chunks == 1u)
+    *a = v;
+  else
+    atomicAdd((unsigned long long*)a, (unsigned long long)v);
+}
+
 // Field models, block per configuration: E_J = -sum_bonds J x x s s,
 // M = sum x s, F = sum sign(h) x s (Sec. 4.1 observables of Eq. 2).
 template <int D>
@@ -1282,16 +1291,17 @@ __global__ void __launch_bounds__(256) k_measure_field_i8(const int8_t* __restri
                                                           const int8_t* __restrict__ J,
                                                           const int8_t* __restrict__ hs,
                                                           const int8_t* __restrict__ occ, int64_t* acc, int S,
-                                                          int slots, int L, uint32_t N) {
+                                                          int slots, int L, uint32_t N, uint32_t chunks) {
   __shared__ long long red[3][8];
-  for (uint32_t lat = blockIdx.x; lat < (uint32_t)(slots * S); lat += gridDim.x) {
+  {
+    const uint32_t lat = blockIdx.x / chunks, chunk = blockIdx.x - lat * chunks;
     const int sigma = (int)(lat / (uint32_t)S), s = (int)(lat - (uint32_t)sigma * S);
     const int8_t* sp = spins + (size_t)lat * N;
     const int8_t* Jp = J + (size_t)s * D * N;
     const int8_t* xo = occ + (size_t)s * N;
     const int8_t* hp = hs + (size_t)s * N;
     long long e = 0, m = 0, f = 0;
-    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
+    for (uint32_t i = chunk * blockDim.x + threadIdx.x; i < N; i += chunks * blockDim.x) {
       const uint32_t x = i % (uint32_t)L, y = (i / (uint32_t)L) % (uint32_t)L;
       const uint32_t z = D == 3 ? i / ((uint32_t)L * (uint32_t)L) : 0u;
       const int si = xo[i] * sp[i];
@@ -1326,16 +1336,15 @@ __global__ void __launch_bounds__(256) k_measure_field_i8(const int8_t* __restri
         F += red[2][w];
       }
       int64_t* a = acc + ((size_t)s * slots + sigma) * kAccStride;
-      a[0] = E;
-      a[1] = M;
-      a[2] = F;
+      acc_add(a + 0, E, chunks);
+      acc_add(a + 1, M, chunks);
+      acc_add(a + 2, F, chunks);
     }
-    __syncthreads();
   }
 }
 
-// One temperature, R = 1 or 2 replicas, L a multiple of 16: block per
-// sample, E and M of each replica and (R = 2) the overlap Q of the two
+// One temperature, R = 1 or 2 replicas, L a multiple of 16: `chunks` blocks
+// per sample, E and M of each replica and (R = 2) the overlap Q of the two
 // (Sec. 4.1) in one pass that reads the sample's couplings once.  16 sites
 // of a row per step: a bond (i, j) is unsatisfied iff the sign bits (bit 7)
 // of s_i, J_ij and s_j XOR to 1, so E = 2 U - D N, M = N - 2 n_- and
@@ -1344,15 +1353,16 @@ __global__ void __launch_bounds__(256) k_measure_field_i8(const int8_t* __restri
 template <int D, int R>
 __global__ void __launch_bounds__(256) k_measure_i8_k1(const int8_t* __restrict__ spins,
                                                        const int8_t* __restrict__ J, int64_t* acc, int S, int L,
-                                                       uint32_t N, int want_q) {
+                                                       uint32_t N, int want_q, uint32_t chunks) {
   __shared__ long long red[2 * R + 1][8];
   const uint32_t qrow = (uint32_t)L / 16u, nq = N / 16u, uL = (uint32_t)L;
-  for (uint32_t s = blockIdx.x; s < (uint32_t)S; s += gridDim.x) {
+  {
+    const uint32_t s = blockIdx.x / chunks, chunk = blockIdx.x - s * chunks;
     const int8_t* Jp = J + (size_t)s * D * N;
     uint32_t un[R], ng[R], df = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) un[r] = ng[r] = 0;
-    for (uint32_t q = threadIdx.x; q < nq; q += blockDim.x) {
+    for (uint32_t q = chunk * blockDim.x + threadIdx.x; q < nq; q += chunks * blockDim.x) {
       const uint32_t row = q / qrow, k = q - row * qrow;
       const uint32_t y = row % uL, z = row / uL;
       const uint32_t base = row * uL + 16u * k;
@@ -1411,22 +1421,23 @@ __global__ void __launch_bounds__(256) k_measure_i8_k1(const int8_t* __restrict_
       }
       for (int r = 0; r < R; ++r) {
         int64_t* a = acc + ((size_t)s * R + r) * kAccStride;
-        a[0] = 2ll * t[2 * r] - (long long)D * N;
-        a[1] = (long long)N - 2ll * t[2 * r + 1];
+        acc_add(a + 0, 2ll * t[2 * r] - (chunk ? 0ll : (long long)D * N), chunks);
+        acc_add(a + 1, (chunk ? 0ll : (long long)N) - 2ll * t[2 * r + 1], chunks);
       }
-      if (R == 2 && want_q) acc[(size_t)s * R * kAccStride + 6] = (long long)N - 2ll * t[2 * R];
+      if (R == 2 && want_q) acc_add(acc + (size_t)s * R * kAccStride + 6, (chunk ? 0ll : (long long)N) - 2ll * t[2 * R], chunks);
     }
-    __syncthreads();
   }
 }
 
-// Block per configuration: E = -sum_bonds J s s and M = sum s (Sec. 4.1).
+// Blocks of `chunks` per configuration: E = -sum_bonds J s s and M = sum s
+// (Sec. 4.1), added to the zeroed accumulators.
 template <int D>
 __global__ void __launch_bounds__(256) k_measure_i8(const int8_t* __restrict__ spins,
                                                     const int8_t* __restrict__ J, int64_t* acc, int S,
-                                                    int R, int slots, int L, uint32_t N) {
+                                                    int R, int slots, int L, uint32_t N, uint32_t chunks) {
   __shared__ long long red[3][8];
-  for (uint32_t lat = blockIdx.x; lat < (uint32_t)(slots * S); lat += gridDim.x) {
+  {
+    const uint32_t lat = blockIdx.x / chunks, chunk = blockIdx.x - lat * chunks;
     const int sigma = (int)(lat / (uint32_t)S), s = (int)(lat - (uint32_t)sigma * S);
     const int8_t* sp = spins + (size_t)lat * N;
     const int8_t* Jp = J + (size_t)s * D * N;
@@ -1438,7 +1449,7 @@ __global__ void __launch_bounds__(256) k_measure_i8(const int8_t* __restrict__ s
       // n_- counted by popcounts of sign-bit masks
       const uint32_t qrow = (uint32_t)L / 16u, nq = N / 16u;
       uint32_t un = 0, ng = 0;
-      for (uint32_t q = threadIdx.x; q < nq; q += blockDim.x) {
+      for (uint32_t q = chunk * blockDim.x + threadIdx.x; q < nq; q += chunks * blockDim.x) {
         const uint32_t row = q / qrow, k = q - row * qrow;
         const uint32_t y = row % (uint32_t)L, z = row / (uint32_t)L;
         const uint32_t base = row * (uint32_t)L + 16u * k;
@@ -1470,7 +1481,7 @@ __global__ void __launch_bounds__(256) k_measure_i8(const int8_t* __restrict__ s
       e = 2ll * un;  // - D N added once per configuration below
       m = -2ll * ng;
     } else
-    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
+    for (uint32_t i = chunk * blockDim.x + threadIdx.x; i < N; i += chunks * blockDim.x) {
       const uint32_t x = i % (uint32_t)L, y = (i / (uint32_t)L) % (uint32_t)L;
       const uint32_t z = D == 3 ? i / ((uint32_t)L * (uint32_t)L) : 0u;
       const int si = sp[i];
@@ -1500,15 +1511,14 @@ __global__ void __launch_bounds__(256) k_measure_i8(const int8_t* __restrict__ s
         E += red[0][w];
         M += red[1][w];
       }
-      if ((L & 15) == 0) {
+      if ((L & 15) == 0 && chunk == 0u) {
         E -= (long long)D * N;
         M += (long long)N;
       }
       int64_t* a = acc + ((size_t)s * slots + sigma) * kAccStride;
-      a[0] = E;
-      a[1] = M;
+      acc_add(a + 0, E, chunks);
+      acc_add(a + 1, M, chunks);
     }
-    __syncthreads();
   }
 }
 
@@ -1517,9 +1527,10 @@ __global__ void __launch_bounds__(256) k_measure_i8(const int8_t* __restrict__ s
 // (Sec. 4.1 overlap).  Stored in acc[s][k*R][6].
 __global__ void __launch_bounds__(256) k_overlap_i8(const int8_t* __restrict__ spins, const int32_t* slot_at,
                                                     const int8_t* __restrict__ occ, int64_t* acc, int S, int R,
-                                                    int K, int slots, uint32_t N) {
+                                                    int K, int slots, uint32_t N, uint32_t chunks) {
   __shared__ long long red[8];
-  for (uint32_t sk = blockIdx.x; sk < (uint32_t)(S * K); sk += gridDim.x) {
+  {
+    const uint32_t sk = blockIdx.x / chunks, chunk = blockIdx.x - sk * chunks;
     const int s = (int)(sk / (uint32_t)K), k = (int)(sk - (uint32_t)s * K);
     const int s0 = slot_at[((size_t)s * R + 0) * K + k] * R + 0;
     const int s1 = slot_at[((size_t)s * R + 1) * K + k] * R + 1;
@@ -1528,17 +1539,17 @@ __global__ void __launch_bounds__(256) k_overlap_i8(const int8_t* __restrict__ s
     long long q = 0;
     if (occ) {  // Q = sum_i x_i s_i^0 s_i^1
       const int8_t* xo = occ + (size_t)s * N;
-      for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) q += xo[i] * a0[i] * a1[i];
+      for (uint32_t i = chunk * blockDim.x + threadIdx.x; i < N; i += chunks * blockDim.x) q += xo[i] * a0[i] * a1[i];
     } else if ((N & 15u) == 0u) {  // 16 sites per step: s0 s1 = -1 iff the sign bits differ
       uint32_t d = 0;
-      for (uint32_t i = 16u * threadIdx.x; i < N; i += 16u * blockDim.x) {
+      for (uint32_t i = 16u * (chunk * blockDim.x + threadIdx.x); i < N; i += 16u * chunks * blockDim.x) {
         const uint4 u = *reinterpret_cast<const uint4*>(a0 + i), v = *reinterpret_cast<const uint4*>(a1 + i);
         d += __popc((u.x ^ v.x) & 0x80808080u) + __popc((u.y ^ v.y) & 0x80808080u) +
              __popc((u.z ^ v.z) & 0x80808080u) + __popc((u.w ^ v.w) & 0x80808080u);
       }
       q = -2ll * d;  // N added once below
     } else {
-      for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) q += a0[i] * a1[i];
+      for (uint32_t i = chunk * blockDim.x + threadIdx.x; i < N; i += chunks * blockDim.x) q += a0[i] * a1[i];
     }
     for (int off = 16; off > 0; off >>= 1) q += __shfl_down_sync(0xffffffffu, q, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = q;
@@ -1546,10 +1557,9 @@ __global__ void __launch_bounds__(256) k_overlap_i8(const int8_t* __restrict__ s
     if (threadIdx.x == 0) {
       long long Q = 0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) Q += red[w];
-      if (!occ && (N & 15u) == 0u) Q += (long long)N;
-      acc[((size_t)s * slots + (size_t)k * R) * kAccStride + 6] = Q;
+      if (!occ && (N & 15u) == 0u && chunk == 0u) Q += (long long)N;
+      acc_add(acc + ((size_t)s * slots + (size_t)k * R) * kAccStride + 6, Q, chunks);
     }
-    __syncthreads();
   }
 }
 
@@ -2026,8 +2036,10 @@ cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
   p.keys = lat.keys;
   p.t_dev = lat.capturing ? lat.t_dev : nullptr;
   if (lat.rng == IANUS_RNG_WHEEL) {
-    const WheelParams wp{p, lat.wheels, lat.rows, lat.hs, lat.occ, lat.fthr};
-    const uint32_t tiles = (lat.rows + kWheelRows - 1) / kWheelRows;
+    uint32_t per = kWheelRows;
+    while (per > 4u && (uint64_t)lat.slots * lat.S * ((lat.rows + per - 1) / per) < 152u * 8u) per /= 2u;
+    const WheelParams wp{p, lat.wheels, lat.rows, per, lat.hs, lat.occ, lat.fthr};
+    const uint32_t tiles = (lat.rows + per - 1) / per;
     const uint32_t warps = std::min<uint32_t>(tiles, kWheelWarps);
     const uint64_t wgrid = (uint64_t)lat.slots * lat.S * ((tiles + warps - 1) / warps);
     if (wgrid > 0x7fffffffull) return cudaErrorInvalidConfiguration;  // beyond any device's memory
@@ -2083,36 +2095,57 @@ cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
   return cudaGetLastError();
 }
 
+// Blocks per configuration of a plain measurement with `units` steps of one
+// thread each: about 8 blocks per SM in all, at least two steps a thread.
+// (One block per configuration left a few large lattices on a few SMs: 370 us
+// for 2 x 2 configurations of L=54; 82^3, 16 samples, 49 sweeps with 25
+// measurements: 21.1 ms against 4.3 ms with the chunks.)
+static uint32_t meas_chunks_i8(uint64_t configs, uint64_t units) {
+  const uint64_t want = (152u * 8u + configs - 1u) / configs, most = (units + 511u) / 512u;
+  return (uint32_t)std::max<uint64_t>(1u, std::min(want, most));
+}
+
 cudaError_t launch_measure_i8(Lattice& lat, int want_q) {
-  const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)lat.slots * lat.S, 152u * 8u);
-  if (lat.field && lat.D == 3)
-    k_measure_field_i8<3><<<grid, 256, 0, lat.stream>>>((const int8_t*)lat.spins, (const int8_t*)lat.J, lat.hs,
-                                                         lat.occ, lat.acc, lat.S, lat.slots, lat.L, lat.N);
-  else if (lat.field)
-    k_measure_field_i8<2><<<grid, 256, 0, lat.stream>>>((const int8_t*)lat.spins, (const int8_t*)lat.J, lat.hs,
-                                                         lat.occ, lat.acc, lat.S, lat.slots, lat.L, lat.N);
-  else if (lat.K == 1 && lat.R <= 2 && lat.L % 16 == 0) {  // E, M (and Q) in one pass per sample
-    const unsigned gs = (unsigned)std::min<uint64_t>((uint64_t)lat.S, 152u * 8u);
-    const int8_t* sp = (const int8_t*)lat.spins;
-    const int8_t* J = (const int8_t*)lat.J;
+  const int8_t* sp = (const int8_t*)lat.spins;
+  const int8_t* J = (const int8_t*)lat.J;
+  const uint32_t configs = (uint32_t)(lat.slots * lat.S);
+  const bool vec = lat.L % 16 == 0;
+  const bool one = !lat.field && lat.K == 1 && lat.R <= 2 && vec;  // E, M (and Q) in one pass per sample
+  const uint32_t ch = one ? meas_chunks_i8((uint64_t)lat.S, lat.N / 16u)
+                          : meas_chunks_i8(configs, !lat.field && vec ? lat.N / 16u : lat.N);
+  const uint64_t pairs = (uint64_t)lat.S * lat.K;
+  const uint32_t cq = meas_chunks_i8(pairs, !lat.field && (lat.N & 15u) == 0u ? lat.N / 16u : lat.N);
+  if (ch > 1 || cq > 1) {
+    const cudaError_t e = cudaMemsetAsync(lat.acc, 0, (size_t)configs * kAccStride * sizeof(int64_t), lat.stream);
+    if (e != cudaSuccess) return e;
+  }
+  if (one) {
+    const unsigned gs = (unsigned)lat.S * ch;
     if (lat.D == 3) {
-      if (lat.R == 2) k_measure_i8_k1<3, 2><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q);
-      else k_measure_i8_k1<3, 1><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q);
+      if (lat.R == 2) k_measure_i8_k1<3, 2><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q, ch);
+      else k_measure_i8_k1<3, 1><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q, ch);
     } else {
-      if (lat.R == 2) k_measure_i8_k1<2, 2><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q);
-      else k_measure_i8_k1<2, 1><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q);
+      if (lat.R == 2) k_measure_i8_k1<2, 2><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q, ch);
+      else k_measure_i8_k1<2, 1><<<gs, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.L, lat.N, want_q, ch);
     }
     return cudaGetLastError();
-  } else if (lat.D == 3)
-    k_measure_i8<3><<<grid, 256, 0, lat.stream>>>((const int8_t*)lat.spins, (const int8_t*)lat.J, lat.acc,
-                                                   lat.S, lat.R, lat.slots, lat.L, lat.N);
-  else
-    k_measure_i8<2><<<grid, 256, 0, lat.stream>>>((const int8_t*)lat.spins, (const int8_t*)lat.J, lat.acc,
-                                                   lat.S, lat.R, lat.slots, lat.L, lat.N);
+  }
+  if (lat.field) {
+    if (lat.D == 3)
+      k_measure_field_i8<3><<<configs * ch, 256, 0, lat.stream>>>(sp, J, lat.hs, lat.occ, lat.acc, lat.S, lat.slots,
+                                                                  lat.L, lat.N, ch);
+    else
+      k_measure_field_i8<2><<<configs * ch, 256, 0, lat.stream>>>(sp, J, lat.hs, lat.occ, lat.acc, lat.S, lat.slots,
+                                                                  lat.L, lat.N, ch);
+  } else {
+    if (lat.D == 3)
+      k_measure_i8<3><<<configs * ch, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.R, lat.slots, lat.L, lat.N, ch);
+    else
+      k_measure_i8<2><<<configs * ch, 256, 0, lat.stream>>>(sp, J, lat.acc, lat.S, lat.R, lat.slots, lat.L, lat.N, ch);
+  }
   if (want_q && lat.R >= 2) {
-    const unsigned gq = (unsigned)std::min<uint64_t>((uint64_t)lat.S * lat.K, 152u * 8u);
-    k_overlap_i8<<<gq, 256, 0, lat.stream>>>((const int8_t*)lat.spins, lat.slot_at, lat.field ? lat.occ : nullptr,
-                                            lat.acc, lat.S, lat.R, lat.K, lat.slots, lat.N);
+    k_overlap_i8<<<(unsigned)pairs * cq, 256, 0, lat.stream>>>(sp, lat.slot_at, lat.field ? lat.occ : nullptr, lat.acc,
+                                                              lat.S, lat.R, lat.K, lat.slots, lat.N, cq);
   }
   return cudaGetLastError();
 }
