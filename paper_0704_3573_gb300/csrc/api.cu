@@ -5,6 +5,7 @@
 // checkpoints and error reporting.  Host logic only; all per-site work runs
 // in the kernels of k_plain.cu, k_msc.cu, k_potts.cu and k_pt.cu.
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -124,7 +125,7 @@ int plan(const ianus_config* c, Sizes& z) {
   z.off_nseg = take(z.poolable ? (size_t)z.G * 4 : 0);
   z.off_ptab = take(layout != IANUS_LAYOUT_U8X4 ? 0
                     : c->model == IANUS_POTTS4_PERM ? (size_t)z.K * perm_table_entries(z.D) * 16
-                                                    : (size_t)z.K * 65536 * 16);
+                                                    : (size_t)z.K * kPottsRows * 16);
   z.off_pttab = take((size_t)std::max(z.K - 1, 0) * z.pt_cap * 8);
   z.off_ptsign = take((size_t)std::max(z.K - 1, 1));
   z.off_slot = take((size_t)z.S * z.R * z.K * 4 * 2);  // slot_at then temp_of
@@ -195,6 +196,16 @@ bool beta_ok(const double* beta, int K) {
   return true;
 }
 
+// Table row of one tuple of Potts counts: the thresholds, 2^32 - 1 standing
+// for 2^32, and a flag for each of those.
+uint4 potts_table_row(double beta, const int* n) {
+  uint64_t T[3];
+  potts_thresholds(beta, n, T);
+  auto word = [](uint64_t t) { return t >= kTwo32 ? 0xffffffffu : (uint32_t)t; };
+  return make_uint4(word(T[0]), word(T[1]), word(T[2]),
+                    (T[0] >= kTwo32 ? 1u : 0u) | (T[1] >= kTwo32 ? 2u : 0u) | (T[2] >= kTwo32 ? 4u : 0u));
+}
+
 // Rebuild and upload the acceptance tables for (algo, beta).
 int upload_tables(Lattice* lat, int algo, const double* beta) {
   const int K = lat->K;
@@ -248,9 +259,8 @@ int upload_tables(Lattice* lat, int algo, const double* beta) {
     lat->jit = nullptr;  // specialised lazily by the first launch that wants it
     lat->jit_algo = -1;
   } else if (lat->model == IANUS_POTTS4_PERM) {
-    // compact table of the permutation model: counts n_k in 0..2D with
-    // n0 + n1 + n2 + n3 = 2D, entry n0 + B (n1 + B n2), B = 2D + 1
-    const int D = lat->D, B = 2 * D + 1;
+    // counts n_k in 0..2D with n0 + n1 + n2 + n3 = 2D
+    const int D = lat->D;
     for (int k = 0; k < K; ++k)
       if (2.0 * D * beta[k] > 700.0) return IANUS_EINVAL;  // exp(2D beta) must stay finite
     const uint32_t NT = perm_table_entries(D);
@@ -261,39 +271,25 @@ int upload_tables(Lattice* lat, int algo, const double* beta) {
         for (int n1 = 0; n0 + n1 <= 2 * D; ++n1)
           for (int n2 = 0; n0 + n1 + n2 <= 2 * D; ++n2) {
             const int n[4] = {n0, n1, n2, 2 * D - n0 - n1 - n2};
-            uint64_t T[3];
-            potts_thresholds(beta[k], n, T);
-            uint4 e;
-            e.x = (uint32_t)T[0];
-            e.y = (uint32_t)T[1];
-            e.z = (uint32_t)T[2];
-            e.w = (T[0] >= kTwo32 ? 1u : 0u) | (T[1] >= kTwo32 ? 2u : 0u) | (T[2] >= kTwo32 ? 4u : 0u);
-            tab[(size_t)k * NT + n0 + B * (n1 + B * n2)] = e;
+            tab[(size_t)k * NT + perm_row(D, n0, n1, n2)] = potts_table_row(beta[k], n);
           }
     CK(cudaMemcpyAsync(lat->ptab, tab.data(), tab.size() * sizeof(uint4), cudaMemcpyHostToDevice, lat->stream));
   } else {
-    if (beta_ok(beta, K)) {
-      for (int k = 0; k < K; ++k)
-        if (beta[k] > 100.0) return IANUS_EINVAL;  // exp(6 beta) must stay finite
-    }
-    std::vector<uint64_t> flat(3u * 28561u);
-    std::vector<uint4> tab((size_t)K * 65536);
+    for (int k = 0; k < K; ++k)
+      if (beta[k] > 100.0) return IANUS_EINVAL;  // exp(6 beta) must stay finite
+    // counts with sum |n_k| <= 2D and even, as the 2D bonds of weight +-1 give
+    const int m = 2 * lat->D;
+    std::vector<uint4> tab((size_t)K * kPottsRows);
     std::memset(tab.data(), 0, tab.size() * sizeof(uint4));
     for (int k = 0; k < K; ++k) {
-      table_potts(beta[k], flat.data(), flat.size());
-      size_t idx = 0;
-      for (int n0 = 0; n0 < 13; ++n0)
-        for (int n1 = 0; n1 < 13; ++n1)
-          for (int n2 = 0; n2 < 13; ++n2)
-            for (int n3 = 0; n3 < 13; ++n3, ++idx) {
-              const uint32_t key = (uint32_t)n0 | ((uint32_t)n1 << 4) | ((uint32_t)n2 << 8) | ((uint32_t)n3 << 12);
-              uint4 e;
-              const uint64_t t0 = flat[3 * idx], t1 = flat[3 * idx + 1], t2 = flat[3 * idx + 2];
-              e.x = (uint32_t)t0;
-              e.y = (uint32_t)t1;
-              e.z = (uint32_t)t2;
-              e.w = (t0 >= kTwo32 ? 1u : 0u) | (t1 >= kTwo32 ? 2u : 0u) | (t2 >= kTwo32 ? 4u : 0u);
-              tab[(size_t)k * 65536 + key] = e;
+      int n[4];
+      for (n[0] = -m; n[0] <= m; ++n[0])
+        for (n[1] = -m; n[1] <= m; ++n[1])
+          for (n[2] = -m; n[2] <= m; ++n[2])
+            for (n[3] = -m; n[3] <= m; ++n[3]) {
+              const int sum = std::abs(n[0]) + std::abs(n[1]) + std::abs(n[2]) + std::abs(n[3]);
+              if (sum > m || (sum & 1)) continue;
+              tab[(size_t)k * kPottsRows + potts_row(n[0], n[1], n[2], n[3])] = potts_table_row(beta[k], n);
             }
     }
     CK(cudaMemcpyAsync(lat->ptab, tab.data(), tab.size() * sizeof(uint4), cudaMemcpyHostToDevice, lat->stream));

@@ -12,14 +12,23 @@
 // and c is the colour, so every neighbour of a colour-c word is a colour-(1-c)
 // word with the same x / 2 (or x / 2 +- 1 along x).
 //
-// Update of one sample: each of the 2D bonds is satisfied by exactly one
-// state k of s_i, k = pi(s_j) for a forward bond (i, j = i + e_d) and
-// k = pi^-1(s_j) for a backward bond (j = i - e_d, i); the counts n_k are
-// packed in nibbles and (n0, n1, n2) index a compact table of cumulative
-// heat-bath thresholds (n3 = 2D - n0 - n1 - n2), read through the L1 cache.
+// Update: each of the 2D bonds is satisfied by exactly one state k of s_i,
+// k = pi(s_j) for a forward bond (i, j = i + e_d) and k = pi^-1(s_j) for a
+// backward bond (j = i - e_d, i); the counts (n0, n1, n2) give a row of
+// cumulative heat-bath thresholds (perm_row, lattice.h).  The row is linear
+// in the counts, so it is summed over the bonds for the 4 samples of a word at
+// once, one byte each (4D: two bytes, then 16 bits):
+//   forward: pi(s_j) by two byte-wise selects of the code's fields on the bits
+//     of s_j; the sums of its bits t0, t1 and t0 t1 give the three counts;
+//   backward: code XOR s_j in every field is zero in field pi^-1(s_j) only;
+//     those one-hot fields are added as 2-bit numbers.
+//
+// Bound: integer issue.  3D L=32, 256 x 2: 21.6 us per colour pass (44 us with
+// each sample's bonds done one by one, pi^-1 by a shared 256-byte table); 4D
+// L=16, 256 x 2: 51 us (102 us).
 #include <algorithm>
 
-#include "lattice.h"
+#include "potts_words.cuh"
 
 namespace ianus {
 
@@ -27,45 +36,6 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr uint32_t kIdentityCode = 0xE4u;  // (0, 1, 2, 3)
-
-template <int D>
-struct PermNbr {
-  uint32_t self, site;
-  uint32_t fw[D], bw[D];  // split indices of i + e_d and i - e_d
-};
-
-// Colour-c word w -> its split index, natural index and neighbours.
-template <int D>
-__device__ __forceinline__ PermNbr<D> perm_neighbours(const Geom& g, int c, uint32_t w) {
-  const uint32_t h = (uint32_t)g.h, L = (uint32_t)g.L;
-  const uint32_t row = w / h, k = w - row * h;
-  uint32_t co[D > 1 ? D : 2];
-  uint32_t r = row, psum = 0;
-#pragma unroll
-  for (int d = 1; d < D; ++d) {
-    co[d] = r % L;
-    r /= L;
-    psum += co[d];
-  }
-  const uint32_t xpar = (uint32_t)(c ^ (int)psum) & 1u;
-  const uint32_t oc = 1u - (uint32_t)c;
-  PermNbr<D> n;
-  n.self = (2u * row + (uint32_t)c) * h + k;
-  n.site = 2u * k + xpar + L * row;
-  const uint32_t base_o = (2u * row + oc) * h;
-  n.fw[0] = base_o + (xpar ? (k + 1u == h ? 0u : k + 1u) : k);  // (x + 1) / 2 mod h
-  n.bw[0] = base_o + (xpar ? k : (k == 0u ? h - 1u : k - 1u));  // (x - 1) / 2 mod h
-  uint32_t stride = 1;
-#pragma unroll
-  for (int d = 1; d < D; ++d) {
-    const uint32_t rp = co[d] + 1u == L ? row - (L - 1u) * stride : row + stride;
-    const uint32_t rm = co[d] == 0u ? row + (L - 1u) * stride : row - stride;
-    n.fw[d] = (2u * rp + oc) * h + k;
-    n.bw[d] = (2u * rm + oc) * h + k;
-    stride *= L;
-  }
-  return n;
-}
 
 // Natural index -> split index, any D.
 __device__ __forceinline__ uint32_t perm_split(const Geom& g, uint32_t i) {
@@ -96,88 +66,76 @@ __device__ __forceinline__ uint32_t perm_code_of(uint32_t p) {
   return code | ((pool & 3u) << 6);
 }
 
-// pi^-1 as a code: field pi(v) of the result holds v.
-__device__ __forceinline__ uint32_t inverse_code(uint32_t code) {
-  uint32_t inv = 0;
-#pragma unroll
-  for (uint32_t v = 0; v < 4u; ++v) inv |= v << (2u * ((code >> (2u * v)) & 3u));
-  return inv;
+// pi(s) in the low two bits of each byte (the rest is not defined), from the
+// codes c of 4 samples.
+__device__ __forceinline__ uint32_t perm_apply(uint32_t c, uint32_t s) {
+  // a byte of ones where bit 1 (bit 0) of the state is set: sign replication of the shifted byte
+  const uint32_t m1 = potts::prmt(s << 6, 0u, 0xBA98u), m0 = potts::prmt(s << 7, 0u, 0xBA98u);
+  const uint32_t c1 = (m1 & (c >> 4)) | (~m1 & c);
+  return (m0 & (c1 >> 2)) | (~m0 & c1);
 }
 
-struct PermParams {
-  uint32_t* spins;         // [slots][Q4][N]
-  const uint32_t* J;       // [Q4][D][N] permutation codes
-  const uint4* tab;        // [K][(2D+1)^3] {T0, T1, T2, always flags}
-  const int32_t* temp_of;  // [S][R][K]
-  Geom geom;
-  int S, R, K, Q4, slots;
-  int colour;
-  uint32_t t_lo, t_hi;
-  uint32_t words_per_block;
-  PhiloxKeys keys;
-  const uint64_t* t_dev;  // non-null in captured graphs
-};
-
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_sweep_perm(const PermParams p) {
-  constexpr uint32_t B = 2 * D + 1;
-  constexpr uint32_t NT = B * B * B;
-  __shared__ uint8_t inv_s[256];
-  for (uint32_t c = threadIdx.x; c < 256u; c += kBlock) inv_s[c] = (uint8_t)inverse_code(c);
-  dependent_launch_entry();  // the table above reads no memory
-  const int sq = blockIdx.y;  // sigma * Q4 + q
-  const int sigma = sq / p.Q4, q = sq - sigma * p.Q4;
-  const int tslot = sigma / p.R, a = sigma - tslot * p.R;
-  const Geom geom = p.geom;
-  const uint32_t N = geom.N;
-  const uint32_t* Jq = p.J + (size_t)q * D * N;
-  uint32_t* sp = p.spins + ((size_t)sigma * p.Q4 + q) * N;
-  const uint4* tab[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int s = 4 * q + b;
-    const int k = s < p.S ? p.temp_of[((size_t)s * p.R + a) * p.K + tslot] : tslot;
-    tab[b] = p.tab + (size_t)k * NT;
-  }
-  const uint32_t c2 = (TAG_POTTS << 28) | ((uint32_t)sigma << 16) | (uint32_t)q;
-  const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
-  __syncthreads();
-  const uint32_t w_begin = blockIdx.x * p.words_per_block;
-  const uint32_t w_end = min(w_begin + p.words_per_block, geom.half);
-  for (uint32_t w = w_begin + threadIdx.x; w < w_end; w += kBlock) {
-    const PermNbr<D> n = perm_neighbours<D>(geom, p.colour, w);
-    uint32_t sf[D], sb[D], jf[D], jb[D];
+struct PermModel {
+  static constexpr uint32_t kRows = D == 4 ? 592u : 256u;
+  uint32_t cf[D], cb[D];
+
+  __device__ __forceinline__ void prepare(const uint32_t* J, uint32_t N, const potts::Nbr<D>& n) {
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      sf[d] = sp[n.fw[d]];
-      sb[d] = sp[n.bw[d]];
-      jf[d] = __ldg(Jq + (size_t)d * N + n.self);
-      jb[d] = __ldg(Jq + (size_t)d * N + n.bw[d]);
+      cf[d] = __ldg(J + (size_t)d * N + n.self);
+      cb[d] = __ldg(J + (size_t)d * N + n.bw[d]);
     }
-    const uint4 x = philox10(n.site, tk.lo, c2, tk.hi, p.keys);
-    const uint32_t rr[4] = {x.x, x.y, x.z, x.w};
-    uint32_t out = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      uint32_t npk = 0;  // nibble k = n_k
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        const uint32_t s_f = (sf[d] >> (8 * b)) & 3u;
-        const uint32_t tf = (jf[d] >> (8 * b + 2 * s_f)) & 3u;  // pi(s_j)
-        const uint32_t s_b = (sb[d] >> (8 * b)) & 3u;
-        const uint32_t tb = ((uint32_t)inv_s[(jb[d] >> (8 * b)) & 0xFFu] >> (2 * s_b)) & 3u;  // pi^-1(s_j)
-        npk += (1u << (4 * tf)) + (1u << (4 * tb));
-      }
-      const uint32_t n0 = npk & 15u, n1 = (npk >> 4) & 15u, n2 = (npk >> 8) & 15u;
-      const uint4 T = __ldg(tab[b] + n0 + B * (n1 + B * n2));
-      const uint32_t r = rr[b];
-      const uint32_t ge0 = !((T.w & 1u) || r < T.x);
-      const uint32_t ge1 = !((T.w & 2u) || r < T.y);
-      const uint32_t ge2 = !((T.w & 4u) || r < T.z);
-      out |= (ge0 + ge1 + ge2) << (8 * b);
-    }
-    sp[n.self] = out;
   }
+
+  __device__ __forceinline__ void rows(const uint32_t* sf, const uint32_t* sb, uint32_t* row) const {
+    using potts::kOnes;
+    uint32_t t0 = 0, t1 = 0, t01 = 0;  // forward: sums of the bits of pi(s_j)
+    uint32_t z[D];                     // backward: bit 2k set where pi^-1(s_j) = k
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const uint32_t t = perm_apply(cf[d], sf[d]), h = t >> 1;
+      t0 += t & kOnes;
+      t1 += h & kOnes;
+      t01 += t & h & kOnes;
+      const uint32_t x = cb[d] ^ (sb[d] * 0x55u);
+      z[d] = ~(x | (x >> 1)) & 0x55555555u;
+    }
+    uint32_t zs = z[0] + z[1];  // 2-bit fields: up to three of them add without overflow
+    if (D >= 3) zs += z[2 % D];
+    if constexpr (D < 4) {
+      // n0 + 37 n1 + 16 n2 per byte: a forward bond adds 1 + 36 t0 + 15 t1 - 52 t0 t1
+      const uint32_t idx = (zs & 0x33333333u) + 37u * ((zs >> 2) & 0x03030303u) + (uint32_t)D * kOnes + 36u * t0 +
+                           15u * t1 - 52u * t01;
+      row[0] = idx & 0xffu;
+      row[1] = (idx >> 8) & 0xffu;
+      row[2] = (idx >> 16) & 0xffu;
+      row[3] = idx >> 24;
+    } else {
+      const uint32_t e = (zs & 0x33333333u) + (z[3 % D] & 0x33333333u);                  // n0, n2 as nibbles
+      const uint32_t o = ((zs >> 2) & 0x33333333u) + ((z[3 % D] >> 2) & 0x33333333u);    // n1, n3
+      // n0 + 9 n1 and n2 per byte; a forward bond adds 1 + 8 t0 - t1 - 8 t0 t1 and t1 - t0 t1
+      const uint32_t a = (e & 0x0f0f0f0fu) + 9u * (o & 0x0f0f0f0fu) + 4u * kOnes + 8u * (t0 - t01) - t1;
+      const uint32_t b = ((e >> 4) & 0x0f0f0f0fu) + t1 - t01;
+      const uint32_t r02 = (a & 0x00ff00ffu) + 73u * (b & 0x00ff00ffu);
+      const uint32_t r13 = ((a >> 8) & 0x00ff00ffu) + 73u * ((b >> 8) & 0x00ff00ffu);
+      // permutation codes keep rows below kRows; the bound holds for any bytes
+      row[0] = min(r02 & 0xffffu, kRows - 1u);
+      row[1] = min(r13 & 0xffffu, kRows - 1u);
+      row[2] = min(r02 >> 16, kRows - 1u);
+      row[3] = min(r13 >> 16, kRows - 1u);
+    }
+  }
+
+  static __device__ __forceinline__ void count_bond(uint32_t s, uint32_t sn, uint32_t J, uint32_t& good, uint32_t&) {
+    good += potts::zero2(perm_apply(J, sn) ^ s);
+  }
+};
+
+template <int D, int RT, bool KONE>
+__global__ void __launch_bounds__(kBlock, RT == 2 ? 4 : 5) k_sweep_perm(const potts::Params p) {
+  __shared__ uint4 tab[KONE ? PermModel<D>::kRows : 1];
+  potts::sweep_words<PermModel<D>, D, RT, KONE>(p, tab);
 }
 
 // Couplings from the PERM stream (jmode 0) or identity permutations (jmode
@@ -203,60 +161,6 @@ __global__ void k_init_perm(uint32_t* spins, uint32_t* J, Geom geom, int Q4, int
       const uint4 r = philox10(i, 0u, (TAG_PINIT << 28) | ((uint32_t)sg << 16) | q, 0u, keys);
       spins[((size_t)sg * Q4 + q) * geom.N + j] =
           (r.x >> 30) | ((r.y >> 30) << 8) | ((r.z >> 30) << 16) | ((r.w >> 30) << 24);
-    }
-  }
-}
-
-// Per (slot, quad) block: E = -sum over forward bonds of delta(s_i, pi(s_j))
-// and the state counts of the 4 samples (Sec. 4.1 observables).
-constexpr int kPermMeasIters = 32;
-
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_measure_perm(const uint32_t* __restrict__ spins,
-                                                         const uint32_t* __restrict__ J, int64_t* acc, Geom geom,
-                                                         int S, int Q4, int slots) {
-  const int sq = blockIdx.y;
-  const int sigma = sq / Q4, q = sq - sigma * Q4;
-  const uint32_t N = geom.N, h = (uint32_t)geom.h;
-  const uint32_t* Jq = J + (size_t)q * D * N;
-  const uint32_t* sp = spins + ((size_t)sigma * Q4 + q) * N;
-  const uint32_t base = blockIdx.x * (uint32_t)(kBlock * kPermMeasIters);
-  long long v[4][5];  // per sample: E, n0..n3
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int f = 0; f < 5; ++f) v[b][f] = 0;
-  for (int it = 0; it < kPermMeasIters; ++it) {
-    const uint32_t j = base + (uint32_t)it * kBlock + threadIdx.x;
-    if (j >= N) continue;
-    const uint32_t rc = j / h, k = j - rc * h;
-    const PermNbr<D> n = perm_neighbours<D>(geom, (int)(rc & 1u), (rc >> 1) * h + k);
-    const uint32_t si = sp[j];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const uint32_t sj = sp[n.fw[d]];
-      const uint32_t code = Jq[(size_t)d * N + j];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const uint32_t t = (code >> (8 * b + 2 * ((sj >> (8 * b)) & 3u))) & 3u;
-        if (t == ((si >> (8 * b)) & 3u)) v[b][0] -= 1;
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < 4; ++b) v[b][1 + ((si >> (8 * b)) & 3u)] += 1;
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int f = 0; f < 5; ++f)
-      for (int off = 16; off > 0; off >>= 1) v[b][f] += __shfl_down_sync(0xffffffffu, v[b][f], off);
-  if ((threadIdx.x & 31) == 0) {
-    for (int b = 0; b < 4; ++b) {
-      const int s = 4 * q + b;
-      if (s >= S) continue;
-      int64_t* ac = acc + ((size_t)s * slots + sigma) * kAccStride;
-      atomicAdd((unsigned long long*)&ac[0], (unsigned long long)v[b][0]);
-      for (int f = 0; f < 4; ++f) atomicAdd((unsigned long long*)&ac[2 + f], (unsigned long long)v[b][1 + f]);
     }
   }
 }
@@ -316,53 +220,25 @@ cudaError_t launch_init_perm(Lattice& lat, int jmode) {
 }
 
 cudaError_t launch_sweep_perm(Lattice& lat, int colour, uint64_t t) {
-  PermParams p;
-  p.spins = (uint32_t*)lat.spins;
-  p.J = (const uint32_t*)lat.J;
-  p.tab = lat.ptab;
-  p.temp_of = lat.temp_of;
-  p.geom = lat.geom;
-  p.S = lat.S;
-  p.R = lat.R;
-  p.K = lat.K;
-  p.Q4 = lat.Q4;
-  p.slots = lat.slots;
-  p.colour = colour;
-  p.t_lo = (uint32_t)(t & 0xffffffffu);
-  p.t_hi = (uint32_t)(t >> 32);
-  p.keys = lat.keys;
-  p.t_dev = lat.capturing ? lat.t_dev : nullptr;
-  const uint32_t half = lat.geom.half;
-  const uint32_t ys = (uint32_t)(lat.slots * lat.Q4);
-  uint32_t target_blocks = (152u * 8u + ys - 1) / ys;
-  uint32_t wpb = (half + target_blocks - 1) / target_blocks;
-  wpb = ((wpb + kBlock - 1) / kBlock) * kBlock;
-  if (wpb < (uint32_t)kBlock) wpb = kBlock;
-  p.words_per_block = wpb;
-  dim3 grid((half + wpb - 1) / wpb, ys);
-  void* args[] = {(void*)&p};
-  const void* k = lat.D == 4   ? (const void*)k_sweep_perm<4>
-                  : lat.D == 3 ? (const void*)k_sweep_perm<3>
-                               : (const void*)k_sweep_perm<2>;
-  return launch_dependent(k, grid, dim3(kBlock), args, 0, lat.stream);
+  const void* k[3][2][2] = {{{(const void*)k_sweep_perm<2, 1, false>, (const void*)k_sweep_perm<2, 1, true>},
+                             {(const void*)k_sweep_perm<2, 2, false>, (const void*)k_sweep_perm<2, 2, true>}},
+                            {{(const void*)k_sweep_perm<3, 1, false>, (const void*)k_sweep_perm<3, 1, true>},
+                             {(const void*)k_sweep_perm<3, 2, false>, (const void*)k_sweep_perm<3, 2, true>}},
+                            {{(const void*)k_sweep_perm<4, 1, false>, (const void*)k_sweep_perm<4, 1, true>},
+                             {(const void*)k_sweep_perm<4, 2, false>, (const void*)k_sweep_perm<4, 2, true>}}};
+  const int rt = lat.R % 2 == 0 ? 2 : 1;
+  return potts::launch_sweep(lat, colour, t, k[lat.D - 2][rt - 1][lat.K == 1], rt, rt == 2 ? 4 : 5);
 }
 
+
 cudaError_t launch_measure_perm(Lattice& lat, int want_q) {
-  cudaError_t e = cudaMemsetAsync(lat.acc, 0, (size_t)lat.S * lat.slots * kAccStride * sizeof(int64_t), lat.stream);
-  if (e != cudaSuccess) return e;
-  const uint32_t per_block = kBlock * kPermMeasIters;
-  dim3 grid((lat.N + per_block - 1) / per_block, (unsigned)(lat.slots * lat.Q4));
-  const uint32_t* sp = (const uint32_t*)lat.spins;
-  const uint32_t* J = (const uint32_t*)lat.J;
   if (lat.D == 4)
-    k_measure_perm<4><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S, lat.Q4, lat.slots);
-  else if (lat.D == 3)
-    k_measure_perm<3><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S, lat.Q4, lat.slots);
-  else
-    k_measure_perm<2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S, lat.Q4, lat.slots);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return want_q && lat.R >= 2 ? launch_overlap_potts(lat) : cudaSuccess;
+    return potts::launch_measure(lat, want_q, potts::k_measure<PermModel<4>, 4, 1>,
+                                 potts::k_measure<PermModel<4>, 4, 2>);
+  if (lat.D == 3)
+    return potts::launch_measure(lat, want_q, potts::k_measure<PermModel<3>, 3, 1>,
+                                 potts::k_measure<PermModel<3>, 3, 2>);
+  return potts::launch_measure(lat, want_q, potts::k_measure<PermModel<2>, 2, 1>, potts::k_measure<PermModel<2>, 2, 2>);
 }
 
 cudaError_t launch_get_spins_perm(Lattice& lat, int8_t* dev_out) {

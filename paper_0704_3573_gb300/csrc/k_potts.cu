@@ -4,14 +4,25 @@
 // A 32-bit word holds one site of 4 samples (byte b = sample 4q+b, state
 // 0..3), the counterpart of the paper's 2-bit Potts spins (Sec. 3.2); one
 // Philox block supplies the 4 random words of the word.  The local counts
-// n_k = sum_j J_ij [s_j == k] are kept as four biased nibbles (n_k + 6) of a
-// 16-bit value, which indexes a table of cumulative heat-bath thresholds
+// n_k = sum_j J_ij [s_j == k] select a row of cumulative heat-bath thresholds
 // (the look-up table of Sec. 3.2); the new state is the smallest k with
 // r < T_k, else 3.  Words of one colour are contiguous (checkerboard-split
 // order, Sec. 3.1).
+//
+// The row is linear in the counts (kPottsCoef, lattice.h), so each neighbour
+// adds a term fixed by its state and coupling sign.  The terms of the 4
+// samples are looked up together: state and sign make a nibble, two
+// neighbours' nibbles fill the word, and a byte permute of an 8-entry table
+// maps four nibbles at a time to the low (5 bits) or high digit of the term.
+// Six terms of 5 bits fit a byte, so the digits are added as bytes.
+//
+// Bound: integer issue and, with few words a thread, the latency of a site's
+// loads.  L=32, 128 x 2: 12 us per colour pass (19 us with the counts of each
+// sample extracted one by one and the rows, 16 bytes in a 1 MB table, read
+// through L1): 238 warp instructions per word against 408.
 #include <algorithm>
 
-#include "lattice.h"
+#include "potts_words.cuh"
 
 namespace ianus {
 
@@ -19,79 +30,65 @@ namespace {
 
 constexpr int kBlock = 256;
 
-struct PottsParams {
-  uint32_t* spins;         // [slots][Q4][N]
-  const uint32_t* J;       // [Q4][D][N]
-  const uint4* ptab;       // [K][65536]
-  const int32_t* temp_of;  // [S][R][K]
-  Geom geom;
-  int S, R, K, Q4, slots;
-  int colour;
-  uint32_t t_lo, t_hi;
-  uint32_t words_per_block;
-  PhiloxKeys keys;
-  const uint64_t* t_dev;  // non-null in captured graphs
-};
+// Low or high 5-bit digit of the term of (state, sign): byte state + 4 sign.
+constexpr uint32_t potts_digit(int state, bool neg, int hi) {
+  const uint32_t c = neg ? (kPottsRows - kPottsCoef[state]) & (kPottsRows - 1u) : kPottsCoef[state];
+  return hi ? c >> 5 : c & 31u;
+}
+constexpr uint32_t potts_digits(bool neg, int hi) {
+  return potts_digit(0, neg, hi) | potts_digit(1, neg, hi) << 8 | potts_digit(2, neg, hi) << 16 |
+         potts_digit(3, neg, hi) << 24;
+}
 
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_sweep_potts(const PottsParams p) {
-  dependent_launch_entry();
-  const int sq = blockIdx.y;  // sigma * Q4 + q
-  const int sigma = sq / p.Q4, q = sq - sigma * p.Q4;
-  const int tslot = sigma / p.R, a = sigma - tslot * p.R;
-  const Geom geom = p.geom;
-  const uint32_t N = geom.N;
-  const uint32_t* Jq = p.J + (size_t)q * D * N;
-  uint32_t* sp = p.spins + ((size_t)sigma * p.Q4 + q) * N;
-  const uint4* tab[4];
+struct JModel {
+  static constexpr uint32_t kRows = kPottsRows;
+  uint32_t nf[D], nb[D];  // bit 2 of a byte: the coupling is -1
+
+  __device__ __forceinline__ void prepare(const uint32_t* J, uint32_t N, const potts::Nbr<D>& n) {
 #pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int s = 4 * q + b;
-    const int k = s < p.S ? p.temp_of[((size_t)s * p.R + a) * p.K + tslot] : tslot;
-    tab[b] = p.ptab + (size_t)k * 65536u;
-  }
-  const uint32_t c2 = (TAG_POTTS << 28) | ((uint32_t)sigma << 16) | (uint32_t)q;
-  const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
-  const uint32_t w_begin = blockIdx.x * p.words_per_block;
-  const uint32_t w_end = min(w_begin + p.words_per_block, geom.half);
-  for (uint32_t w = w_begin + threadIdx.x; w < w_end; w += kBlock) {
-    const Nbr n = split_neighbours(geom, p.colour, w);
-    uint32_t jw[2 * D], nb[2 * D];
-    jw[0] = __ldg(Jq + n.self);
-    jw[1] = __ldg(Jq + n.xm);
-    jw[2] = __ldg(Jq + N + n.self);
-    jw[3] = __ldg(Jq + N + n.ym);
-    nb[0] = sp[n.xp];
-    nb[1] = sp[n.xm];
-    nb[2] = sp[n.yp];
-    nb[3] = sp[n.ym];
-    if (D == 3) {
-      jw[4] = __ldg(Jq + 2u * N + n.self);
-      jw[5] = __ldg(Jq + 2u * N + n.zm);
-      nb[4] = sp[n.zp];
-      nb[5] = sp[n.zm];
+    for (int d = 0; d < D; ++d) {
+      nf[d] = __ldg(J + (size_t)d * N + n.self);
+      nb[d] = __ldg(J + (size_t)d * N + n.bw[d]);
     }
-    const uint4 x = philox10(n.site, tk.lo, c2, tk.hi, p.keys);
-    const uint32_t rr[4] = {x.x, x.y, x.z, x.w};
-    uint32_t out = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      uint32_t npk = 0x6666u;  // nibble k holds n_k + 6
-#pragma unroll
-      for (int j = 0; j < 2 * D; ++j) {
-        const uint32_t st = (nb[j] >> (8 * b)) & 3u;
-        const int Jv = (int)(int8_t)(uint8_t)(jw[j] >> (8 * b));
-        npk += (uint32_t)(Jv << (4 * st));
-      }
-      const uint4 T = __ldg(tab[b] + npk);
-      const uint32_t r = rr[b];
-      const uint32_t ge0 = !((T.w & 1u) || r < T.x);
-      const uint32_t ge1 = !((T.w & 2u) || r < T.y);
-      const uint32_t ge2 = !((T.w & 4u) || r < T.z);
-      out |= (ge0 + ge1 + ge2) << (8 * b);
-    }
-    sp[n.self] = out;
   }
+
+  __device__ __forceinline__ void rows(const uint32_t* sf, const uint32_t* sb, uint32_t* row) const {
+    constexpr uint32_t lp = potts_digits(false, 0), ln = potts_digits(true, 0);
+    constexpr uint32_t hp = potts_digits(false, 1), hn = potts_digits(true, 1);
+    uint32_t l01 = 0, l23 = 0, h01 = 0, h23 = 0;  // samples 0 and 1, 2 and 3: two bytes each
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const uint32_t y = (sf[d] | (nf[d] & 0x04040404u)) + 16u * (sb[d] | (nb[d] & 0x04040404u));
+      const uint32_t z = y >> 16;
+      l01 += potts::prmt(lp, ln, y);
+      h01 += potts::prmt(hp, hn, y);
+      l23 += potts::prmt(lp, ln, z);
+      h23 += potts::prmt(hp, hn, z);
+    }
+    // both neighbours of every direction, then low + 32 high, two samples per word
+    auto fold = [](uint32_t x) { return (x & 0x00ff00ffu) + ((x >> 8) & 0x00ff00ffu); };
+    const uint32_t r01 = (fold(l01) + 32u * fold(h01)) & 0x03ff03ffu;
+    const uint32_t r23 = (fold(l23) + 32u * fold(h23)) & 0x03ff03ffu;
+    row[0] = r01 & 0xffffu;
+    row[1] = r01 >> 16;
+    row[2] = r23 & 0xffffu;
+    row[3] = r23 >> 16;
+  }
+
+  // a satisfied bond (equal states) counts -J
+  static __device__ __forceinline__ void count_bond(uint32_t s, uint32_t sn, uint32_t J, uint32_t& good,
+                                                    uint32_t& bad) {
+    const uint32_t eq = potts::zero2(s ^ sn);
+    good += eq & ~(J >> 1);
+    bad += eq & (J >> 1);
+  }
+};
+
+template <int D, int RT, bool KONE>
+__global__ void __launch_bounds__(kBlock, RT == 2 ? 4 : 5) k_sweep_potts(const potts::Params p) {
+  __shared__ uint4 tab[KONE ? kPottsRows : 1];
+  potts::sweep_words<JModel<D>, D, RT, KONE>(p, tab);
 }
 
 __global__ void k_init_potts(uint32_t* spins, uint32_t* J, Geom geom, int Q4, int slots, int ferro,
@@ -122,68 +119,7 @@ __global__ void k_init_potts(uint32_t* spins, uint32_t* J, Geom geom, int Q4, in
   }
 }
 
-// Per (slot, quad) block: E = -sum_bonds J delta and the state counts of the
-// 4 samples of the quad (Sec. 4.1 observables for the Potts glass).
 constexpr int kPottsMeasIters = 32;
-
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_measure_potts(const uint32_t* __restrict__ spins,
-                                                          const uint32_t* __restrict__ J, int64_t* acc, Geom geom,
-                                                          int S, int Q4, int slots) {
-  const int sq = blockIdx.y;  // sigma * Q4 + q
-  const int sigma = sq / Q4, q = sq - sigma * Q4;
-  const uint32_t N = geom.N, L = (uint32_t)geom.L, h = (uint32_t)geom.h;
-  const uint32_t* Jq = J + (size_t)q * D * N;
-  const uint32_t* sp = spins + ((size_t)sigma * Q4 + q) * N;
-  const uint32_t base = blockIdx.x * (uint32_t)(kBlock * kPottsMeasIters);
-  long long v[4][5];  // per sample: E, n0..n3
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int f = 0; f < 5; ++f) v[b][f] = 0;
-  for (int it = 0; it < kPottsMeasIters; ++it) {
-    const uint32_t j = base + (uint32_t)it * kBlock + threadIdx.x;
-    if (j >= N) continue;
-    const uint32_t rc = j / h, k = j - rc * h;
-    const uint32_t row = rc >> 1, c = rc & 1u;
-    const uint32_t y = row % L, z = row / L;
-    const uint32_t x = 2u * k + ((c ^ (y + z)) & 1u);
-    const uint32_t si = sp[j];
-    uint32_t nbw[D], jw[D];
-    nbw[0] = sp[split_index(geom, (int)((x + 1u) % L), (int)y, (int)z)];
-    nbw[1] = sp[split_index(geom, (int)x, (int)((y + 1u) % L), (int)z)];
-    jw[0] = Jq[j];
-    jw[1] = Jq[N + j];
-    if (D == 3) {
-      nbw[2] = sp[split_index(geom, (int)x, (int)y, (int)((z + 1u) % L))];
-      jw[2] = Jq[2u * N + j];
-    }
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const uint32_t st = (si >> (8 * b)) & 3u;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        const uint32_t sn = (nbw[d] >> (8 * b)) & 3u;
-        if (sn == st) v[b][0] -= (int)(int8_t)(uint8_t)(jw[d] >> (8 * b));
-      }
-      v[b][1 + st] += 1;
-    }
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int f = 0; f < 5; ++f)
-      for (int off = 16; off > 0; off >>= 1) v[b][f] += __shfl_down_sync(0xffffffffu, v[b][f], off);
-  if ((threadIdx.x & 31) == 0) {
-    for (int b = 0; b < 4; ++b) {
-      const int s = 4 * q + b;
-      if (s >= S) continue;
-      int64_t* ac = acc + ((size_t)s * slots + sigma) * kAccStride;
-      atomicAdd((unsigned long long*)&ac[0], (unsigned long long)v[b][0]);
-      for (int f = 0; f < 4; ++f) atomicAdd((unsigned long long*)&ac[2 + f], (unsigned long long)v[b][1 + f]);
-    }
-  }
-}
 
 // Q = sum_i delta(s_i^0, s_i^1) between the replica-0 and replica-1
 // configurations holding temperature k; stored in acc[s][k*R][6].
@@ -315,49 +251,19 @@ cudaError_t launch_init_potts(Lattice& lat, int jmode) {
 
 cudaError_t launch_sweep_potts(Lattice& lat, int colour, uint64_t t) {
   if (lat.model == IANUS_POTTS4_PERM) return launch_sweep_perm(lat, colour, t);
-  PottsParams p;
-  p.spins = (uint32_t*)lat.spins;
-  p.J = (const uint32_t*)lat.J;
-  p.ptab = lat.ptab;
-  p.temp_of = lat.temp_of;
-  p.geom = lat.geom;
-  p.S = lat.S;
-  p.R = lat.R;
-  p.K = lat.K;
-  p.Q4 = lat.Q4;
-  p.slots = lat.slots;
-  p.colour = colour;
-  p.t_lo = (uint32_t)(t & 0xffffffffu);
-  p.t_hi = (uint32_t)(t >> 32);
-  p.keys = lat.keys;
-  p.t_dev = lat.capturing ? lat.t_dev : nullptr;
-  const uint32_t half = lat.geom.half;
-  const uint32_t ys = (uint32_t)(lat.slots * lat.Q4);
-  uint32_t target_blocks = (152u * 8u + ys - 1) / ys;
-  uint32_t wpb = (half + target_blocks - 1) / target_blocks;
-  wpb = ((wpb + kBlock - 1) / kBlock) * kBlock;
-  if (wpb < (uint32_t)kBlock) wpb = kBlock;
-  p.words_per_block = wpb;
-  dim3 grid((half + wpb - 1) / wpb, ys);
-  void* args[] = {(void*)&p};
-  const void* k = lat.D == 3 ? (const void*)k_sweep_potts<3> : (const void*)k_sweep_potts<2>;
-  return launch_dependent(k, grid, dim3(kBlock), args, 0, lat.stream);
+  const void* k[2][2][2] = {{{(const void*)k_sweep_potts<2, 1, false>, (const void*)k_sweep_potts<2, 1, true>},
+                             {(const void*)k_sweep_potts<2, 2, false>, (const void*)k_sweep_potts<2, 2, true>}},
+                            {{(const void*)k_sweep_potts<3, 1, false>, (const void*)k_sweep_potts<3, 1, true>},
+                             {(const void*)k_sweep_potts<3, 2, false>, (const void*)k_sweep_potts<3, 2, true>}}};
+  const int rt = lat.R % 2 == 0 ? 2 : 1;
+  return potts::launch_sweep(lat, colour, t, k[lat.D - 2][rt - 1][lat.K == 1], rt, rt == 2 ? 4 : 5);
 }
 
 cudaError_t launch_measure_potts(Lattice& lat, int want_q) {
   if (lat.model == IANUS_POTTS4_PERM) return launch_measure_perm(lat, want_q);
-  cudaError_t e = cudaMemsetAsync(lat.acc, 0, (size_t)lat.S * lat.slots * kAccStride * sizeof(int64_t), lat.stream);
-  if (e != cudaSuccess) return e;
-  const uint32_t per_block = kBlock * kPottsMeasIters;
-  dim3 grid((lat.N + per_block - 1) / per_block, (unsigned)(lat.slots * lat.Q4));
   if (lat.D == 3)
-    k_measure_potts<3><<<grid, kBlock, 0, lat.stream>>>((const uint32_t*)lat.spins, (const uint32_t*)lat.J,
-                                                         lat.acc, lat.geom, lat.S, lat.Q4, lat.slots);
-  else
-    k_measure_potts<2><<<grid, kBlock, 0, lat.stream>>>((const uint32_t*)lat.spins, (const uint32_t*)lat.J,
-                                                         lat.acc, lat.geom, lat.S, lat.Q4, lat.slots);
-  if (want_q && lat.R >= 2) return launch_overlap_potts(lat);
-  return cudaGetLastError();
+    return potts::launch_measure(lat, want_q, potts::k_measure<JModel<3>, 3, 1>, potts::k_measure<JModel<3>, 3, 2>);
+  return potts::launch_measure(lat, want_q, potts::k_measure<JModel<2>, 2, 1>, potts::k_measure<JModel<2>, 2, 2>);
 }
 
 cudaError_t launch_overlap_potts(Lattice& lat) {

@@ -76,7 +76,7 @@ struct Lattice {
   void* J;              // I8: int8 [S][D][N];     BITS64: u64 [G][D][N];     U8X4: u32 [Q4][D][N]
   uint64_t* thr;        // Ising: u64 [K][kMaxClasses] threshold per class u
   uint64_t* tp;         // BITS64: u64 [G][slots][kMaxClasses][kPlanes]
-  uint4* ptab;          // Potts: uint4 [K][65536]; permutation Potts: [K][(2D+1)^3]
+  uint4* ptab;          // Potts: uint4 [K][kPottsRows]; permutation Potts: [K][perm_table_entries(D)]
   uint64_t* pttab;      // PT: u64 [K-1][pt_len], T_PT(|d| = 4m) at m-1
   int8_t* pt_sign;      // PT: sign of beta[k] - beta[k+1], [K-1]
   int32_t* slot_at;     // [S][R][K]
@@ -292,8 +292,56 @@ cudaError_t launch_get_spins_perm(Lattice& lat, int8_t* dev_out);
 cudaError_t launch_set_spins_perm(Lattice& lat, const int8_t* dev_in);
 cudaError_t launch_get_couplings_perm(Lattice& lat, int8_t* dev_out);
 cudaError_t launch_set_couplings_perm(Lattice& lat, const int8_t* dev_in);
-// compact permutation-model table: entry n0 + B (n1 + B n2), B = 2D + 1
-inline uint32_t perm_table_entries(int D) { return (uint32_t)(2 * D + 1) * (2 * D + 1) * (2 * D + 1); }
+// Rows of the heat-bath tables.  J-weighted model: row sum_k n_k coef[k] mod
+// 1024, the coefficients chosen by search so that the 833 reachable counts
+// (sum |n_k| at most 2D <= 6 and even) get different rows; the sum is linear,
+// so the kernel adds the neighbours' terms without forming the counts.
+constexpr uint32_t kPottsRows = 1024;
+constexpr uint32_t kPottsCoef[4] = {535, 249, 756, 476};
+constexpr uint32_t potts_row(int n0, int n1, int n2, int n3) {
+  return ((uint32_t)n0 * kPottsCoef[0] + (uint32_t)n1 * kPottsCoef[1] + (uint32_t)n2 * kPottsCoef[2] +
+          (uint32_t)n3 * kPottsCoef[3]) & (kPottsRows - 1u);
+}
+constexpr bool potts_rows_differ() {
+  bool seen[kPottsRows] = {};
+  for (int a = -6; a <= 6; ++a) {
+    const int ra = 6 - (a < 0 ? -a : a);
+    for (int b = -ra; b <= ra; ++b) {
+      const int rb = ra - (b < 0 ? -b : b);
+      for (int c = -rb; c <= rb; ++c) {
+        const int rc = rb - (c < 0 ? -c : c);
+        for (int d = -rc; d <= rc; ++d) {
+          if ((a + b + c + d) & 1) continue;
+          const uint32_t r = potts_row(a, b, c, d);
+          if (seen[r]) return false;
+          seen[r] = true;
+        }
+      }
+    }
+  }
+  return true;
+}
+static_assert(potts_rows_differ(), "two reachable counts share a table row");
+// Permutation model (n_0 + n_1 + n_2 + n_3 = 2D): n_0 + 37 n_1 + 16 n_2 in 2D
+// and 3D (below 256, so a byte holds it), n_0 + 9 n_1 + 73 n_2 in 4D; no two
+// reachable counts share a row.
+constexpr uint32_t perm_table_entries(int D) { return D == 4 ? 592u : 256u; }
+constexpr uint32_t perm_row(int D, int n0, int n1, int n2) {
+  return D == 4 ? (uint32_t)(n0 + 9 * n1 + 73 * n2) : (uint32_t)(n0 + 37 * n1 + 16 * n2);
+}
+constexpr bool perm_rows_differ(int D) {
+  bool seen[592] = {};
+  for (int a = 0; a <= 2 * D; ++a)
+    for (int b = 0; a + b <= 2 * D; ++b)
+      for (int c = 0; a + b + c <= 2 * D; ++c) {
+        const uint32_t r = perm_row(D, a, b, c);
+        if (r >= perm_table_entries(D) || seen[r]) return false;
+        seen[r] = true;
+      }
+  return true;
+}
+static_assert(perm_rows_differ(2) && perm_rows_differ(3) && perm_rows_differ(4),
+              "two reachable counts share a table row");
 // shared (k_pt.cu)
 cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, uint64_t* sweep_out, int want_q);
 cudaError_t launch_pt_swap(Lattice& lat);
