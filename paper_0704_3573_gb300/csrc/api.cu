@@ -562,8 +562,6 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   lat->persist_timeout_ns = 2000000000ull;  // 2 s
   lat->persist_absent = -1;
   lat->jitf_algo = -1;
-  lat->jitp[0] = lat->jitp[1] = nullptr;
-  lat->jitp_tried[0] = lat->jitp_tried[1] = false;
   lat->mut = 0;
   lat->acc_ok = false;
   lat->bytes = z.total;

@@ -183,6 +183,8 @@ struct BitsParams {
   uint32_t words_per_block;  // colour-c words handled by one block (a multiple of 32)
   PhiloxKeys keys;
   const uint64_t* t_dev;     // non-null in captured graphs: sweep = *t_dev + t_lo
+  const uint64_t* hbits;     // field models: [G][N], lane bit set where h_i < 0
+  const uint64_t* xbits;     // [G][N], lane bit set where x_i = 1
 };
 
 // Launch parameters of the persistent form of the lane-queue sweep

@@ -128,8 +128,6 @@ cudaKernel_t jit_kernel(const Lattice& lat, const UniformLut& u, int algo, int m
   if (lat.K != 1 || (lat.R != 1 && lat.R != 2)) return nullptr;  // one temperature
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  if (mode == 3) return jit_lt_kernel(lat, u, algo, min_blocks, block);
-  if (mode == 4) return jit_ltp_kernel(lat, u, algo, min_blocks, block);
   std::string pre;
   pre += "#define IANUS_JIT_D " + std::to_string(lat.D) + "\n";
   pre += "#define IANUS_JIT_ALGO " + std::to_string(algo) + "\n";
@@ -151,39 +149,6 @@ cudaKernel_t jit_kernel(const Lattice& lat, const UniformLut& u, int algo, int m
   pre += "#define IANUS_JIT_LL " + std::to_string(lat.geom.lL) + "\n";
   pre += "#include \"jit_sweep.cuh\"\n";
   return compile_cached(dev, pre, kJitSweepSrc, "jit_sweep.cuh", "ianus_jit_sweep", (int)kJitSmemBytes);
-}
-
-static cudaKernel_t jit_lt_kernel_impl(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block,
-                                       bool persist) {
-  if (lat.K != 1 || (lat.R != 1 && lat.R != 2)) return nullptr;  // one temperature
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  std::string pre;
-  pre += "#define IANUS_JIT_D " + std::to_string(lat.D) + "\n";
-  pre += "#define IANUS_JIT_ALGO " + std::to_string(algo) + "\n";
-  pre += "#define IANUS_JIT_R " + std::to_string(lat.R) + "\n";
-  pre += "#define IANUS_JIT_P2 " + std::to_string(lat.geom.lL > 0 ? 1 : 0) + "\n";
-  pre += "#define IANUS_JIT_LUTS ";
-  for (int q = 0; q < 32; ++q) pre += std::to_string((unsigned)u.t[q]) + (q < 31 ? "," : "\n");
-  pre += "#define IANUS_JIT_ALWAYS " + std::to_string((unsigned)u.always) + "\n";
-  pre += "#define IANUS_JIT_NEED " + std::to_string((unsigned)u.need) + "\n";
-  pre += "#define IANUS_JIT_MINB " + std::to_string(min_blocks) + "\n";
-  pre += "#define IANUS_JIT_BLOCK " + std::to_string(block) + "\n";
-  pre += "#define IANUS_JIT_L " + std::to_string(lat.L) + "\n";
-  pre += "#define IANUS_JIT_LH " + std::to_string(lat.geom.lh) + "\n";
-  pre += "#define IANUS_JIT_LL " + std::to_string(lat.geom.lL) + "\n";
-  pre += std::string("#define IANUS_JIT_PERSIST ") + (persist ? "1" : "0") + "\n";
-  pre += "#include \"jit_sweep_lt.cuh\"\n";
-  return compile_cached(dev, pre, kJitSweepLtSrc, "jit_sweep_lt.cuh",
-                        persist ? "ianus_jit_sweep_ltp" : "ianus_jit_sweep_lt", 0);
-}
-
-cudaKernel_t jit_lt_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block) {
-  return jit_lt_kernel_impl(lat, u, algo, min_blocks, block, false);
-}
-
-cudaKernel_t jit_ltp_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block) {
-  return jit_lt_kernel_impl(lat, u, algo, min_blocks, block, true);
 }
 
 cudaKernel_t jit_field_kernel(const Lattice& lat, int algo, int min_blocks) {
@@ -212,7 +177,6 @@ cudaKernel_t jit_field_kernel(const Lattice& lat, int algo, int min_blocks) {
   return compile_cached(dev, pre, kJitFieldSrc, "jit_field.cuh", "ianus_jit_field_sweep", 0);
 }
 
-
 cudaKernel_t jit_planes_kernel(const Lattice& lat, int algo, int rt, bool queue, int min_blocks, size_t smem) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
@@ -232,6 +196,64 @@ cudaKernel_t jit_planes_kernel(const Lattice& lat, int algo, int rt, bool queue,
   // replica count: allow it all the shared memory a block may have
   (void)smem;
   return compile_cached(dev, pre, kJitPlanesSrc, "sweep_planes.cuh", "ianus_jit_planes_sweep", 227 * 1024);
+}
+
+// Preamble of jit_sweep_lt.cuh but for its thresholds, RT replicas a thread.
+static std::string lt_preamble(const Lattice& lat, int algo, int rt, int min_blocks, int block) {
+  std::string pre;
+  pre += "#define IANUS_JIT_D " + std::to_string(lat.D) + "\n";
+  pre += "#define IANUS_JIT_ALGO " + std::to_string(algo) + "\n";
+  pre += "#define IANUS_JIT_R " + std::to_string(rt) + "\n";
+  pre += "#define IANUS_JIT_P2 " + std::to_string(lat.geom.lL > 0 ? 1 : 0) + "\n";
+  pre += "#define IANUS_JIT_MINB " + std::to_string(min_blocks) + "\n";
+  pre += "#define IANUS_JIT_BLOCK " + std::to_string(block) + "\n";
+  pre += "#define IANUS_JIT_L " + std::to_string(lat.L) + "\n";
+  pre += "#define IANUS_JIT_LH " + std::to_string(lat.geom.lh) + "\n";
+  pre += "#define IANUS_JIT_LL " + std::to_string(lat.geom.lL) + "\n";
+  return pre;
+}
+
+static std::string bytes_list(const uint8_t* t) {
+  std::string s;
+  for (int q = 0; q < 32; ++q) s += std::to_string((unsigned)t[q]) + (q < 31 ? "," : "\n");
+  return s;
+}
+
+static cudaKernel_t lt_compile(const std::string& pre, bool persist) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  const std::string all = pre + "#define IANUS_JIT_PERSIST " + (persist ? "1" : "0") + "\n" +
+                          "#include \"jit_sweep_lt.cuh\"\n";
+  return compile_cached(dev, all, kJitSweepLtSrc, "jit_sweep_lt.cuh",
+                        persist ? "ianus_jit_sweep_ltp" : "ianus_jit_sweep_lt", 0);
+}
+
+cudaKernel_t jit_lt_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block,
+                           bool persist) {
+  if (lat.K != 1 || (lat.R != 1 && lat.R != 2)) return nullptr;  // one temperature
+  std::string pre = lt_preamble(lat, algo, lat.R, min_blocks, block);
+  pre += "#define IANUS_JIT_LUTS " + bytes_list(u.t);
+  pre += "#define IANUS_JIT_ALWAYS " + std::to_string((unsigned)u.always) + "\n";
+  pre += "#define IANUS_JIT_NEED " + std::to_string((unsigned)u.need) + "\n";
+  return lt_compile(pre, persist);
+}
+
+cudaKernel_t jit_lt_field_kernel(const Lattice& lat, int algo, int min_blocks, int block) {
+  if (!lat.flut_ok || lat.K != 1 || (lat.R != 1 && lat.R != 2)) return nullptr;  // one temperature
+  std::string pre = lt_preamble(lat, algo, lat.R, min_blocks, block);
+  pre += "#define IANUS_JIT_FIELD " + std::to_string(lat.dilute ? 2 : 1) + "\n";
+  for (int f = 0; f < 2; ++f)
+    for (int h = 0; h < 2; ++h) {
+      const std::string fh = std::to_string(f) + std::to_string(h);
+      pre += "#define IANUS_JIT_LUT" + fh + " " + bytes_list(lat.flut.t[f][h]);
+      pre += "#define IANUS_JIT_ALWAYS" + fh + " " + std::to_string((unsigned)lat.flut.always[f][h]) + "\n";
+      pre += "#define IANUS_JIT_NEED" + fh + " " + std::to_string((unsigned)lat.flut.need[f][h]) + "\n";
+    }
+  return lt_compile(pre, false);
+}
+
+cudaKernel_t jit_lt_lanes_kernel(const Lattice& lat, int algo, int rt, int min_blocks, int block) {
+  return lt_compile(lt_preamble(lat, algo, rt, min_blocks, block) + "#define IANUS_JIT_LANES 1\n", false);
 }
 
 }  // namespace ianus

@@ -1072,6 +1072,35 @@ constexpr JitShape kJitShapes[] = {
 constexpr int kNumJitShapes = sizeof(kJitShapes) / sizeof(kJitShapes[0]);
 static_assert(kNumJitShapes + 1 == kMaxVariant, "variants 2..kMaxVariant are the shapes");
 constexpr int kAutoJitVariant = 24;  // the lane-queue kernel, 4 blocks of 256 per SM
+constexpr int kLtBlock = 256, kLtBlocks = 4;  // the same shape for fields and per-lane planes
+
+// Blocks per SM of the lane-queue field sweep: a pair of replicas with field
+// words (and u3 with dilution) needs more than 64 registers.
+int field_blocks(const Lattice& lat) { return lat.R == 2 ? 3 : kLtBlocks; }
+
+// The automatic and the lane-queue variants sweep fields and per-lane planes
+// with that kernel; variants 2..21 with the earlier one-word-per-thread shapes.
+bool lane_queue(const Lattice& lat) { return lat.variant == 0 || lat.variant >= 22; }
+
+// Replicas a thread of the per-lane-plane sweep does together.
+int lanes_replicas(const Lattice& lat) { return lat.R % 2 == 0 ? 2 : 1; }
+
+// Launches a colour pass of a lane-queue kernel (jit_sweep_lt.cuh): ys block
+// rows, about min_blocks blocks per SM in all (one wave), whole warps of words.
+cudaError_t launch_lt(const Lattice& lat, cudaKernel_t k, BitsParams& p, uint32_t ys, int min_blocks, int block) {
+  uint32_t w;
+  if (lat.block_words) {
+    w = (lat.block_words + 31u) / 32u * 32u;
+  } else {
+    const uint32_t per_row = std::max<uint32_t>(1u, 152u * (uint32_t)min_blocks / ys);
+    w = (lat.geom.half + per_row - 1u) / per_row;
+    w = std::max<uint32_t>(32u, (w + 31u) / 32u * 32u);
+  }
+  p.words_per_block = w;
+  void* args[] = {(void*)&p};
+  return launch_dependent((const void*)k, dim3((lat.geom.half + w - 1u) / w, ys), dim3((unsigned)block), args, 0,
+                          lat.stream);
+}
 
 // The specialised kernel shape (>= 2) that variant `variant` selects on this
 // lattice with lane-uniform tables (ulut_ok), or 1 for the per-lane kernel.
@@ -1172,15 +1201,19 @@ cudaError_t launch_sweep_persistent(Lattice& lat, int inv, uint64_t t0, uint32_t
 cudaKernel_t specialised_sweep_kernel(const Lattice& lat, const UniformLut& u, int algo, int v) {
   if (v < 2 || v >= 2 + kNumJitShapes) return nullptr;
   const JitShape& js = kJitShapes[v - 2];
+  if (js.mode >= 3) return jit_lt_kernel(lat, u, algo, js.min_blocks, js.block, js.mode == 4);
   return jit_kernel(lat, u, algo, js.mode, js.phase_a, js.min_blocks, js.group, js.jreload, js.ufirst, js.block);
 }
 
 void prepare_sweep_bits(Lattice& lat, int inv) {
   const int algo = inv ? 1 : 0;
   if (lat.field) {
-    if (lat.flut_ok && lat.variant != 1 && lat.jitf_algo != algo) {
-      lat.jitf = jit_field_kernel(lat, algo, lat.dilute && lat.R == 2 ? 2 : 3);  // the diluted pair of replicas needs room
+    const bool lq = lane_queue(lat);
+    if (lat.flut_ok && lat.variant != 1 && (lat.jitf_algo != algo || lat.jitf_lq != lq)) {
+      lat.jitf = lq ? jit_lt_field_kernel(lat, algo, field_blocks(lat), kLtBlock)
+                    : jit_field_kernel(lat, algo, lat.dilute && lat.R == 2 ? 2 : 3);
       lat.jitf_algo = algo;
+      lat.jitf_lq = lq;
     }
     return;
   }
@@ -1192,11 +1225,13 @@ void prepare_sweep_bits(Lattice& lat, int inv) {
   }
   // the per-lane planes (also the fallback of a failed specialisation),
   // compiled for the geometry unless variant 1 asks for the precompiled kernel
-  if ((v < 2 || !lat.jit) && lat.variant != 1 && !lat.jitp_tried[algo]) {
+  const int lq = lane_queue(lat) ? 1 : 0;
+  if ((v < 2 || !lat.jit) && lat.variant != 1 && !lat.jitp_tried[algo][lq]) {
     const int rt = lat.R == 1 || lat.R == 2 ? lat.R : 0;
     const bool q = algo == 1 && bits_sweep_smem(lat.R, true) <= 227u * 1024u;
-    lat.jitp[algo] = jit_planes_kernel(lat, algo, rt, q, q ? 3 : 4, (size_t)bits_sweep_smem(lat.R, q));
-    lat.jitp_tried[algo] = true;
+    lat.jitp[algo][lq] = lq ? jit_lt_lanes_kernel(lat, algo, lanes_replicas(lat), kLtBlocks, kLtBlock)
+                            : jit_planes_kernel(lat, algo, rt, q, q ? 3 : 4, (size_t)bits_sweep_smem(lat.R, q));
+    lat.jitp_tried[algo][lq] = true;
   }
 }
 
@@ -1325,6 +1360,8 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
   p.t_hi = (uint32_t)(t >> 32);
   p.keys = lat.keys;
   p.t_dev = lat.capturing ? lat.t_dev : nullptr;
+  p.hbits = lat.hbits;
+  p.xbits = lat.xbits;
   // blocks per (group, temperature slot): enough to fill the GPU ~4 deep
   const uint32_t half = lat.geom.half;
   const uint32_t gts = (uint32_t)(lat.G * lat.K);
@@ -1348,11 +1385,10 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
     const bool want_jit = lat.flut_ok && lat.variant != 1 && (lat.variant != 0 || words >= (1ull << 20));
     if (want_jit) {
       prepare_sweep_bits(lat, inv);
+      if (lat.jitf && lane_queue(lat)) return launch_lt(lat, lat.jitf, p, (uint32_t)lat.G, field_blocks(lat), kLtBlock);
       if (lat.jitf) {
-        const uint64_t* hb = lat.hbits;
-        const uint64_t* xb = lat.xbits;
         const uint8_t* lut = (const uint8_t*)(lat.fthr + (size_t)lat.K * kFieldClasses);
-        void* args[] = {(void*)&p, (void*)&hb, (void*)&xb, (void*)&lut};
+        void* args[] = {(void*)&p, (void*)&p.hbits, (void*)&p.xbits, (void*)&lut};
         return launch_dependent((const void*)lat.jitf, grid, dim3(kBlock), args, 0, lat.stream);
       }
     }
@@ -1372,21 +1408,7 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
     prepare_sweep_bits(lat, inv);
     // mode 4 (persistent) passes that run one at a time use its per-pass form
     const cudaKernel_t k3 = js.mode == 4 ? jit_lt_kernel(lat, lat.ulut, algo, js.min_blocks, js.block) : lat.jit;
-    if (k3 && (js.mode == 3 || js.mode == 4)) {
-      // one wave: about min_blocks blocks per SM in all, whole warps of words
-      uint32_t w3;
-      if (lat.block_words) {
-        w3 = (lat.block_words + 31u) / 32u * 32u;
-      } else {
-        const uint32_t per_group = std::max<uint32_t>(1u, 152u * (uint32_t)js.min_blocks / (uint32_t)lat.G);
-        w3 = (half + per_group - 1u) / per_group;
-        w3 = std::max<uint32_t>(32u, (w3 + 31u) / 32u * 32u);
-      }
-      p.words_per_block = w3;
-      void* args[] = {(void*)&p};
-      return launch_dependent((const void*)k3, dim3((half + w3 - 1u) / w3, (unsigned)lat.G), dim3(js.block), args, 0,
-                              lat.stream);
-    }
+    if (k3 && js.mode >= 3) return launch_lt(lat, k3, p, (uint32_t)lat.G, js.min_blocks, js.block);
     if (lat.jit) {
       const uint8_t* lut_t = (const uint8_t*)(lat.thr + (size_t)lat.K * kMaxClasses);
       void* args[] = {(void*)&p, (void*)&lut_t};
@@ -1398,11 +1420,14 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
   // (variant 1, or no run-time compiler) the precompiled one.
   if (lat.variant != 1) {
     prepare_sweep_bits(lat, inv);
-    if (lat.jitp[algo]) {
+    const cudaKernel_t k = lat.jitp[algo][lane_queue(lat) ? 1 : 0];
+    if (k && lane_queue(lat)) {
+      const uint64_t ys = (uint64_t)gts * (uint64_t)(lat.R / lanes_replicas(lat));
+      if (ys <= 65535u) return launch_lt(lat, k, p, (uint32_t)ys, kLtBlocks, kLtBlock);
+    } else if (k) {
       const bool q = algo == 1 && bits_sweep_smem(lat.R, true) <= 227u * 1024u;
       void* args[] = {(void*)&p};
-      return launch_dependent((const void*)lat.jitp[algo], grid, dim3(kBlock), args,
-                              (size_t)bits_sweep_smem(lat.R, q), lat.stream);
+      return launch_dependent((const void*)k, grid, dim3(kBlock), args, (size_t)bits_sweep_smem(lat.R, q), lat.stream);
     }
   }
   if (lat.D == 3)

@@ -111,6 +111,7 @@ struct Lattice {
   bool flut_ok;
   cudaKernel_t jitf;    // field sweep specialised for flut (null: per-lane planes)
   int jitf_algo;        // algorithm it was requested for; -1 = not yet
+  bool jitf_lq;         // it is the lane-queue shape
   // Parisi-Rapuano wheels (IANUS_RNG_WHEEL, I8 only): ring of 64 words per
   // (slot, sample, colour, row), I(k) at ring index k mod 64;
   // u32 [slots * S][2][64][rows], rows = N / L
@@ -144,8 +145,8 @@ struct Lattice {
   UniformLut ulut;           // valid when ulut_ok (n_temps == 1)
   bool ulut_ok;
   cudaKernel_t jit;          // sweep kernel specialised for ulut (null: use the per-lane planes)
-  cudaKernel_t jitp[2];      // per-lane-plane sweep compiled for the geometry, per algorithm (null: precompiled)
-  bool jitp_tried[2];
+  cudaKernel_t jitp[2][2];   // per-lane-plane sweep by algorithm and shape (1: lane-queue; null: precompiled)
+  bool jitp_tried[2][2];
   int jit_algo;              // algorithm the specialisation was requested for; -1 = not yet
   int jit_variant;           // variant it was built for
   uint32_t block_words;      // words per block of the bit-sliced sweep; 0 = heuristic
@@ -187,10 +188,15 @@ constexpr size_t kJitSmemBytes = 8 * 64 * (5 * 8 + 3 * 4);
 cudaKernel_t jit_kernel(const Lattice& lat, const UniformLut& u, int algo, int mode, int phase_a, int min_blocks,
                         int group, int jreload, int ufirst, int block);
 // The lane-queue shape of the same sweep (jit_sweep_lt.cuh): shared Philox
-// rounds 0..1, four plane pairs for every word, undecided lanes queued.
-cudaKernel_t jit_lt_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block);
-// Its persistent form (IANUS_JIT_PERSIST): many sweeps per launch.
-cudaKernel_t jit_ltp_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block);
+// rounds 0..1, four plane pairs for every word, undecided words queued;
+// persist: many sweeps per launch (IANUS_JIT_PERSIST).
+cudaKernel_t jit_lt_kernel(const Lattice& lat, const UniformLut& u, int algo, int min_blocks, int block,
+                           bool persist = false);
+// The same for the field models' tables lat.flut, and against per-lane
+// threshold planes with rt (1 or 2) replicas a thread, which depends on the
+// geometry only.
+cudaKernel_t jit_lt_field_kernel(const Lattice& lat, int algo, int min_blocks, int block);
+cudaKernel_t jit_lt_lanes_kernel(const Lattice& lat, int algo, int rt, int min_blocks, int block);
 // The specialised shape (>= 2) that `variant` selects on this lattice when
 // its tables are lane-uniform, or 1 when it selects none (k_msc.cu).
 int specialised_variant(const Lattice& lat, int variant);
@@ -212,11 +218,10 @@ bool persistent_variant(const Lattice& lat);
 // (no run-time compiler, or too many blocks to be resident at once): the
 // caller then sweeps with the per-pass kernels.
 cudaError_t launch_sweep_persistent(Lattice& lat, int inv, uint64_t t0, uint32_t nsweeps, bool* ran);
-// Run-time specialised random-field sweep for lat.flut (jit.cu; null when
-// unavailable).
+// The earlier shapes of the field and per-lane-plane sweeps (variants 2..21):
+// one word to its end per thread, full Philox blocks with fields.
+// rt replicas at compile time (0: run time), per-warp queues.
 cudaKernel_t jit_field_kernel(const Lattice& lat, int algo, int min_blocks);
-// The per-lane-plane sweep (sweep_planes.cuh) compiled for the lattice's
-// geometry: rt replicas at compile time (0: run time), per-warp queues.
 cudaKernel_t jit_planes_kernel(const Lattice& lat, int algo, int rt, bool queue, int min_blocks, size_t smem);
 
 // ---- launchers; each returns cudaGetLastError() of its launches ----
