@@ -683,7 +683,8 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
     if (st) return (ianus_status)st;
   }
   const int inv = algo == IANUS_HEATBATH;
-  if (lat->use_resident && resident_i8_fits(*lat) && (lat->R == 1 || measure_every == 0) && nsweeps >= 2) {
+  if (lat->use_resident && resident_i8_fits(*lat) && (lat->R == 1 || measure_every == 0) && nsweeps >= 2 &&
+      (lat->resident_mode != 1 || resident_i8_pays(*lat, measure_every))) {
     // small plain lattice: whole configurations in shared memory, many sweeps per launch
     uint64_t left = nsweeps;
     while (left > 0) {

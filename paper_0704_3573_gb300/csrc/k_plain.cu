@@ -30,6 +30,7 @@ struct I8Params {
   uint32_t t_lo, t_hi;
   PhiloxKeys keys;
   const uint64_t* t_dev;  // non-null in captured graphs
+  uint32_t lc;            // samples a thread of the shared-plane kernels updates (a multiple of 8, at most 64)
 };
 
 // r < T for the random r of (sample, slot, site, sweep), decided from the
@@ -143,12 +144,15 @@ __device__ __noinline__ bool lazy_less_from(uint32_t T32, uint32_t m0, const I8P
   return false;  // r == T
 }
 
-// grid: (tiles of kTileSites colour words, groups, slots)
+// grid: (tiles of kTileSites colour words, groups x sample chunks, slots)
 template <int D>
 __global__ void __launch_bounds__(kTileThreads) k_sweep_i8_tiled(const I8Params p) {
   __shared__ __align__(16) uint8_t s_r8[kTileSites * kTileRow];
   __shared__ uint64_t s_thr[64][kMaxClasses];
-  const uint32_t g = blockIdx.y;
+  // block row y: samples lane0 .. lane1 - 1 of group g
+  const uint32_t chunks = 64u / p.lc, g = blockIdx.y / chunks;
+  const uint32_t lane0 = p.lc * (blockIdx.y - g * chunks), lane1 = min(lane0 + p.lc, (uint32_t)p.S - 64u * g);
+  if (64u * g + lane0 >= (uint32_t)p.S) return;
   const int sigma = (int)blockIdx.z;
   const uint32_t L = (uint32_t)p.L, h = L / 2u;
   const uint32_t w0 = blockIdx.x * (uint32_t)kTileSites;
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(kTileThreads) k_sweep_i8_tiled(const I8Params 
     uint8_t* dst = s_r8 + t * kTileRow;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
+      if (8u * (uint32_t)c < lane0 || 8u * (uint32_t)c >= lane1) continue;
       // byte 7 - p of M = byte c of plane p's 64-bit word (lanes 8c .. 8c+7)
       const int hw = c >> 2, sh = 8 * (c & 3);
       uint64_t M = 0;
@@ -199,7 +204,7 @@ __global__ void __launch_bounds__(kTileThreads) k_sweep_i8_tiled(const I8Params 
     }
   }
   // thresholds of the group's samples (their temperatures may differ)
-  for (uint32_t e = t; e < 64u * kMaxClasses; e += kTileThreads) {
+  for (uint32_t e = lane0 * kMaxClasses + t; e < lane1 * kMaxClasses; e += kTileThreads) {
     const uint32_t lane = e / kMaxClasses, u = e - lane * kMaxClasses;
     const uint32_t s = 64u * g + lane;
     uint64_t T = 0;
@@ -212,11 +217,10 @@ __global__ void __launch_bounds__(kTileThreads) k_sweep_i8_tiled(const I8Params 
   }
   __syncthreads();
   if (!has_site) return;
-  // phase B: site t, every sample of the group
-  const uint32_t lanes = min(64u, (uint32_t)p.S - 64u * g);
+  // phase B: site t, every sample of the block's chunk
   const uint32_t N = p.N;
   const int8_t* r8row = reinterpret_cast<const int8_t*>(s_r8 + t * kTileRow);
-  for (uint32_t lane = 0; lane < lanes; ++lane) {
+  for (uint32_t lane = lane0; lane < lane1; ++lane) {
     const uint32_t s = 64u * g + lane;
     int8_t* sp = p.spins + ((size_t)sigma * p.S + s) * N;
     const int8_t* Jp = p.J + (size_t)s * D * N;
@@ -286,7 +290,10 @@ __global__ void __launch_bounds__(kWordThreads, 6) k_sweep_i8_words(const I8Para
   __shared__ __align__(16) uint8_t s_r8[2 * kWordThreads * kTileRow];
   __shared__ uint32_t s_thr[64][kMaxClasses];  // low 32 bits of T (the lazy path)
   __shared__ uint16_t s_t8[64][kMaxClasses];   // top 8 bits of T, 256 for T = 2^32 (always below)
-  const uint32_t g = blockIdx.y;
+  // block row y: samples lane0 .. lane1 - 1 of group g
+  const uint32_t chunks = 64u / p.lc, g = blockIdx.y / chunks;
+  const uint32_t lane0 = p.lc * (blockIdx.y - g * chunks), lane1 = min(lane0 + p.lc, (uint32_t)p.S - 64u * g);
+  if (64u * g + lane0 >= (uint32_t)p.S) return;
   const int sigma = (int)blockIdx.z;
   const uint32_t L = (uint32_t)p.L, N = p.N, nq = N / 4u, qrow = L / 4u;
   const uint32_t q0 = blockIdx.x * (uint32_t)kWordThreads;
@@ -320,6 +327,7 @@ __global__ void __launch_bounds__(kWordThreads, 6) k_sweep_i8_words(const I8Para
       uint8_t* dst = s_r8 + ((uint32_t)j * kWordThreads + t) * kTileRow;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
+        if (8u * (uint32_t)c < lane0 || 8u * (uint32_t)c >= lane1) continue;
         const int hw = c >> 2, sh = 8 * (c & 3);
         uint64_t M = 0;
 #pragma unroll
@@ -330,7 +338,7 @@ __global__ void __launch_bounds__(kWordThreads, 6) k_sweep_i8_words(const I8Para
       }
     }
   }
-  for (uint32_t e = t; e < 64u * kMaxClasses; e += kWordThreads) {
+  for (uint32_t e = lane0 * kMaxClasses + t; e < lane1 * kMaxClasses; e += kWordThreads) {
     const uint32_t lane = e / kMaxClasses, u = e - lane * kMaxClasses;
     const uint32_t s = 64u * g + lane;
     uint64_t T = 0;
@@ -356,15 +364,14 @@ __global__ void __launch_bounds__(kWordThreads, 6) k_sweep_i8_words(const I8Para
     o.zp = L * (y + L * (z + 1u == L ? 0u : z + 1u)) + x0;
     o.zm = L * (y + L * (z == 0u ? L - 1u : z - 1u)) + x0;
   }
-  const uint32_t lanes = min(64u, (uint32_t)p.S - 64u * g);
   const uint32_t sh1 = 8u * b0, sh2 = 8u * (b0 + 2u);
   int8_t* spl = p.spins + ((size_t)sigma * p.S + 64u * g) * N;
   const int8_t* Jl = p.J + (size_t)64u * g * D * N;
   WordLoads<D> cur, nxt;
-  load_word<D>(cur, spl, Jl, N, o);
+  load_word<D>(cur, spl + (size_t)lane0 * N, Jl + (size_t)lane0 * D * N, N, o);
 #pragma unroll 1
-  for (uint32_t lane = 0; lane < lanes; ++lane) {
-    if (lane + 1u < lanes) load_word<D>(nxt, spl + (size_t)(lane + 1u) * N, Jl + (size_t)(lane + 1u) * D * N, N, o);
+  for (uint32_t lane = lane0; lane < lane1; ++lane) {
+    if (lane + 1u < lane1) load_word<D>(nxt, spl + (size_t)(lane + 1u) * N, Jl + (size_t)(lane + 1u) * D * N, N, o);
     // sign bit 7 of each byte: bond unsatisfied
     const uint32_t self = cur.self;
     uint32_t cnt = ((self ^ __funnelshift_r(self, cur.next, 8) ^ cur.j0s) >> 7) & 0x01010101u;  // x + 1
@@ -2016,8 +2023,41 @@ cudaError_t launch_init_i8(Lattice& lat, int jmode) {
   return cudaGetLastError();
 }
 
+// Kernels of a plain colour pass: one thread per update (a pass costs little
+// but each update draws its own Philox blocks, 54 updates/ns), the random
+// planes shared by the 64 samples of a group (a thread takes 8 to 64 samples
+// in turn), and the bit-sliced tiles.
+enum class PlainPath { kThread, kShared, kSliced };
+
+// Estimated us per sweep, from sweeps of 2D and 3D lattices of L = 6 .. 240
+// with 1 to 200 samples: the fixed part is the latency of two passes.
+struct PlainChoice {
+  PlainPath path;
+  double us;
+};
+
+PlainChoice plain_choice(const Lattice& lat) {
+  const double k = 1e-3 * (double)lat.slots * (double)lat.S * (double)lat.N;  // thousand updates per sweep
+  PlainChoice best{PlainPath::kThread, 6.2 + k / 54.0};
+  const double shared = 6.0 + 1.1 * std::min(lat.S, 8) + k / 150.0;
+  if (shared < best.us) best = PlainChoice{PlainPath::kShared, shared};
+  if (i8_sliced_fits(lat)) {
+    const double sliced = (lat.L == 128 ? 16.0 : lat.D == 2 ? 8.5 : 12.0) + k / 400.0;
+    if (sliced < best.us) best = PlainChoice{PlainPath::kSliced, sliced};
+  }
+  return best;
+}
+
+PlainPath plain_path(const Lattice& lat) {
+  // with the small-lattice sweeps switched off, the large-lattice choice
+  if (lat.variant == 0 && !lat.use_resident) return i8_sliced_fits(lat) ? PlainPath::kSliced : PlainPath::kShared;
+  if (lat.variant == 0) return plain_choice(lat).path;
+  return lat.variant == 1 ? PlainPath::kThread : PlainPath::kShared;
+}
+
 cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
   I8Params p;
+  p.lc = 64u;
   p.spins = (int8_t*)lat.spins;
   p.J = (const int8_t*)lat.J;
   p.thr = lat.thr;
@@ -2068,26 +2108,28 @@ cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
       k_sweep_field_i8<2><<<grid, 256, 0, lat.stream>>>(fp);
     return cudaGetLastError();
   }
-  if (lat.variant == 0 && i8_sliced_fits(lat)) {  // bit-sliced in shared memory, the automatic choice
+  const PlainPath path = plain_path(lat);
+  if (path == PlainPath::kSliced) {  // bit-sliced in shared memory
     if (lat.D == 3) return inv ? launch_sliced<3, 1>(lat, p) : launch_sliced<3, 0>(lat, p);
     return inv ? launch_sliced<2, 1>(lat, p) : launch_sliced<2, 0>(lat, p);
   }
-  if (lat.variant != 1 && lat.L % 4 == 0) {  // the word kernel: 4-byte words, planes shared by the group
-    const dim3 wgrid((lat.N / 4u + kWordThreads - 1) / kWordThreads, (unsigned)lat.G, (unsigned)lat.slots);
-    if (lat.D == 3)
-      k_sweep_i8_words<3><<<wgrid, kWordThreads, 0, lat.stream>>>(p);
+  if (path == PlainPath::kShared) {  // planes shared by the group: the word kernel, or by bytes
+    const uint32_t per = lat.L % 4 == 0 ? 4u * kWordThreads : 2u * kTileSites;
+    const uint32_t tiles = (lat.N + per - 1) / per;
+    // samples a thread: all 64 when that fills the GPU, else down to 8, so
+    // that few tiles do not take their samples one after another
+    p.lc = 64u;
+    while (p.lc > 8u && (uint64_t)tiles * (uint64_t)lat.G * (64u / p.lc) * (uint64_t)lat.slots < 152u * 6u) p.lc /= 2u;
+    const dim3 sgrid(tiles, (unsigned)lat.G * (64u / p.lc), (unsigned)lat.slots);
+    if (lat.L % 4 == 0)
+      lat.D == 3 ? k_sweep_i8_words<3><<<sgrid, kWordThreads, 0, lat.stream>>>(p)
+                 : k_sweep_i8_words<2><<<sgrid, kWordThreads, 0, lat.stream>>>(p);
     else
-      k_sweep_i8_words<2><<<wgrid, kWordThreads, 0, lat.stream>>>(p);
+      lat.D == 3 ? k_sweep_i8_tiled<3><<<sgrid, kTileThreads, 0, lat.stream>>>(p)
+                 : k_sweep_i8_tiled<2><<<sgrid, kTileThreads, 0, lat.stream>>>(p);
     return cudaGetLastError();
   }
-  if (lat.variant != 1) {  // the tiled kernel (planes shared by the group); variant 1: one thread per update
-    const dim3 tgrid((p.half + kTileSites - 1) / kTileSites, (unsigned)lat.G, (unsigned)lat.slots);
-    if (lat.D == 3)
-      k_sweep_i8_tiled<3><<<tgrid, kTileThreads, 0, lat.stream>>>(p);
-    else
-      k_sweep_i8_tiled<2><<<tgrid, kTileThreads, 0, lat.stream>>>(p);
-    return cudaGetLastError();
-  }
+  // one thread per update
   if (lat.D == 3)
     k_sweep_i8<3><<<grid, 256, 0, lat.stream>>>(p);
   else
@@ -2096,12 +2138,13 @@ cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
 }
 
 // Blocks per configuration of a plain measurement with `units` steps of one
-// thread each: about 8 blocks per SM in all, at least two steps a thread.
+// thread each: about 8 blocks per SM in all, at least two steps a thread; one
+// block (and no clearing of the accumulators) below 4096 steps.
 // (One block per configuration left a few large lattices on a few SMs: 370 us
 // for 2 x 2 configurations of L=54; 82^3, 16 samples, 49 sweeps with 25
 // measurements: 21.1 ms against 4.3 ms with the chunks.)
 static uint32_t meas_chunks_i8(uint64_t configs, uint64_t units) {
-  const uint64_t want = (152u * 8u + configs - 1u) / configs, most = (units + 511u) / 512u;
+  const uint64_t want = (152u * 8u + configs - 1u) / configs, most = units < 4096u ? 1u : (units + 511u) / 512u;
   return (uint32_t)std::max<uint64_t>(1u, std::min(want, most));
 }
 
@@ -2230,6 +2273,39 @@ int resident_cluster_size(const Lattice& lat, unsigned configs, bool force) {
   return 0;
 }
 
+// The cluster size of the automatic resident mode, asked of the driver once.
+int automatic_cluster_size(Lattice& lat, unsigned configs) {
+  if (!lat.cluster_known) {
+    lat.cluster_size = resident_cluster_size(lat, configs, false);
+    lat.cluster_known = true;
+  }
+  return lat.cluster_size;
+}
+
+// Whether the resident sweep is the faster one: a colour pass of a block takes
+// about 0.3 us and 1.35 us for each round of its threads over the sites, 44
+// updates/ns over the GPU at most; launch by launch, a measurement costs its
+// own launches (9 us).  3D L=34, one sample: 87 us a sweep resident (L has no
+// divisor for a larger cluster than 2), 6.6 us launched; L=16, 64 samples: 5.6
+// against 10.
+bool resident_i8_pays(Lattice& lat, uint32_t measure_every) {
+  const unsigned configs = (unsigned)(lat.slots * lat.S);
+  const int C = automatic_cluster_size(lat, configs);
+  double rounds, threads;
+  if (C > 0) {
+    const ClusterShape sh = cluster_shape(lat, C);
+    rounds = std::ceil(0.5 * sh.PA / sh.threads);
+    threads = (double)configs * C * sh.threads;
+  } else {
+    rounds = std::ceil(lat.N / 2 / 1024.0);
+    threads = configs * 1024.0;
+  }
+  const double k = 1e-3 * (double)configs * (double)lat.N;
+  const double share = std::max(1.0, threads / (152.0 * 1024.0));
+  const double resident = std::max(2.0 * (0.3 + 1.35 * rounds) * share, k / 44.0);
+  return resident <= plain_choice(lat).us + (measure_every ? 9.0 / measure_every : 0.0);
+}
+
 cudaError_t launch_resident_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t measure_every) {
   ResidentParams p;
   p.spins = (int8_t*)lat.spins;
@@ -2254,7 +2330,7 @@ cudaError_t launch_resident_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t
   const size_t smem = (size_t)lat.N * (1 + lat.D);
   const unsigned blocks = (unsigned)(lat.slots * lat.S);
   if (lat.resident_mode == 1 || lat.resident_mode == 3) {
-    const int C = resident_cluster_size(lat, blocks, lat.resident_mode == 3);
+    const int C = lat.resident_mode == 3 ? resident_cluster_size(lat, blocks, true) : automatic_cluster_size(lat, blocks);
     if (C > 0)
       return lat.D == 3 ? cluster_dispatch<3>(lat, &p, blocks, C, false, nullptr)
                         : cluster_dispatch<2>(lat, &p, blocks, C, false, nullptr);

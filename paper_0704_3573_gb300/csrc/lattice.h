@@ -156,6 +156,8 @@ struct Lattice {
   bool capturing;            // launchers pass t_dev (and an offset) while true
   bool use_graphs;
   bool use_resident;         // resident mode for small I8 lattices (default on)
+  int cluster_size;          // blocks per configuration of the resident plain sweep (when cluster_known)
+  bool cluster_known;
   int resident_mode;         // 1 = clusters when few configurations, 2 = one block each, 3 = clusters
   // The accumulators hold the measurement of the state at (acc_sweeps,
   // acc_mut) when acc_ok; mut counts changes of the state other than sweeps.
@@ -240,6 +242,8 @@ cudaError_t launch_measure_i8(Lattice& lat, int want_q);
 // (1 + D) N bytes <= kResidentSmemMax.
 constexpr size_t kResidentSmemMax = 200 * 1024;
 bool resident_i8_fits(const Lattice& lat);
+// Whether it is also the faster sweep (asked of the automatic resident mode).
+bool resident_i8_pays(Lattice& lat, uint32_t measure_every);
 // Resident bit-sliced sweeps (k_resident_bits.cu): one block per (group,
 // temperature slot) -- or per group of a fused pool -- holding its spins,
 // couplings and threshold planes in shared memory for many sweeps.  The
