@@ -185,6 +185,7 @@ struct BitsParams {
   const uint64_t* t_dev;     // non-null in captured graphs: sweep = *t_dev + t_lo
   const uint64_t* hbits;     // field models: [G][N], lane bit set where h_i < 0
   const uint64_t* xbits;     // [G][N], lane bit set where x_i = 1
+  uint32_t y0;               // first block row of this launch (lane-queue kernel)
 };
 
 // Launch parameters of the persistent form of the lane-queue sweep

@@ -717,7 +717,7 @@ __device__ __forceinline__ void fill_uniform(Shared& sh, uint32_t g, uint32_t si
 #if !IANUS_JIT_PERSIST
 
 // One colour pass: block (x, y) updates colour words [x wpb, (x + 1) wpb) of
-// R replicas of one (group, temperature slot), y = (g K + tslot) chunks + j.
+// R replicas of one (group, temperature slot), p.y0 + y = (g K + tslot) chunks + j.
 extern "C" __global__ void __launch_bounds__(ianus::jlt::kBlock, IANUS_JIT_MINB)
     ianus_jit_sweep_lt(const ianus::BitsParams p) {
   using namespace ianus;
@@ -730,7 +730,7 @@ extern "C" __global__ void __launch_bounds__(ianus::jlt::kBlock, IANUS_JIT_MINB)
   // here uses the SMs the previous launch's last blocks leave idle.
   const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
   const uint32_t chunks = (uint32_t)p.R / R;
-  const uint32_t gt = blockIdx.y / chunks, j = blockIdx.y - gt * chunks;
+  const uint32_t row = p.y0 + blockIdx.y, gt = row / chunks, j = row - gt * chunks;
   const uint32_t g = kLanes ? gt / (uint32_t)p.K : gt, tslot = kLanes ? gt - g * (uint32_t)p.K : 0u;
   const uint32_t sigma0 = tslot * (uint32_t)p.R + j * R;
   fill_uniform(sh, g, sigma0, tk, p.keys);

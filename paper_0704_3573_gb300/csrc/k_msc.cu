@@ -1097,9 +1097,13 @@ cudaError_t launch_lt(const Lattice& lat, cudaKernel_t k, BitsParams& p, uint32_
     w = std::max<uint32_t>(32u, (w + 31u) / 32u * 32u);
   }
   p.words_per_block = w;
+  // the rows of this chain (all of them but inside a graph of several)
+  const uint32_t n = lat.chains > 1 ? (uint32_t)lat.chains : 1u;
+  p.y0 = ys * (uint32_t)lat.chain / n;
+  const uint32_t y1 = ys * ((uint32_t)lat.chain + 1u) / n;
   void* args[] = {(void*)&p};
-  return launch_dependent((const void*)k, dim3((lat.geom.half + w - 1u) / w, ys), dim3((unsigned)block), args, 0,
-                          lat.stream);
+  return launch_dependent((const void*)k, dim3((lat.geom.half + w - 1u) / w, y1 - p.y0), dim3((unsigned)block), args,
+                          0, lat.stream);
 }
 
 // The specialised kernel shape (>= 2) that variant `variant` selects on this
@@ -1233,6 +1237,25 @@ void prepare_sweep_bits(Lattice& lat, int inv) {
                             : jit_planes_kernel(lat, algo, rt, q, q ? 3 : 4, (size_t)bits_sweep_smem(lat.R, q));
     lat.jitp_tried[algo][lq] = true;
   }
+}
+
+int sweep_chains_bits(const Lattice& lat, int inv) {
+  if (!lane_queue(lat)) return 1;
+  uint64_t rows;
+  if (lat.field) {
+    if (!lat.jitf) return 1;
+    rows = (uint64_t)lat.G;
+  } else {
+    const int v = jit_variant_for(lat);
+    if (v >= 2 && lat.jit && kJitShapes[v - 2].mode == 3)
+      rows = (uint64_t)lat.G;
+    else if (v < 2 && lat.jitp[inv ? 1 : 0][1])
+      rows = (uint64_t)lat.G * lat.K * (lat.R / lanes_replicas(lat));
+    else
+      return 1;
+  }
+  if (rows < 2 || rows > 65535 || rows * lat.geom.half < kChainSites) return 1;
+  return rows >= 4 ? 4 : 2;
 }
 
 cudaError_t launch_init_bits(Lattice& lat, int jmode) {

@@ -30,6 +30,7 @@ struct I8Params {
   uint32_t t_lo, t_hi;
   PhiloxKeys keys;
   const uint64_t* t_dev;  // non-null in captured graphs
+  uint32_t g0;            // first group of this launch (bit-sliced tiles)
   uint32_t lc;            // samples a thread of the shared-plane kernels updates (a multiple of 8, at most 64)
 };
 
@@ -1751,7 +1752,7 @@ __global__ void __launch_bounds__(kSlThreads, 3) k_sweep_i8_sliced(const I8Param
   // side by side, so the couplings they share are read from DRAM once
   const uint32_t tiles_y = L / kSlY;
   const uint32_t y0 = (blockIdx.y % tiles_y) * kSlY, z0 = (blockIdx.y / tiles_y) * TZ;
-  const uint32_t g = blockIdx.z;
+  const uint32_t g = p.g0 + blockIdx.z;
   const int sigma0 = (int)blockIdx.x * SB;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
@@ -2000,11 +2001,14 @@ cudaError_t launch_sliced_c(Lattice& lat, const I8Params& p, dim3 grid, size_t s
 // Two configuration slots per block when the lattice has an even number of
 // slots, else one.
 template <int D, int ALGO>
-cudaError_t launch_sliced(Lattice& lat, const I8Params& p) {
+cudaError_t launch_sliced(Lattice& lat, I8Params& p) {
   const int SB = lat.slots % 2 == 0 ? 2 : 1;
   const size_t smem = sl_smem_bytes(D, (uint32_t)lat.L, SB);
   const uint32_t tiles = (uint32_t)lat.L / kSlY * (D == 3 ? (uint32_t)lat.L / kSlZ : 1u);
-  const dim3 grid((unsigned)(lat.slots / SB), tiles, (unsigned)lat.G);
+  const uint32_t n = lat.chains > 1 ? (uint32_t)lat.chains : 1u;  // this chain's groups
+  p.g0 = (uint32_t)lat.G * (uint32_t)lat.chain / n;
+  const uint32_t g1 = (uint32_t)lat.G * ((uint32_t)lat.chain + 1u) / n;
+  const dim3 grid((unsigned)(lat.slots / SB), tiles, g1 - p.g0);
   switch (lat.L / 32 * 2 + (SB - 1)) {
     case 2: return launch_sliced_c<D, ALGO, 1, 1>(lat, p, grid, smem);
     case 3: return launch_sliced_c<D, ALGO, 1, 2>(lat, p, grid, smem);
@@ -2055,8 +2059,14 @@ PlainPath plain_path(const Lattice& lat) {
   return lat.variant == 1 ? PlainPath::kThread : PlainPath::kShared;
 }
 
+int sweep_chains_i8(const Lattice& lat) {
+  if (lat.rng == IANUS_RNG_WHEEL || lat.field || plain_path(lat) != PlainPath::kSliced || lat.G < 2) return 1;
+  return std::min(lat.G, kMaxChains);
+}
+
 cudaError_t launch_sweep_i8(Lattice& lat, int colour, uint64_t t, int inv) {
   I8Params p;
+  p.g0 = 0u;
   p.lc = 64u;
   p.spins = (int8_t*)lat.spins;
   p.J = (const int8_t*)lat.J;

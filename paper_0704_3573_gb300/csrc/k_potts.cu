@@ -259,6 +259,12 @@ cudaError_t launch_sweep_potts(Lattice& lat, int colour, uint64_t t) {
   return potts::launch_sweep(lat, colour, t, k[lat.D - 2][rt - 1][lat.K == 1], rt, rt == 2 ? 4 : 5);
 }
 
+int sweep_chains_potts(const Lattice& lat) {
+  const uint64_t pieces = (uint64_t)(lat.R % 2 == 0 ? lat.R / 2 : lat.R) * (uint64_t)lat.Q4;
+  if (pieces < 4 || pieces * lat.geom.half * (uint64_t)lat.K < kChainSites) return 1;
+  return 4;
+}
+
 cudaError_t launch_measure_potts(Lattice& lat, int want_q) {
   if (lat.model == IANUS_POTTS4_PERM) return launch_measure_perm(lat, want_q);
   if (lat.D == 3)

@@ -59,6 +59,8 @@ struct Segment {
 };
 constexpr int kMaxSegs = 64;  // per group
 
+constexpr int kMaxChains = 4;
+
 struct Lattice {
   ianus_config cfg;
   int model, D, L, S, R, K, slots, layout;
@@ -165,6 +167,8 @@ struct Lattice {
   bool acc_ok;
   bool t_dev_valid;          // *t_dev == sweeps
   cudaStream_t cap_stream;
+  cudaStream_t side_streams[kMaxChains - 1];  // the other chains of a captured block
+  int chain, chains;         // while capturing a graph of several chains: the one launched now
   std::map<uint32_t, cudaGraphExec_t>* graphs;  // by block length
 };
 
@@ -356,6 +360,14 @@ cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, ui
 cudaError_t launch_pt_swap(Lattice& lat);
 cudaError_t launch_set_tick(Lattice& lat, uint64_t value);
 cudaError_t launch_advance_tick(Lattice& lat, uint64_t by);
+// Independent chains a captured block of sweeps is split into (1 .. kMaxChains):
+// configurations that never meet: the lane-queue sweep's block rows, the
+// Potts sweep's quads and replicas, the plain bit-sliced tiles' groups.  Passes of fewer than kChainSites threads
+// (a block of 256 per SM) last as long as one launch and are not split.
+constexpr uint32_t kChainSites = 152u * 256u;
+int sweep_chains_bits(const Lattice& lat, int inv);
+int sweep_chains_potts(const Lattice& lat);
+int sweep_chains_i8(const Lattice& lat);
 // Compiles the specialised bit-sliced kernel if the next sweep will use it
 // (so that no compilation happens during stream capture).
 void prepare_sweep_bits(Lattice& lat, int inv);

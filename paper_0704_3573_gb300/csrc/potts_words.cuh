@@ -102,7 +102,7 @@ struct Params {
   uint32_t colour;
   uint32_t t_lo, t_hi;
   uint32_t per;            // words per block, < 2^30
-  uint64_t total;          // words of a temperature slot: R / RT * Q4 * half
+  uint64_t first, end;     // this launch's words of a temperature slot's R / RT * Q4 * half
   PhiloxKeys keys;
   const uint64_t* t_dev;  // non-null in captured graphs
 };
@@ -133,8 +133,8 @@ __device__ __forceinline__ void sweep_words(const Params& p, uint4* tab) {
   const Tick tk = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
   const int tslot = blockIdx.y;
   const uint32_t N = p.grid.N;
-  const uint64_t w0 = (uint64_t)blockIdx.x * p.per;
-  const uint32_t count = (uint32_t)min((uint64_t)p.per, p.total - w0);
+  const uint64_t w0 = p.first + (uint64_t)blockIdx.x * p.per;
+  const uint32_t count = (uint32_t)min((uint64_t)p.per, p.end - w0);
   const uint32_t piece0 = (uint32_t)(w0 / p.grid.half.d);
   const uint32_t off0 = (uint32_t)(w0 - (uint64_t)piece0 * p.grid.half.d);
   if (KONE) __syncthreads();
@@ -218,18 +218,21 @@ inline cudaError_t launch_sweep(Lattice& lat, int colour, uint64_t t, const void
   p.t_hi = (uint32_t)(t >> 32);
   p.keys = lat.keys;
   p.t_dev = lat.capturing ? lat.t_dev : nullptr;
-  p.total = (uint64_t)(p.R / RT) * (uint64_t)lat.Q4 * p.grid.half.d;
+  const uint64_t pieces = (uint64_t)(p.R / RT) * (uint64_t)lat.Q4, total = pieces * p.grid.half.d;
+  const uint64_t n = lat.chains > 1 ? (uint64_t)lat.chains : 1u;  // this chain's share, whole pieces
+  p.first = pieces * (uint64_t)lat.chain / n * p.grid.half.d;
+  p.end = pieces * ((uint64_t)lat.chain + 1u) / n * p.grid.half.d;
   // one wave of blocks; two or four where a thread keeps 5 or 10 words, so that
   // blocks working at the same time are neighbours in memory and the last ones
   // are short (potts_L64 64 x 2: 1695 -> 1658 us for 20 sweeps; L=96, 128 x 2:
   // 2866 -> 2701 us for 5; L=32, 128 x 2, 3.4 words a thread, would lose 8 %)
-  const uint64_t wave = 152ull * blocks_per_sm, per_thread = p.total * p.K / (wave * kBlock);
+  const uint64_t wave = 152ull * blocks_per_sm, per_thread = total * p.K / (wave * kBlock);
   const uint64_t waves = per_thread >= 40 ? 4 : per_thread >= 10 ? 2 : 1;
   const uint64_t want = std::max<uint64_t>(1, wave * waves / (uint64_t)p.K);
-  const uint64_t per = std::min<uint64_t>(((p.total + want - 1) / want + 31) / 32 * 32, 1u << 29);
+  const uint64_t per = std::min<uint64_t>(((total + want - 1) / want + 31) / 32 * 32, 1u << 29);
   p.per = (uint32_t)per;
   void* args[] = {(void*)&p};
-  return launch_dependent(k, dim3((unsigned)((p.total + per - 1) / per), (unsigned)p.K), dim3(kBlock), args, 0,
+  return launch_dependent(k, dim3((unsigned)((p.end - p.first + per - 1) / per), (unsigned)p.K), dim3(kBlock), args, 0,
                           lat.stream);
 }
 
