@@ -5,6 +5,7 @@
 // checkpoints and error reporting.  Host logic only; all per-site work runs
 // in the kernels of k_plain.cu, k_msc.cu, k_potts.cu and k_pt.cu.
 #include <cmath>
+#include <functional>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -313,6 +314,10 @@ int upload_tables(Lattice* lat, int algo, const double* beta) {
       for (uint32_t q = 0; q < m; ++q) pt[(size_t)k * lat->pt_cap + q] = col[q];
       len = std::max(len, m);
     }
+    lat->pt_falls = true;
+    for (int k = 0; k + 1 < K && lat->pt_falls; ++k)
+      lat->pt_falls = std::is_sorted(pt.begin() + (size_t)k * lat->pt_cap, pt.begin() + (size_t)(k + 1) * lat->pt_cap,
+                                     std::greater<uint64_t>());
     lat->pt_len = lat->pt_cap;  // rows are stored with stride pt_cap; zeros end each row
     (void)len;
     CK(cudaMemcpyAsync(lat->pttab, pt.data(), pt.size() * 8, cudaMemcpyHostToDevice, lat->stream));

@@ -117,6 +117,22 @@ __host__ __device__ __forceinline__ uint32_t split_index(const Geom& g, int x, i
   return (2u * row + (uint32_t)c) * (uint32_t)g.h + (uint32_t)(x >> 1);
 }
 
+// n / d for n < 2^31 by a multiplication (Granlund and Montgomery, PLDI'94).
+struct FastDiv {
+  uint32_t m, s, d;
+};
+
+#ifndef __CUDACC_RTC__
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f{0, 0, d};
+  while ((1ull << f.s) < d) ++f.s;
+  f.m = (uint32_t)(((((1ull << f.s) - d) << 32) / d) + 1u);
+  return f;
+}
+#endif
+
+__device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) { return (__umulhi(n, f.m) + n) >> f.s; }
+
 // Colour-c word w of the split layout -> coordinates and the split indices of
 // the site and of its 2D neighbours (which all have colour 1-c).
 struct Nbr {

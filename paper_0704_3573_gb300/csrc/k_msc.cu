@@ -540,43 +540,42 @@ __global__ void k_build_field_planes(uint64_t* ftp, const uint64_t* fthr, const 
   }
 }
 
-// ---- measurements: per-lane counts by vertical counters and warp bit-transposes ----
+// ---- measurements: per-lane counts in vertical counters ----
 //
 // Each thread adds the 64-bit words of its sites (bits of the unsatisfied
 // forward bonds as a 2-bit number, the spin-down bits, the disagreement bits
-// of two replicas) into per-lane counters held as bit-planes (LaneCounter),
-// up to kMeasChunk words at a time.  A flush transposes each plane's low and
-// high 32x32 halves across the warp, which leaves in thread t the plane bits
-// of sample lanes t and 32 + t of all 32 threads, so a popcount weighted by
-// the plane gives each lane's count over the warp's sites.  At the end the
+// of two replicas) into per-lane counters held as bit-planes (LaneCounter):
+// four words at a time through carry-save adders, so that only one carry of
+// four ripples through the upper planes, and kMeasChunk words at most before
+// a flush.  A flush adds the counters of the warp's threads as bit-sliced
+// numbers, a butterfly of five steps (the first splits the 64 lanes between
+// the half-warps), and reads each lane's total off the planes.  At the end the
 // block sums its warps in shared memory and adds one value per lane and
 // quantity to the accumulators.  Per site and configuration this gives U
 // (E = 2U - D N), B (M = N - 2B) and X (Q = N - 2X).
+//
+// Bound: load latency (64 to 128 registers for the planes and four sites in
+// flight, 8 to 16 warps an SM) and integer issue.  One launch, state in L2:
+// random fields L=64, 256 samples 34 -> 13.5 us; L=32, 32 temperatures x 64 x
+// 2 25 -> 17.5 us; L=64, 256 x 2 22.3 -> 20 us; L=128, 256 x 2 (from memory)
+// 112 us.  Two words at a time in 80 registers was slower (27 us at L=64).
 
 constexpr int kMeasWarps = kBlock / 32;
-constexpr int kMeasMaxQ = 7;  // quantities per block: U and B of two replicas, X, field F
+constexpr int kMeasMaxQ = 5;     // quantities per block: U and B of two replicas and X; 2 U - O, X, F
+constexpr int kMeasBatch = 4;    // words a thread adds together
+constexpr int kMeasChunk = 20;   // words a thread adds between flushes: up to 3 each (a site's forward
+                                 // bonds) fit 6 planes, up to 1 each fit 5
+constexpr int kPlanesBond = 6, kPlanesBit = 5;
 
-// 32x32 bit transpose across the warp: afterwards thread j holds, in bit t,
-// bit j of the word thread t passed in (five butterfly exchanges).
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const uint32_t sft = 16u >> i;
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
-    x = (lane & sft) ? ((x & ~M[i]) | ((y >> sft) & M[i])) : ((x & M[i]) | ((y << sft) & ~M[i]));
-  }
-  return x;
+__device__ __forceinline__ uint64_t maj3(uint64_t a, uint64_t b, uint64_t c) { return (a & b) | (c & (a ^ b)); }
+
+// c = sum bit, returns the carry of c + x + y.
+__device__ __forceinline__ uint64_t csa(uint64_t& c, uint64_t x, uint64_t y) {
+  const uint64_t k = maj3(x, y, c);
+  c ^= x ^ y;
+  return k;
 }
 
-// Per-lane counts held vertically across a thread's words: plane b has bit
-// l set when bit b of lane l's count is set.  add1 adds 0/1 per lane, add2 a
-// 2-bit number (s + 2 cy) per lane, both as ripple-carry adders over the
-// planes; flush adds the warp's per-lane totals (lanes t and 32 + t in
-// thread t) by one transpose per plane and half, and clears the counter.
-// A counter of K planes holds up to 2^K - 1, which bounds the words a
-// thread may add between flushes (kMeasChunk).
 template <int K>
 struct LaneCounter {
   uint64_t c[K];
@@ -584,67 +583,92 @@ struct LaneCounter {
 #pragma unroll
     for (int b = 0; b < K; ++b) c[b] = 0;
   }
-  __device__ __forceinline__ void add1(uint64_t x) {
+  // x of weight 2^B into plane B and up.
+  template <int B>
+  __device__ __forceinline__ void ripple(uint64_t x) {
 #pragma unroll
-    for (int b = 0; b < K; ++b) {
+    for (int b = B; b < K; ++b) {
       const uint64_t t = c[b] & x;
       c[b] ^= x;
       x = t;
     }
   }
-  __device__ __forceinline__ void add2(uint64_t s, uint64_t cy) {
-    const uint64_t t0 = c[0] & s;
-    c[0] ^= s;
-    uint64_t x = (c[1] & t0) | (c[1] & cy) | (t0 & cy);
-    c[1] ^= t0 ^ cy;
-#pragma unroll
-    for (int b = 2; b < K; ++b) {
-      const uint64_t t = c[b] & x;
-      c[b] ^= x;
-      x = t;
-    }
+  // four words of 0/1 per lane
+  __device__ __forceinline__ void add1(const uint64_t (&x)[kMeasBatch]) {
+    const uint64_t t0 = csa(c[0], x[0], x[1]), t1 = csa(c[0], x[2], x[3]);
+    ripple<2>(csa(c[1], t0, t1));
   }
+  // four 2-bit numbers s + 2 k per lane
+  __device__ __forceinline__ void add2(const uint64_t (&s)[kMeasBatch], const uint64_t (&k)[kMeasBatch]) {
+    const uint64_t t0 = csa(c[0], s[0], s[1]), t1 = csa(c[0], s[2], s[3]);
+    const uint64_t u0 = csa(c[1], k[0], k[1]), u1 = csa(c[1], k[2], k[3]), u2 = csa(c[1], t0, t1);
+    const uint64_t v0 = csa(c[2], u0, u1), v1 = c[2] & u2;
+    c[2] ^= u2;
+    ripple<4>(csa(c[3], v0, v1));
+  }
+  // Adds 2^shift sign times the warp's totals of lanes meas_lane(), + 1 to lo, hi and clears.
   __device__ __forceinline__ void flush(int shift, long long sign, long long& lo, long long& hi) {
+    const uint32_t t = threadIdx.x & 31u;
+    uint32_t p[K + 5], carry = 0;
 #pragma unroll
     for (int b = 0; b < K; ++b) {
-      lo += sign * ((long long)__popc(warp_transpose32((uint32_t)c[b])) << (shift + b));
-      hi += sign * ((long long)__popc(warp_transpose32((uint32_t)(c[b] >> 32))) << (shift + b));
+      const uint32_t l = (uint32_t)c[b], h = (uint32_t)(c[b] >> 32);
+      const uint32_t x = (t & 16u) ? h : l, y = __shfl_xor_sync(0xffffffffu, (t & 16u) ? l : h, 16);
+      p[b] = x ^ y ^ carry;
+      carry = (x & y) | (carry & (x ^ y));
       c[b] = 0;
     }
+    p[K] = carry;
+#pragma unroll
+    for (int st = 0; st < 4; ++st) {
+      carry = 0;
+#pragma unroll
+      for (int b = 0; b < K + 1 + st; ++b) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, p[b], 8 >> st), x = p[b];
+        p[b] = x ^ y ^ carry;
+        carry = (x & y) | (carry & (x ^ y));
+      }
+      p[K + 1 + st] = carry;
+    }
+    const uint32_t at = 2u * (t & 15u);
+    uint32_t n0 = 0, n1 = 0;
+#pragma unroll
+    for (int b = 0; b < K + 5; ++b) {
+      n0 |= ((p[b] >> at) & 1u) << b;
+      n1 |= ((p[b] >> (at + 1u)) & 1u) << b;
+    }
+    lo += sign * ((long long)n0 << shift);
+    hi += sign * ((long long)n1 << shift);
   }
 };
 
-// Words a thread adds between flushes: 21 words of up to 3 (a site's
-// forward bonds) fit 6 planes, of up to 1 fit 5.
-constexpr int kMeasChunk = 21;
-constexpr int kPlanesBond = 6, kPlanesBit = 5;
+// First of the two sample lanes whose totals this thread holds after a flush.
+__device__ __forceinline__ uint32_t meas_lane() {
+  const uint32_t t = threadIdx.x & 31u;
+  return 32u * (t >> 4) + 2u * (t & 15u);
+}
+
+struct MeasGeom {
+  FastDiv h, L;
+  uint32_t N;
+};
 
 // Split index j -> split indices of the forward neighbours x+1, y+1, z+1.
 struct Fwd {
   uint32_t x, y, z;
 };
 
-template <bool P2>
-__device__ __forceinline__ Fwd split_forward(const Geom& g, uint32_t j) {
-  const uint32_t h = (uint32_t)g.h, L = (uint32_t)g.L;
-  uint32_t rc, k, y, z;
-  if (P2) {
-    rc = j >> g.lh;
-    k = j & (h - 1u);
-    y = (rc >> 1) & (L - 1u);
-    z = (rc >> 1) >> g.lL;
-  } else {
-    rc = j / h;
-    k = j - rc * h;
-    y = (rc >> 1) % L;
-    z = (rc >> 1) / L;
-  }
-  const uint32_t row = rc >> 1, c = rc & 1u, oc = c ^ 1u;
-  const uint32_t x = 2u * k + ((c ^ (y + z)) & 1u);
+template <int D>
+__device__ __forceinline__ Fwd split_forward(const MeasGeom& g, uint32_t j) {
+  const uint32_t h = g.h.d, L = g.L.d;
+  const uint32_t rc = div_by(j, g.h), k = j - rc * h, row = rc >> 1, c = rc & 1u;
+  const uint32_t z = D == 3 ? div_by(row, g.L) : 0u, y = row - z * L;
+  const uint32_t xpar = (c ^ y ^ z) & 1u;
+  const uint32_t o = j + (c ? 0u - h : h);  // the other colour's word of the same row and k
   Fwd f;
-  f.x = (2u * row + oc) * h + (x + 1u == L ? 0u : (x + 1u) >> 1);
-  f.y = (2u * ((y + 1u == L ? 0u : y + 1u) + L * z) + oc) * h + k;
-  f.z = g.D == 3 ? (2u * (y + L * (z + 1u == L ? 0u : z + 1u)) + oc) * h + k : 0u;
+  f.x = o + (xpar ? (k + 1u == h ? 0u - k : 1u) : 0u);
+  f.y = o + (y + 1u == L ? 0u - 2u * h * (L - 1u) : 2u * h);
+  f.z = D == 3 ? o + (z + 1u == L ? 0u - 2u * h * L * (L - 1u) : 2u * h * L) : 0u;
   return f;
 }
 
@@ -656,7 +680,7 @@ __device__ __forceinline__ void bond_count(uint64_t b, uint64_t nx, uint64_t ny,
   if (D == 3) {
     const uint64_t ez = b ^ nz ^ Jz;
     s1 = ex ^ ey ^ ez;
-    c1 = (ex & ey) | (ex & ez) | (ey & ez);
+    c1 = maj3(ex, ey, ez);
   } else {
     s1 = ex ^ ey;
     c1 = ex & ey;
@@ -667,10 +691,11 @@ __device__ __forceinline__ void bond_count(uint64_t b, uint64_t nx, uint64_t ny,
 // per (lane, quantity) into acc[sample][row_of(q)][field_of(q)].
 __device__ __forceinline__ void block_flush(long long (*red)[64], const long long (*tot)[2], int nq, int g, int S,
                                             int64_t* acc, const int* row_off, const int* field, int row_stride) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const uint32_t l0 = meas_lane();
   for (int q = 0; q < nq; ++q) {
-    red[warp * kMeasMaxQ + q][lane] = tot[q][0];
-    red[warp * kMeasMaxQ + q][32 + lane] = tot[q][1];
+    red[warp * kMeasMaxQ + q][l0] = tot[q][0];
+    red[warp * kMeasMaxQ + q][l0 + 1u] = tot[q][1];
   }
   __syncthreads();
   for (int idx = threadIdx.x; idx < nq * 64; idx += kBlock) {
@@ -686,10 +711,10 @@ __device__ __forceinline__ void block_flush(long long (*red)[64], const long lon
 
 // One temperature (slot = replica): U and B of every replica and, with two
 // replicas, X, in one pass.  Grid (chunks, groups).
-template <int D, int R, bool P2>
+template <int D, int R>
 __global__ void __launch_bounds__(kBlock, 2) k_measure_bits_k1(const uint64_t* __restrict__ spins,
-                                                            const uint64_t* __restrict__ J, int64_t* acc, Geom geom,
-                                                            int S) {
+                                                               const uint64_t* __restrict__ J, int64_t* acc,
+                                                               MeasGeom geom, int S) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
   const int g = blockIdx.y;
   const uint32_t N = geom.N;
@@ -709,24 +734,36 @@ __global__ void __launch_bounds__(kBlock, 2) k_measure_bits_k1(const uint64_t* _
   cx.zero();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * kBlock;
-  uint32_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
+  uint64_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
   while (base < N) {
-    for (int n = 0; n < kMeasChunk && base < N; ++n, base += stride) {
-      const uint32_t j = base + lane;
-      if (j >= N) continue;
-      const Fwd f = split_forward<P2>(geom, j);
-      const uint64_t Jx = Jg[j], Jy = Jg[N + j], Jz = D == 3 ? Jg[2u * N + j] : 0ull;
-      uint64_t bw[R];
+    for (int n = 0; n < kMeasChunk / kMeasBatch && base < N; ++n, base += (uint64_t)kMeasBatch * stride) {
+      uint64_t s1[R][kMeasBatch], c1[R][kMeasBatch], bw[R][kMeasBatch];
+#pragma unroll
+      for (int q = 0; q < kMeasBatch; ++q) {
+        const uint64_t jj = base + (uint64_t)q * stride + lane;
+        const bool in = jj < N;
+        const uint32_t j = in ? (uint32_t)jj : 0u;
+        const Fwd f = split_forward<D>(geom, j);
+        const uint64_t Jx = Jg[j], Jy = Jg[N + j], Jz = D == 3 ? Jg[2u * N + j] : 0ull;
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+          const uint64_t* sp = sg + (size_t)a * N;
+          bw[a][q] = sp[j];
+          bond_count<D>(bw[a][q], sp[f.x], sp[f.y], D == 3 ? sp[f.z] : 0ull, Jx, Jy, Jz, s1[a][q], c1[a][q]);
+          if (!in) bw[a][q] = s1[a][q] = c1[a][q] = 0;
+        }
+      }
 #pragma unroll
       for (int a = 0; a < R; ++a) {
-        const uint64_t* sp = sg + (size_t)a * N;
-        uint64_t s1, c1;
-        bw[a] = sp[j];
-        bond_count<D>(bw[a], sp[f.x], sp[f.y], D == 3 ? sp[f.z] : 0ull, Jx, Jy, Jz, s1, c1);
-        cu[a].add2(s1, c1);
+        cu[a].add2(s1[a], c1[a]);
         cb[a].add1(bw[a]);
       }
-      if (R == 2) cx.add1(bw[0] ^ bw[R - 1]);
+      if (R == 2) {
+        uint64_t x[kMeasBatch];
+#pragma unroll
+        for (int q = 0; q < kMeasBatch; ++q) x[q] = bw[0][q] ^ bw[R - 1][q];
+        cx.add1(x);
+      }
     }
 #pragma unroll
     for (int a = 0; a < R; ++a) {
@@ -751,10 +788,10 @@ __global__ void __launch_bounds__(kBlock, 2) k_measure_bits_k1(const uint64_t* _
 
 // Any number of temperatures: U and B of one slot.  Grid (chunks, groups x
 // slots).
-template <int D, bool P2, bool EONLY = false>
+template <int D, bool EONLY = false>
 __global__ void __launch_bounds__(kBlock) k_measure_bits(const uint64_t* __restrict__ spins,
-                                                         const uint64_t* __restrict__ J, int64_t* acc, Geom geom,
-                                                         int S, int R, int K, int slots) {
+                                                         const uint64_t* __restrict__ J, int64_t* acc, MeasGeom geom,
+                                                         int S, int slots) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
   const int gt = blockIdx.y;  // g * slots + sigma
   const int g = gt / slots, sigma = gt - g * slots;
@@ -768,16 +805,21 @@ __global__ void __launch_bounds__(kBlock) k_measure_bits(const uint64_t* __restr
   cb.zero();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * kBlock;
-  uint32_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
+  uint64_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
   while (base < N) {
-    for (int n = 0; n < kMeasChunk && base < N; ++n, base += stride) {
-      const uint32_t j = base + lane;
-      if (j >= N) continue;
-      const Fwd f = split_forward<P2>(geom, j);
-      const uint64_t bw = sp[j];
-      uint64_t s1, c1;
-      bond_count<D>(bw, sp[f.x], sp[f.y], D == 3 ? sp[f.z] : 0ull, Jg[j], Jg[N + j], D == 3 ? Jg[2u * N + j] : 0ull,
-                    s1, c1);
+    for (int n = 0; n < kMeasChunk / kMeasBatch && base < N; ++n, base += (uint64_t)kMeasBatch * stride) {
+      uint64_t s1[kMeasBatch], c1[kMeasBatch], bw[kMeasBatch];
+#pragma unroll
+      for (int q = 0; q < kMeasBatch; ++q) {
+        const uint64_t jj = base + (uint64_t)q * stride + lane;
+        const bool in = jj < N;
+        const uint32_t j = in ? (uint32_t)jj : 0u;
+        const Fwd f = split_forward<D>(geom, j);
+        bw[q] = sp[j];
+        bond_count<D>(bw[q], sp[f.x], sp[f.y], D == 3 ? sp[f.z] : 0ull, Jg[j], Jg[N + j],
+                      D == 3 ? Jg[2u * N + j] : 0ull, s1[q], c1[q]);
+        if (!in) bw[q] = s1[q] = c1[q] = 0;
+      }
       cu.add2(s1, c1);
       if (!EONLY) cb.add1(bw);
     }
@@ -792,13 +834,14 @@ __global__ void __launch_bounds__(kBlock) k_measure_bits(const uint64_t* __restr
 // E_J = sum over forward bonds with both ends occupied of (2 e - 1), as
 // 2 U - O with U, O the per-site counts of occupied unsatisfied and occupied
 // bonds (each a 2-bit sum); M = sum x s = X - 2 sum x b and F = sum sign(h)
-// x s = X - 2 sum x (b ^ hb), X = sum x.  acc[0..2] = E_J, M, F.
-template <int D, bool P2>
-__global__ void __launch_bounds__(kBlock) k_measure_field_bits(const uint64_t* __restrict__ spins,
-                                                               const uint64_t* __restrict__ J,
-                                                               const uint64_t* __restrict__ hbits,
-                                                               const uint64_t* __restrict__ xbits, int64_t* acc,
-                                                               Geom geom, int S, int slots) {
+// x s = X - 2 sum x (b ^ hb), X = sum x.  acc[0..2] = E_J, M, F.  Without
+// dilution (DIL false) O = D N and X = N need no counting.
+template <int D, bool DIL>
+__global__ void __launch_bounds__(kBlock, 2) k_measure_field_bits(const uint64_t* __restrict__ spins,
+                                                                  const uint64_t* __restrict__ J,
+                                                                  const uint64_t* __restrict__ hbits,
+                                                                  const uint64_t* __restrict__ xbits, int64_t* acc,
+                                                                  MeasGeom geom, int S, int slots) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
   const int gt = blockIdx.y;  // g * slots + sigma
   const int g = gt / slots, sigma = gt - g * slots;
@@ -819,34 +862,66 @@ __global__ void __launch_bounds__(kBlock) k_measure_field_bits(const uint64_t* _
   cxf.zero();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * kBlock;
-  uint32_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
+  uint64_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
   while (base < N) {
-    for (int n = 0; n < kMeasChunk && base < N; ++n, base += stride) {
-      const uint32_t j = base + lane;
-      if (j >= N) continue;
-      const Fwd f = split_forward<P2>(geom, j);
-      const uint64_t b = sp[j];
-      const uint64_t xs = Xg[j];
-      const uint64_t ox = xs & Xg[f.x], oy = xs & Xg[f.y], oz = D == 3 ? xs & Xg[f.z] : 0ull;
-      const uint64_t ux = ox & (b ^ sp[f.x] ^ Jg[j]), uy = oy & (b ^ sp[f.y] ^ Jg[N + j]);
-      const uint64_t uz = D == 3 ? oz & (b ^ sp[f.z] ^ Jg[2u * N + j]) : 0ull;
-      cuu.add2(ux ^ uy ^ uz, (ux & uy) | (ux & uz) | (uy & uz));
-      coo.add2(ox ^ oy ^ oz, (ox & oy) | (ox & oz) | (oy & oz));
-      cxs.add1(xs);
-      cxb.add1(xs & b);
-      cxf.add1(xs & (b ^ Hg[j]));
+    for (int n = 0; n < kMeasChunk / kMeasBatch && base < N; ++n, base += (uint64_t)kMeasBatch * stride) {
+      uint64_t us[kMeasBatch], uc[kMeasBatch], os[kMeasBatch], oc[kMeasBatch];
+      uint64_t xw[kMeasBatch], xb[kMeasBatch], xf[kMeasBatch];
+#pragma unroll
+      for (int q = 0; q < kMeasBatch; ++q) {
+        const uint64_t jj = base + (uint64_t)q * stride + lane;
+        const bool in = jj < N;
+        const uint32_t j = in ? (uint32_t)jj : 0u;
+        const Fwd f = split_forward<D>(geom, j);
+        const uint64_t b = sp[j];
+        uint64_t ux = b ^ sp[f.x] ^ Jg[j], uy = b ^ sp[f.y] ^ Jg[N + j];
+        uint64_t uz = D == 3 ? b ^ sp[f.z] ^ Jg[2u * N + j] : 0ull;
+        if (DIL) {
+          const uint64_t xs = Xg[j];
+          const uint64_t ox = xs & Xg[f.x], oy = xs & Xg[f.y], oz = D == 3 ? xs & Xg[f.z] : 0ull;
+          ux &= ox;
+          uy &= oy;
+          uz &= oz;
+          os[q] = in ? ox ^ oy ^ oz : 0ull;
+          oc[q] = in ? maj3(ox, oy, oz) : 0ull;
+          xw[q] = in ? xs : 0ull;
+        } else {
+          xw[q] = in ? ~0ull : 0ull;
+        }
+        us[q] = in ? ux ^ uy ^ uz : 0ull;
+        uc[q] = in ? maj3(ux, uy, uz) : 0ull;
+        xb[q] = xw[q] & b;
+        xf[q] = xw[q] & (b ^ Hg[j]);
+      }
+      cuu.add2(us, uc);
+      cxb.add1(xb);
+      cxf.add1(xf);
+      if (DIL) {
+        coo.add2(os, oc);
+        cxs.add1(xw);
+      }
     }
     // E_J = 2U - O, M = X - 2 XB, F = X - 2 XF
     cuu.flush(1, 1, tot[0][0], tot[0][1]);
-    coo.flush(0, -1, tot[0][0], tot[0][1]);
-    long long xl = 0, xh = 0;
-    cxs.flush(0, 1, xl, xh);
-    tot[1][0] += xl;
-    tot[1][1] += xh;
-    tot[2][0] += xl;
-    tot[2][1] += xh;
     cxb.flush(1, -1, tot[1][0], tot[1][1]);
     cxf.flush(1, -1, tot[2][0], tot[2][1]);
+    if (DIL) {
+      coo.flush(0, -1, tot[0][0], tot[0][1]);
+      long long xl = 0, xh = 0;
+      cxs.flush(0, 1, xl, xh);
+      tot[1][0] += xl;
+      tot[1][1] += xh;
+      tot[2][0] += xl;
+      tot[2][1] += xh;
+    }
+  }
+  if (!DIL && blockIdx.x == 0 && threadIdx.x < 32u) {  // O = D N and X = N, once per lane
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      tot[0][l] -= (long long)D * N;
+      tot[1][l] += N;
+      tot[2][l] += N;
+    }
   }
   const int row_off[3] = {sigma, sigma, sigma}, field[3] = {0, 1, 2};
   block_flush(red, tot, 3, g, S, acc, row_off, field, slots);
@@ -854,12 +929,104 @@ __global__ void __launch_bounds__(kBlock) k_measure_field_bits(const uint64_t* _
 
 // Overlap at temperature k between replicas 0 and 1 (Sec. 4.1).  After
 // parallel-tempering swaps the configuration holding temperature k differs
-// per sample, so the word of replica a at temperature k is assembled lane by
-// lane: W_a = OR_t (sel[a][t] & spins[t*R + a]), sel[a][t] = lanes whose
-// temperature k sits in slot t.  X = count per lane of W_0 ^ W_1, Q = N - 2X,
-// stored in acc[s][k*R][6].  Grid (chunks, groups x temperatures).
-// With occupations (field models) the value Q = sum x (1 - 2 (w0 ^ w1)) is
-// stored instead of the count.
+// per sample: lane l of temperature k compares slot slot_at[l][0][k] of
+// replica 0 with slot_at[l][1][k] of replica 1.  X = disagreements per lane,
+// Q = N - 2X, stored in acc[s][k*R][6]; with occupations (field models) the
+// value Q = sum x (1 - 2 (w0 ^ w1)) instead of the count.
+//
+// Up to kOverlapTemps temperatures: a block takes 32 sites at a time.  Each
+// slot's 32 words are transposed across a warp into one 32-site word per
+// lane, in shared memory [slot][lane]; a thread then looks up the two slots of
+// its (temperature, lane) pairs and counts the differing bits.  Every spin
+// word is read once, where a pass per temperature reads them K times: K = 32,
+// L = 32, 64 x 2: 58 -> 26.6 us.  Grid (chunks, groups).
+constexpr int kOverlapTemps = 64;
+
+// 32x32 bit transpose across the warp: afterwards thread j holds, in bit t,
+// bit j of the word thread t passed in (five butterfly exchanges).
+__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const uint32_t sft = 16u >> i;
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
+    x = (lane & sft) ? ((x & ~M[i]) | ((y >> sft) & M[i])) : ((x & M[i]) | ((y << sft) & ~M[i]));
+  }
+  return x;
+}
+
+template <int PAIRS>
+__global__ void __launch_bounds__(kBlock, PAIRS <= 8 ? 4 : 2) k_overlap_bits_tile(const uint64_t* __restrict__ spins,
+                                                              const int32_t* __restrict__ slot_at,
+                                                              const uint64_t* __restrict__ xbits, int64_t* acc,
+                                                              uint32_t N, int S, int R, int K, int slots) {
+  extern __shared__ uint32_t rows[];  // [2 K (+ 1 with occupations)][64]: slot t of replica a in row a K + t
+  const int g = blockIdx.y;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint64_t* sg = spins + (size_t)g * slots * N;
+  // this thread's pairs: p = threadIdx + 256 i, lane p mod 64 of temperature p / 64
+  uint32_t at0[PAIRS], at1[PAIRS];
+  int n[PAIRS];
+#pragma unroll
+  for (int i = 0; i < PAIRS; ++i) {
+    const int p = (int)threadIdx.x + kBlock * i, k = p >> 6, l = p & 63, s = 64 * g + l;
+    const bool in = k < K && s < S;
+    at0[i] = 64u * (uint32_t)(in ? slot_at[((size_t)s * R + 0) * K + k] : 0) + (uint32_t)l;
+    at1[i] = 64u * (uint32_t)(K + (in ? slot_at[((size_t)s * R + 1) * K + k] : 0)) + (uint32_t)l;
+    n[i] = 0;
+  }
+  const int nrows = 2 * K + (xbits ? 1 : 0);
+  for (uint32_t j0 = blockIdx.x * 32u; j0 < N; j0 += gridDim.x * 32u) {
+    const uint32_t j = j0 + lane;
+    for (int r0 = (int)warp; r0 < nrows; r0 += 4 * kMeasWarps) {  // four rows' loads in flight
+      uint64_t w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * kMeasWarps;
+        w[q] = 0;
+        if (j < N && r < 2 * K) {
+          const int a = r >= K ? 1 : 0, t = r - a * K;
+          w[q] = sg[((size_t)t * R + a) * N + j];
+        } else if (j < N && r < nrows) {
+          w[q] = xbits[(size_t)g * N + j];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * kMeasWarps;
+        if (r >= nrows) break;  // uniform across the warp
+        rows[64 * r + (int)lane] = warp_transpose32((uint32_t)w[q]);
+        rows[64 * r + 32 + (int)lane] = warp_transpose32((uint32_t)(w[q] >> 32));
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PAIRS; ++i) {
+      const int p = (int)threadIdx.x + kBlock * i;
+      if ((p >> 6) >= K) continue;
+      const uint32_t d = rows[at0[i]] ^ rows[at1[i]];
+      if (xbits) {
+        const uint32_t x = rows[64 * 2 * K + (p & 63)];
+        n[i] += __popc(x) - 2 * __popc(x & d);
+      } else {
+        n[i] += __popc(d);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < PAIRS; ++i) {
+    const int p = (int)threadIdx.x + kBlock * i, k = p >> 6, s = 64 * g + (p & 63);
+    if (k < K && s < S && n[i] != 0)
+      atomicAdd((unsigned long long*)&acc[((size_t)s * slots + (size_t)k * R) * kAccStride + 6],
+                (unsigned long long)(long long)n[i]);
+  }
+}
+
+// More temperatures: the word of replica a at temperature k assembled lane by
+// lane, W_a = OR_t (sel[a][t] & spins[t*R + a]), sel[a][t] = lanes whose
+// temperature k sits in slot t.  Grid (chunks, groups x temperatures).
 __global__ void __launch_bounds__(kBlock) k_overlap_bits(const uint64_t* __restrict__ spins,
                                                          const int32_t* __restrict__ slot_at,
                                                          const uint64_t* __restrict__ xbits, int64_t* acc,
@@ -886,24 +1053,26 @@ __global__ void __launch_bounds__(kBlock) k_overlap_bits(const uint64_t* __restr
   cw.zero();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * kBlock;
-  uint32_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
+  uint64_t base = blockIdx.x * kBlock + (threadIdx.x & ~31u);  // uniform across the warp
   while (base < N) {
-    for (int n = 0; n < kMeasChunk && base < N; ++n, base += stride) {
-      const uint32_t j = base + lane;
-      if (j >= N) continue;
-      uint64_t w0 = 0, w1 = 0;
-      for (int t = 0; t < K; ++t) {
-        const uint64_t m0 = sel[t], m1 = sel[K + t];
-        if (m0) w0 |= m0 & sg[((size_t)t * R + 0) * N + j];
-        if (m1) w1 |= m1 & sg[((size_t)t * R + 1) * N + j];
+    for (int n = 0; n < kMeasChunk / kMeasBatch && base < N; ++n, base += (uint64_t)kMeasBatch * stride) {
+      uint64_t d[kMeasBatch], x[kMeasBatch];
+#pragma unroll
+      for (int q = 0; q < kMeasBatch; ++q) {
+        const uint64_t jj = base + (uint64_t)q * stride + lane;
+        const bool in = jj < N;
+        const uint32_t j = in ? (uint32_t)jj : 0u;
+        uint64_t w0 = 0, w1 = 0;
+        for (int t = 0; t < K; ++t) {
+          const uint64_t m0 = sel[t], m1 = sel[K + t];
+          if (m0) w0 |= m0 & sg[((size_t)t * R + 0) * N + j];
+          if (m1) w1 |= m1 & sg[((size_t)t * R + 1) * N + j];
+        }
+        x[q] = !in ? 0ull : xbits ? xbits[(size_t)g * N + j] : ~0ull;
+        d[q] = x[q] & (w0 ^ w1);
       }
-      if (xbits) {
-        const uint64_t xw = xbits[(size_t)g * N + j];
-        cw.add1(xw);
-        cd.add1(xw & (w0 ^ w1));
-      } else {
-        cd.add1(w0 ^ w1);
-      }
+      cd.add1(d);
+      if (xbits) cw.add1(x);
     }
     if (xbits) {  // Q = sum x (1 - 2 (w0 ^ w1))
       cw.flush(0, 1, tot[0][0], tot[0][1]);
@@ -1469,35 +1638,51 @@ inline unsigned meas_blocks(uint32_t N, unsigned ys) {
   return want < 1u ? 1u : (want > most ? most : want);
 }
 
-template <int D, bool P2>
+template <int PAIRS>
+cudaError_t overlap_tile(Lattice& lat, const uint64_t* xbits) {
+  const size_t smem = (size_t)(2 * lat.K + (xbits ? 1 : 0)) * 64 * sizeof(uint32_t);
+  // about four blocks per SM, each tile of 32 sites once
+  const unsigned tiles = (lat.N + 31u) / 32u, want = (152u * 4u + (unsigned)lat.G - 1u) / (unsigned)lat.G;
+  k_overlap_bits_tile<PAIRS><<<dim3(std::min(tiles, want), (unsigned)lat.G), kBlock, smem, lat.stream>>>(
+      (const uint64_t*)lat.spins, lat.slot_at, xbits, lat.acc, lat.N, lat.S, lat.R, lat.K, lat.slots);
+  return cudaGetLastError();
+}
+
+template <int D>
 cudaError_t measure_dispatch(Lattice& lat, int want_q, bool energy_only) {
   const uint64_t* sp = (const uint64_t*)lat.spins;
   const uint64_t* J = (const uint64_t*)lat.J;
-  if (energy_only && !lat.field) {  // U of every configuration, for the PT swap
-    dim3 grid(meas_blocks(lat.N, (unsigned)(lat.G * lat.slots)), (unsigned)(lat.G * lat.slots));
-    k_measure_bits<D, P2, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S, lat.R, lat.K,
-                                                                 lat.slots);
-    return cudaGetLastError();
-  }
+  const MeasGeom geom{fast_div((uint32_t)lat.geom.h), fast_div((uint32_t)lat.geom.L), lat.N};
   if (lat.K == 1 && (lat.R == 1 || lat.R == 2) && !lat.field) {
     // one pass for E, M and (R == 2) Q
     dim3 grid(meas_blocks(lat.N, (unsigned)lat.G), (unsigned)lat.G);
     if (lat.R == 2)
-      k_measure_bits_k1<D, 2, P2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S);
+      k_measure_bits_k1<D, 2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S);
     else
-      k_measure_bits_k1<D, 1, P2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S);
+      k_measure_bits_k1<D, 1><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S);
     return cudaGetLastError();
   }
   dim3 grid(meas_blocks(lat.N, (unsigned)(lat.G * lat.slots)), (unsigned)(lat.G * lat.slots));
-  if (lat.field)
-    k_measure_field_bits<D, P2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.hbits, lat.xbits, lat.acc, lat.geom,
-                                                                 lat.S, lat.slots);
+  if (energy_only && !lat.field) {  // U of every configuration, for the PT swap
+    k_measure_bits<D, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots);
+    return cudaGetLastError();
+  }
+  if (lat.field && lat.dilute)
+    k_measure_field_bits<D, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.hbits, lat.xbits, lat.acc, geom, lat.S,
+                                                                   lat.slots);
+  else if (lat.field)
+    k_measure_field_bits<D, false><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.hbits, lat.xbits, lat.acc, geom, lat.S,
+                                                                    lat.slots);
   else
-    k_measure_bits<D, P2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, lat.geom, lat.S, lat.R, lat.K, lat.slots);
+    k_measure_bits<D><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots);
   if (want_q && lat.R >= 2) {
+    const uint64_t* xb = lat.field ? lat.xbits : nullptr;
+    if (lat.K <= 16) return overlap_tile<4>(lat, xb);
+    if (lat.K <= 32) return overlap_tile<8>(lat, xb);
+    if (lat.K <= kOverlapTemps) return overlap_tile<kOverlapTemps / 4>(lat, xb);
     dim3 gq(meas_blocks(lat.N, (unsigned)(lat.G * lat.K)), (unsigned)(lat.G * lat.K));
-    k_overlap_bits<<<gq, kBlock, 2 * lat.K * sizeof(uint64_t), lat.stream>>>(
-        sp, lat.slot_at, lat.field ? lat.xbits : nullptr, lat.acc, lat.N, lat.S, lat.R, lat.K, lat.slots);
+    k_overlap_bits<<<gq, kBlock, 2 * lat.K * sizeof(uint64_t), lat.stream>>>(sp, lat.slot_at, xb, lat.acc, lat.N,
+                                                                             lat.S, lat.R, lat.K, lat.slots);
   }
   return cudaGetLastError();
 }
@@ -1505,12 +1690,7 @@ cudaError_t measure_dispatch(Lattice& lat, int want_q, bool energy_only) {
 cudaError_t launch_measure_bits(Lattice& lat, int want_q, bool energy_only) {
   cudaError_t e = cudaMemsetAsync(lat.acc, 0, (size_t)lat.S * lat.slots * kAccStride * sizeof(int64_t), lat.stream);
   if (e != cudaSuccess) return e;
-  const bool p2 = lat.geom.lL > 0;
-  if (lat.D == 3)
-    return p2 ? measure_dispatch<3, true>(lat, want_q, energy_only)
-              : measure_dispatch<3, false>(lat, want_q, energy_only);
-  return p2 ? measure_dispatch<2, true>(lat, want_q, energy_only)
-            : measure_dispatch<2, false>(lat, want_q, energy_only);
+  return lat.D == 3 ? measure_dispatch<3>(lat, want_q, energy_only) : measure_dispatch<2>(lat, want_q, energy_only);
 }
 
 cudaError_t launch_get_spins_bits(Lattice& lat, int8_t* dev_out) {

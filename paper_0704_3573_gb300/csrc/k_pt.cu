@@ -93,10 +93,13 @@ __global__ void k_pt_swap(const int64_t* __restrict__ acc, int32_t* slot_at, int
 }
 
 // The same step with one warp per chain (K <= 32): thread j holds the slot
-// at temperature j, the temperature of slot j and the energy of slot j; the
-// random words of all pairs are drawn first, in parallel (they do not depend
-// on the permutation); the pairs then go in order, each decided by thread k
-// and broadcast.
+// at temperature j, the temperature of slot j and the energy of slot j.  What
+// does not depend on the permutation is done first, by all pairs at once: the
+// random words, and the largest energy difference that a pair's word accepts
+// (T_PT falls with m, so r < T_PT(m) iff m is at most the number of table
+// entries above r, found by bisection).  The pairs then go in order on
+// registers alone, each decided by thread k and broadcast; with the table read
+// inside that chain of K - 1 steps each step waited for a load.
 __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at, int32_t* temp_of,
                                uint64_t* accepted, const uint64_t* __restrict__ pttab,
                                const int8_t* __restrict__ pt_sign, uint32_t pt_len, int S, int R, int K, int slots,
@@ -115,19 +118,29 @@ __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at
     my_ta = ta[lane];
     my_E = config_energy(acc + ((size_t)s * slots + (size_t)lane * R + a) * kAccStride, mode, D, N);
   }
-  uint32_t my_r = 0;
+  uint32_t my_m = 0;  // pairs accept |d| = 4m up to this m
   int my_sg = 0;
   if (lane + 1 < K) {
     const uint32_t c2 = (TAG_PT << 28) | ((uint32_t)a << 16) | ((uint32_t)s >> 2);
     const uint4 x = philox10((uint32_t)lane, tau_lo, c2, tau_hi, keys);
     const uint32_t sel = (uint32_t)s & 3u;
-    my_r = sel == 0 ? x.x : sel == 1 ? x.y : sel == 2 ? x.z : x.w;
+    const uint32_t r = sel == 0 ? x.x : sel == 1 ? x.y : sel == 2 ? x.z : x.w;
     my_sg = pt_sign[lane];
+    const uint64_t* row = pttab + (size_t)lane * pt_len;
+    uint32_t hi = pt_len;  // entries above r: my_m .. hi
+    while (my_m < hi) {
+      const uint32_t mid = (my_m + hi) >> 1;
+      if ((uint64_t)r < __ldg(row + mid))
+        my_m = mid + 1u;
+      else
+        hi = mid;
+    }
   }
+  // energies travel with the permutation: thread j's is that of the slot at temperature j
+  long long E = __shfl_sync(0xffffffffu, my_E, my_sa);
   uint64_t my_acc = 0;
   for (int k = 0; k + 1 < K; ++k) {
-    const int A = __shfl_sync(0xffffffffu, my_sa, k), B = __shfl_sync(0xffffffffu, my_sa, k + 1);
-    const long long EA = __shfl_sync(0xffffffffu, my_E, A), EB = __shfl_sync(0xffffffffu, my_E, B);
+    const long long EA = __shfl_sync(0xffffffffu, E, k), EB = __shfl_sync(0xffffffffu, E, k + 1);
     int swap = 0;
     if (lane == k) {
       const long long d = EB - EA;
@@ -135,21 +148,23 @@ __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at
         swap = 1;
       } else {
         const unsigned long long ad = (unsigned long long)(d > 0 ? d : -d);
-        if (ad & 3ull) {
+        if (ad & 3ull)
           atomicOr(err, ERR_PT_PARITY);
-        } else {
-          const unsigned long long m = ad >> 2;
-          const uint64_t T = (m <= pt_len) ? __ldg(pttab + (size_t)k * pt_len + (m - 1)) : 0ull;
-          swap = (uint64_t)my_r < T ? 1 : 0;
-        }
+        else
+          swap = (ad >> 2) <= (unsigned long long)my_m ? 1 : 0;
       }
     }
     if (__shfl_sync(0xffffffffu, swap, k)) {
+      const int A = __shfl_sync(0xffffffffu, my_sa, k), B = __shfl_sync(0xffffffffu, my_sa, k + 1);
       if (lane == k) {
         my_sa = B;
+        E = EB;
         my_acc += 1;
       }
-      if (lane == k + 1) my_sa = A;
+      if (lane == k + 1) {
+        my_sa = A;
+        E = EA;
+      }
       if (lane == B) my_ta = k;
       if (lane == A) my_ta = k + 1;
     }
@@ -187,9 +202,9 @@ cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, ui
 
 cudaError_t launch_pt_swap(Lattice& lat) {
   const int total = lat.S * lat.R;
-  if (lat.K <= 32) {  // one warp per chain
-    const unsigned grid = (unsigned)((total + 7) / 8);
-    k_pt_swap_warp<<<grid, 256, 0, lat.stream>>>(
+  if (lat.K <= 32 && lat.pt_falls) {  // one warp per chain
+    const unsigned grid = (unsigned)((total + 3) / 4);
+    k_pt_swap_warp<<<grid, 128, 0, lat.stream>>>(
         lat.acc, lat.slot_at, lat.temp_of, lat.accepted, lat.pttab, lat.pt_sign, lat.pt_len, lat.S, lat.R, lat.K,
         lat.slots, lat.layout, lat.D, lat.N, (uint32_t)(lat.steps & 0xffffffffu), (uint32_t)(lat.steps >> 32),
         lat.keys, lat.err);

@@ -134,6 +134,7 @@ struct Lattice {
   uint64_t ser_first;   // first row still readable
   uint32_t pt_len;      // entries per PT pair table (<= pt_cap)
   uint32_t pt_cap;      // allocated entries per pair
+  bool pt_falls;        // every pair's table falls (bisection finds the entries above a number)
   uint64_t sweeps;      // absolute sweep counter
   uint64_t steps;       // PT swap steps done
   PhiloxKeys keys;

@@ -12,20 +12,6 @@ namespace potts {
 constexpr int kBlock = 256;
 constexpr uint32_t kOnes = 0x01010101u;
 
-// n / d for n < 2^31 by a multiplication (Granlund and Montgomery, PLDI'94).
-struct FastDiv {
-  uint32_t m, s, d;
-};
-
-inline FastDiv fast_div(uint32_t d) {
-  FastDiv f{0, 0, d};
-  while ((1ull << f.s) < d) ++f.s;
-  f.m = (uint32_t)(((((1ull << f.s) - d) << 32) / d) + 1u);
-  return f;
-}
-
-__device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) { return (__umulhi(n, f.m) + n) >> f.s; }
-
 // prmt.b32: byte i of the result is byte (sel >> 4i) & 7 of {b, a}, or, with
 // bit 3 of the selector nibble set, that byte's sign bit eight times
 // (__byte_perm clears those selector bits).
