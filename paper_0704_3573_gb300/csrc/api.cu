@@ -141,7 +141,7 @@ int plan(const ianus_config* c, Sizes& z) {
   z.off_sM = take((size_t)z.cap * SKR * z.mq * 8);
   z.off_sQ = take((size_t)z.cap * z.S * z.K * 8);
   z.off_err = take(8);
-  z.off_tdev = take(8);
+  z.off_tdev = take(16);
   // progress flags of the persistent one-temperature bit-sliced sweep
   z.off_flags = take(layout == IANUS_LAYOUT_BITS64 && !field && z.K == 1 ? (size_t)kMaxPersistBlocks * 4 : 0);
   z.total = o;
@@ -356,6 +356,7 @@ int record_row(Lattice* lat) {
                         lat->ser_Q + row * (size_t)lat->S * lat->K, lat->ser_sweep + row, 1);
   if (st) return st;
   lat->ser_count += 1;
+  lat->t_dev_valid = false;
   return IANUS_OK;
 }
 
@@ -401,19 +402,34 @@ int do_pt_swap(Lattice* lat) {
 
 void drop_graphs(Lattice* lat) {
   if (!lat->graphs) return;
-  for (auto& kv : *lat->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto& kv : *lat->graphs)
+    if (kv.second) cudaGraphExecDestroy(kv.second);
   lat->graphs->clear();
 }
 
+// One colour pass of the chain being captured.
+cudaError_t launch_pass(Lattice* lat, int colour, uint64_t t, int inv) {
+  if (lat->layout == IANUS_LAYOUT_I8) return launch_sweep_i8(*lat, colour, t, inv);
+  if (lat->layout == IANUS_LAYOUT_BITS64) return launch_sweep_bits(*lat, colour, t, inv);
+  return launch_sweep_potts(*lat, colour, t);
+}
+
 // Captures B sweeps (2B colour kernels reading the device sweep counter at
-// offsets 0..B-1) and the counter advance on a private stream.  A large
-// lattice is captured as up to four chains, each a part of its configurations
-// on a stream of its own: while one chain's pass drains and its next one
-// starts, the others' blocks keep the SMs busy (L=64, 256 x 2, heat bath: 20.0
-// -> 18.2 us per colour pass; random fields L=64, 256: 14.2 -> 12.3).
-int build_graph(Lattice* lat, int inv, uint32_t B, cudaGraphExec_t* out) {
+// offsets 0..B-1), or with cycles > 0 that many times B sweeps and a
+// measurement into the next series row, and the counters' advance on private
+// streams.  A large lattice is captured as up to four chains, each a part of
+// its configurations on a stream of its own: while one chain's pass drains and
+// its next one starts, the others' blocks keep the SMs busy (L=64, 256 x 2,
+// heat bath: 20.0 -> 18.2 us per colour pass; random fields L=64, 256: 14.2 ->
+// 12.3).  A bit-sliced chain's counts follow its sweeps without waiting for
+// the other chains (but for the overlap, which reads them all), and the
+// accumulators are cleared and turned into the series row on another stream
+// beside the next sweeps (L=20, 100 x 4 replicas, 100 sweeps with 10
+// measurements: 1344 -> 1204 us).
+int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, cudaGraphExec_t* out) {
+  const bool bits = lat->layout == IANUS_LAYOUT_BITS64;
   int chains = 1;
-  if (lat->layout == IANUS_LAYOUT_BITS64) {
+  if (bits) {
     prepare_sweep_bits(*lat, inv);  // compile before capturing
     chains = sweep_chains_bits(*lat, inv);
   } else if (lat->layout == IANUS_LAYOUT_U8X4) {
@@ -421,42 +437,80 @@ int build_graph(Lattice* lat, int inv, uint32_t B, cudaGraphExec_t* out) {
   } else {
     chains = sweep_chains_i8(*lat);
   }
+  const int side = cycles > 0 && bits ? kMaxChains : chains - 1;  // side streams in use
   if (!lat->cap_stream) CK(cudaStreamCreateWithFlags(&lat->cap_stream, cudaStreamNonBlocking));
-  for (int k = 0; k + 1 < chains; ++k)
-    if (!lat->side_streams[k]) CK(cudaStreamCreateWithFlags(&lat->side_streams[k], cudaStreamNonBlocking));
+  for (int k = 0; k < side; ++k)
+    if ((k + 1 < chains || k + 1 == kMaxChains) && !lat->side_streams[k])
+      CK(cudaStreamCreateWithFlags(&lat->side_streams[k], cudaStreamNonBlocking));
   cudaEvent_t ev = nullptr;
-  if (chains > 1) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-  cudaStream_t user = lat->stream;
+  CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  const cudaStream_t user = lat->stream, main = lat->cap_stream, aux = lat->side_streams[kMaxChains - 1];
+  const int want_q = lat->R >= 2;
   lat->capturing = true;
   lat->chains = chains;
   cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(lat->cap_stream, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess && chains > 1) {
-    e = cudaEventRecord(ev, lat->cap_stream);
-    for (int k = 0; e == cudaSuccess && k + 1 < chains; ++k) e = cudaStreamWaitEvent(lat->side_streams[k], ev, 0);
-  }
-  for (int k = 0; k < chains; ++k) {
+  cudaError_t e = cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal);
+  auto stream_of = [&](int k) { return k == 0 ? main : lat->side_streams[k - 1]; };
+  // `to` continues after what `from` holds now
+  auto after = [&](cudaStream_t to, cudaStream_t from) {
+    if (e == cudaSuccess) e = cudaEventRecord(ev, from);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
+  };
+  auto sweeps = [&](int k, uint32_t s0) {
     lat->chain = k;
-    lat->stream = k == 0 ? lat->cap_stream : lat->side_streams[k - 1];
-    for (uint32_t s = 0; e == cudaSuccess && s < B; ++s)
-      for (int c = 0; e == cudaSuccess && c < 2; ++c) {
-        if (lat->layout == IANUS_LAYOUT_I8)
-          e = launch_sweep_i8(*lat, c, s, inv);
-        else if (lat->layout == IANUS_LAYOUT_BITS64)
-          e = launch_sweep_bits(*lat, c, s, inv);
-        else
-          e = launch_sweep_potts(*lat, c, s);
+    lat->stream = stream_of(k);
+    for (uint32_t s = s0; e == cudaSuccess && s < s0 + B; ++s)
+      for (int c = 0; e == cudaSuccess && c < 2; ++c) e = launch_pass(lat, c, s, inv);
+  };
+  auto clear = [&]() {
+    if (e == cudaSuccess)
+      e = cudaMemsetAsync(lat->acc, 0, (size_t)lat->S * lat->slots * kAccStride * sizeof(int64_t), aux);
+  };
+  for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+  if (cycles == 0) {
+    for (int k = 0; k < chains; ++k) sweeps(k, 0);
+    for (int k = 1; k < chains; ++k) after(main, stream_of(k));
+  } else if (bits) {
+    after(aux, main);
+    clear();
+    for (uint32_t n = 0; n < cycles; ++n) {
+      for (int k = 0; k < chains; ++k) {
+        sweeps(k, n * B);
+        after(stream_of(k), aux);  // cleared accumulators
+        if (e == cudaSuccess) e = launch_measure_bits_counts(*lat, false);
       }
+      if (overlap_apart(*lat, want_q)) {
+        for (int k = 1; k < chains; ++k) after(main, stream_of(k));
+        lat->stream = main;
+        if (e == cudaSuccess) e = launch_overlap_bits(*lat);
+        for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+      }
+      for (int k = 0; k < chains; ++k) after(aux, stream_of(k));
+      lat->stream = aux;
+      if (e == cudaSuccess) e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
+      if (n + 1 < cycles) clear();
+    }
+    for (int k = 1; k < chains; ++k) after(main, stream_of(k));
+    after(main, aux);
+  } else {
+    for (uint32_t n = 0; n < cycles; ++n) {
+      for (int k = 0; k < chains; ++k) sweeps(k, n * B);
+      for (int k = 1; k < chains; ++k) after(main, stream_of(k));
+      lat->stream = main;
+      lat->chain = lat->chains = 0;
+      if (e == cudaSuccess)
+        e = lat->layout == IANUS_LAYOUT_I8 ? launch_measure_i8(*lat, want_q) : launch_measure_potts(*lat, want_q);
+      lat->chains = chains;
+      if (n + 1 < cycles)
+        for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+      if (e == cudaSuccess) e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
+    }
   }
-  for (int k = 0; e == cudaSuccess && k + 1 < chains; ++k) {
-    e = cudaEventRecord(ev, lat->side_streams[k]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(lat->cap_stream, ev, 0);
-  }
-  lat->stream = lat->cap_stream;
+  lat->stream = main;
   lat->chain = lat->chains = 0;
-  if (e == cudaSuccess) e = launch_advance_tick(*lat, B);
-  cudaError_t e2 = cudaStreamEndCapture(lat->cap_stream, &g);
-  if (ev) cudaEventDestroy(ev);
+  if (e == cudaSuccess) e = launch_advance_tick(*lat, (uint64_t)B * std::max(cycles, 1u), cycles);
+  cudaError_t e2 = cudaStreamEndCapture(main, &g);
+  cudaEventDestroy(ev);
   lat->stream = user;
   lat->capturing = false;
   if (e != cudaSuccess || e2 != cudaSuccess || !g) {
@@ -517,15 +571,62 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
     auto it = lat->graphs->find(B);
     if (it == lat->graphs->end()) {
       cudaGraphExec_t ex = nullptr;
-      int st = build_graph(lat, inv, B, &ex);
+      int st = build_graph(lat, inv, B, 0, &ex);
       if (st) return st;
       it = lat->graphs->emplace(B, ex).first;
     }
-    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps));
+    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count));
     CK(cudaGraphLaunch(it->second, lat->stream));
     lat->sweeps += B;
     lat->t_dev_valid = true;  // the graph advanced the counter by B
     n -= B;
+  }
+  return IANUS_OK;
+}
+
+// Runs up to `left` measured cycles of B sweeps through a captured graph and
+// returns how many it ran (0: the caller goes on launch by launch).  Small
+// lattices take several cycles a graph.  A graph is captured when this call
+// replays it six times or more (a first pass should not wait for captures that
+// it hardly uses), or when an earlier call wanted it.
+constexpr uint32_t kCycleKey = 1u << 30, kCycleSweeps = 64, kCycleMost = 16;
+
+int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, uint32_t* ran) {
+  *ran = 0;
+  if (!lat->use_graphs || !lat->graphs || B > kCycleSweeps) return IANUS_OK;
+  if (lat->layout == IANUS_LAYOUT_BITS64 &&
+      (persistent_variant(*lat) ||
+       (B >= 2 && lat->use_resident && lat->variant == 0 && resident_bits_fits(*lat))))
+    return IANUS_OK;
+  // a graph's start costs about 6 us: hidden by 16 sweeps of a large lattice,
+  // by 64 of a small one (one measured sweep a graph: L=64, 58 samples 1.4 ms
+  // for 44 against 1.2 ms launched one by one)
+  const bool large = (uint64_t)lat->S * lat->slots * lat->N >= (1u << 22);
+  const uint32_t most = std::min(kCycleMost, std::max(1u, (large ? 16u : kCycleSweeps) / B));
+  uint32_t n = 1;
+  while (2u * n <= most && 2u * n <= left) n *= 2u;
+  for (; n > 0; n /= 2u) {
+    const uint32_t key = kCycleKey | B << 8 | n;
+    auto it = lat->graphs->find(key);
+    if (it == lat->graphs->end() && left < 6ull * n) {
+      lat->graphs->emplace(key, nullptr);  // wanted: built when it is asked for again
+      continue;
+    }
+    if (it == lat->graphs->end() || !it->second) {
+      cudaGraphExec_t ex = nullptr;
+      const int st = build_graph(lat, inv, B, n, &ex);
+      if (st) return st;
+      (*lat->graphs)[key] = ex;
+      it = lat->graphs->find(key);
+    }
+    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count));
+    CK(cudaGraphLaunch(it->second, lat->stream));
+    lat->sweeps += (uint64_t)B * n;
+    lat->ser_count += n;
+    lat->t_dev_valid = true;  // the graph advanced the counters
+    acc_fresh(lat);
+    *ran = n;
+    return IANUS_OK;
   }
   return IANUS_OK;
 }
@@ -736,6 +837,13 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
   }
   uint64_t left = nsweeps;
   while (left > 0) {
+    if (measure_every && lat->sweeps % measure_every == 0 && left >= measure_every) {
+      uint32_t ran = 0;
+      int st = cycles_graphed(lat, inv, measure_every, left / measure_every, &ran);
+      if (st) return (ianus_status)st;
+      left -= (uint64_t)ran * measure_every;
+      if (ran) continue;
+    }
     uint64_t chunk = left;  // sweeps up to the next measurement point
     if (measure_every) chunk = std::min<uint64_t>(chunk, measure_every - lat->sweeps % measure_every);
     int st = sweeps_graphed(lat, inv, chunk);

@@ -710,13 +710,13 @@ __device__ __forceinline__ void block_flush(long long (*red)[64], const long lon
 }
 
 // One temperature (slot = replica): U and B of every replica and, with two
-// replicas, X, in one pass.  Grid (chunks, groups).
+// replicas, X, in one pass.  Grid (chunks, groups), from group y0.
 template <int D, int R>
 __global__ void __launch_bounds__(kBlock, 2) k_measure_bits_k1(const uint64_t* __restrict__ spins,
                                                                const uint64_t* __restrict__ J, int64_t* acc,
-                                                               MeasGeom geom, int S) {
+                                                               MeasGeom geom, int S, int y0) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
-  const int g = blockIdx.y;
+  const int g = y0 + blockIdx.y;
   const uint32_t N = geom.N;
   const uint64_t* Jg = J + (size_t)g * D * N;
   const uint64_t* sg = spins + (size_t)g * R * N;
@@ -787,13 +787,13 @@ __global__ void __launch_bounds__(kBlock, 2) k_measure_bits_k1(const uint64_t* _
 }
 
 // Any number of temperatures: U and B of one slot.  Grid (chunks, groups x
-// slots).
+// slots), from row y0.
 template <int D, bool EONLY = false>
 __global__ void __launch_bounds__(kBlock) k_measure_bits(const uint64_t* __restrict__ spins,
                                                          const uint64_t* __restrict__ J, int64_t* acc, MeasGeom geom,
-                                                         int S, int slots) {
+                                                         int S, int slots, int y0) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
-  const int gt = blockIdx.y;  // g * slots + sigma
+  const int gt = y0 + blockIdx.y;  // g * slots + sigma
   const int g = gt / slots, sigma = gt - g * slots;
   const uint32_t N = geom.N;
   const uint64_t* Jg = J + (size_t)g * D * N;
@@ -841,9 +841,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_measure_field_bits(const uint64_t
                                                                   const uint64_t* __restrict__ J,
                                                                   const uint64_t* __restrict__ hbits,
                                                                   const uint64_t* __restrict__ xbits, int64_t* acc,
-                                                                  MeasGeom geom, int S, int slots) {
+                                                                  MeasGeom geom, int S, int slots, int y0) {
   __shared__ long long red[kMeasWarps * kMeasMaxQ][64];
-  const int gt = blockIdx.y;  // g * slots + sigma
+  const int gt = y0 + blockIdx.y;  // g * slots + sigma
   const int g = gt / slots, sigma = gt - g * slots;
   const uint32_t N = geom.N;
   const uint64_t* Jg = J + (size_t)g * D * N;
@@ -1649,48 +1649,63 @@ cudaError_t overlap_tile(Lattice& lat, const uint64_t* xbits) {
 }
 
 template <int D>
-cudaError_t measure_dispatch(Lattice& lat, int want_q, bool energy_only) {
+cudaError_t counts_dispatch(Lattice& lat, bool energy_only) {
   const uint64_t* sp = (const uint64_t*)lat.spins;
   const uint64_t* J = (const uint64_t*)lat.J;
   const MeasGeom geom{fast_div((uint32_t)lat.geom.h), fast_div((uint32_t)lat.geom.L), lat.N};
-  if (lat.K == 1 && (lat.R == 1 || lat.R == 2) && !lat.field) {
-    // one pass for E, M and (R == 2) Q
-    dim3 grid(meas_blocks(lat.N, (unsigned)lat.G), (unsigned)lat.G);
-    if (lat.R == 2)
-      k_measure_bits_k1<D, 2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S);
-    else
-      k_measure_bits_k1<D, 1><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S);
-    return cudaGetLastError();
+  const bool one = lat.K == 1 && (lat.R == 1 || lat.R == 2) && !lat.field;  // one pass for E, M and (R == 2) Q
+  const uint32_t rows = (uint32_t)(one ? lat.G : lat.G * lat.slots);
+  // the rows of this chain: a multiple of its sweep's block rows (launch_lt)
+  uint32_t y0 = 0, y1 = rows;
+  if (lat.chains > 1) {
+    const uint32_t sweep_rows = one || lat.field ? (uint32_t)lat.G : rows / (uint32_t)lanes_replicas(lat);
+    const uint32_t per = rows / sweep_rows, n = (uint32_t)lat.chains;
+    y0 = per * (sweep_rows * (uint32_t)lat.chain / n);
+    y1 = per * (sweep_rows * ((uint32_t)lat.chain + 1u) / n);
   }
-  dim3 grid(meas_blocks(lat.N, (unsigned)(lat.G * lat.slots)), (unsigned)(lat.G * lat.slots));
-  if (energy_only && !lat.field) {  // U of every configuration, for the PT swap
-    k_measure_bits<D, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots);
-    return cudaGetLastError();
-  }
-  if (lat.field && lat.dilute)
+  const dim3 grid(meas_blocks(lat.N, rows), y1 - y0);
+  const int y = (int)y0;
+  if (one && lat.R == 2)
+    k_measure_bits_k1<D, 2><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, y);
+  else if (one)
+    k_measure_bits_k1<D, 1><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, y);
+  else if (lat.field && lat.dilute)
     k_measure_field_bits<D, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.hbits, lat.xbits, lat.acc, geom, lat.S,
-                                                                   lat.slots);
+                                                                   lat.slots, y);
   else if (lat.field)
     k_measure_field_bits<D, false><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.hbits, lat.xbits, lat.acc, geom, lat.S,
-                                                                    lat.slots);
+                                                                    lat.slots, y);
+  else if (energy_only)  // U of every configuration, for the PT swap
+    k_measure_bits<D, true><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots, y);
   else
-    k_measure_bits<D><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots);
-  if (want_q && lat.R >= 2) {
-    const uint64_t* xb = lat.field ? lat.xbits : nullptr;
-    if (lat.K <= 16) return overlap_tile<4>(lat, xb);
-    if (lat.K <= 32) return overlap_tile<8>(lat, xb);
-    if (lat.K <= kOverlapTemps) return overlap_tile<kOverlapTemps / 4>(lat, xb);
-    dim3 gq(meas_blocks(lat.N, (unsigned)(lat.G * lat.K)), (unsigned)(lat.G * lat.K));
-    k_overlap_bits<<<gq, kBlock, 2 * lat.K * sizeof(uint64_t), lat.stream>>>(sp, lat.slot_at, xb, lat.acc, lat.N,
-                                                                             lat.S, lat.R, lat.K, lat.slots);
-  }
+    k_measure_bits<D><<<grid, kBlock, 0, lat.stream>>>(sp, J, lat.acc, geom, lat.S, lat.slots, y);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_measure_bits_counts(Lattice& lat, bool energy_only) {
+  return lat.D == 3 ? counts_dispatch<3>(lat, energy_only) : counts_dispatch<2>(lat, energy_only);
+}
+
+bool overlap_apart(const Lattice& lat, int want_q) {
+  return want_q && lat.R >= 2 && !(lat.K == 1 && lat.R == 2 && !lat.field);
+}
+
+cudaError_t launch_overlap_bits(Lattice& lat) {
+  const uint64_t* xb = lat.field ? lat.xbits : nullptr;
+  if (lat.K <= 16) return overlap_tile<4>(lat, xb);
+  if (lat.K <= 32) return overlap_tile<8>(lat, xb);
+  if (lat.K <= kOverlapTemps) return overlap_tile<kOverlapTemps / 4>(lat, xb);
+  dim3 gq(meas_blocks(lat.N, (unsigned)(lat.G * lat.K)), (unsigned)(lat.G * lat.K));
+  k_overlap_bits<<<gq, kBlock, 2 * lat.K * sizeof(uint64_t), lat.stream>>>(
+      (const uint64_t*)lat.spins, lat.slot_at, xb, lat.acc, lat.N, lat.S, lat.R, lat.K, lat.slots);
   return cudaGetLastError();
 }
 
 cudaError_t launch_measure_bits(Lattice& lat, int want_q, bool energy_only) {
   cudaError_t e = cudaMemsetAsync(lat.acc, 0, (size_t)lat.S * lat.slots * kAccStride * sizeof(int64_t), lat.stream);
-  if (e != cudaSuccess) return e;
-  return lat.D == 3 ? measure_dispatch<3>(lat, want_q, energy_only) : measure_dispatch<2>(lat, want_q, energy_only);
+  if (e == cudaSuccess) e = launch_measure_bits_counts(lat, energy_only);
+  if (e == cudaSuccess && !energy_only && overlap_apart(lat, want_q)) e = launch_overlap_bits(lat);
+  return e;
 }
 
 cudaError_t launch_get_spins_bits(Lattice& lat, int8_t* dev_out) {

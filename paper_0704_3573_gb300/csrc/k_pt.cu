@@ -15,9 +15,29 @@ __device__ __forceinline__ long long config_energy(const int64_t* row, int mode,
   return (long long)row[0];
 }
 
-__global__ void k_finalize(const int64_t* __restrict__ acc, const int32_t* __restrict__ slot_at, int64_t* E,
-                           int64_t* M, int64_t* Q, uint64_t* sweep_out, uint64_t sweep, int S, int R, int K,
-                           int slots, int mode, int D, uint32_t N, int want_q, int field) {
+// Where the outputs go: the given arrays, or (captured graphs, tick non-null)
+// the series row tick[1] + row_off of a ring of cap rows, its sweep tick[0] +
+// sweep.
+struct FinalizeOut {
+  int64_t *E, *M, *Q;
+  uint64_t* sweep_out;
+  uint64_t sweep;
+  const uint64_t* tick;
+  uint32_t row_off, cap;
+};
+
+__global__ void k_finalize(const int64_t* __restrict__ acc, const int32_t* __restrict__ slot_at, FinalizeOut o,
+                           int S, int R, int K, int slots, int mode, int D, uint32_t N, int want_q, int field,
+                           int mq) {
+  if (o.tick) {
+    const size_t row = (size_t)((o.tick[1] + o.row_off) % o.cap), SK = (size_t)S * K;
+    o.E += row * SK * R;
+    o.M += row * SK * R * mq;
+    o.Q += row * SK;
+    o.sweep_out += row;
+    o.sweep += o.tick[0];
+  }
+  int64_t *E = o.E, *M = o.M, *Q = o.Q;
   const int total = S * K * R;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
     const int a = idx % R, sk = idx / R;
@@ -42,7 +62,7 @@ __global__ void k_finalize(const int64_t* __restrict__ acc, const int32_t* __res
       Q[sk] = mode == IANUS_LAYOUT_BITS64 && !field ? (int64_t)N - 2 * x : x;
     }
   }
-  if (sweep_out && blockIdx.x == 0 && threadIdx.x == 0) *sweep_out = sweep;
+  if (o.sweep_out && blockIdx.x == 0 && threadIdx.x == 0) *o.sweep_out = o.sweep;
 }
 
 // One thread per chain (sample s, replica a): pairs k = 0..K-2 in order.
@@ -176,28 +196,43 @@ __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at
   if (lane + 1 < K && my_acc) accepted[(size_t)idx * (K - 1) + lane] += my_acc;
 }
 
-__global__ void k_set_tick(uint64_t* t, uint64_t v) { *t = v; }
-__global__ void k_advance_tick(uint64_t* t, uint64_t by) { *t += by; }
+// tick[0] = sweeps done, tick[1] = series rows recorded
+__global__ void k_set_tick(uint64_t* t, uint64_t sweeps, uint64_t rows) {
+  t[0] = sweeps;
+  t[1] = rows;
+}
+__global__ void k_advance_tick(uint64_t* t, uint64_t by, uint64_t rows) {
+  t[0] += by;
+  t[1] += rows;
+}
 
-}  // namespace
-
-cudaError_t launch_set_tick(Lattice& lat, uint64_t value) {
-  k_set_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, value);
+cudaError_t finalize_launch(Lattice& lat, const FinalizeOut& o, int want_q) {
+  const int total = lat.S * lat.K * lat.R;
+  const unsigned grid = (unsigned)std::min(152 * 4, (total + 255) / 256);
+  k_finalize<<<grid > 0 ? grid : 1, 256, 0, lat.stream>>>(lat.acc, lat.slot_at, o, lat.S, lat.R, lat.K, lat.slots,
+                                                         lat.layout, lat.D, lat.N, want_q, lat.field ? 1 : 0, lat.mq);
   return cudaGetLastError();
 }
 
-cudaError_t launch_advance_tick(Lattice& lat, uint64_t by) {
-  k_advance_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, by);
+}  // namespace
+
+cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows) {
+  k_set_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, sweeps, rows);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows) {
+  k_advance_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, by, rows);
   return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, uint64_t* sweep_out, int want_q) {
-  const int total = lat.S * lat.K * lat.R;
-  const unsigned grid = (unsigned)std::min(152 * 4, (total + 255) / 256);
-  k_finalize<<<grid > 0 ? grid : 1, 256, 0, lat.stream>>>(lat.acc, lat.slot_at, E, M, Q, sweep_out, lat.sweeps,
-                                                         lat.S, lat.R, lat.K, lat.slots, lat.layout, lat.D, lat.N,
-                                                         want_q, lat.field ? 1 : 0);
-  return cudaGetLastError();
+  return finalize_launch(lat, FinalizeOut{E, M, Q, sweep_out, lat.sweeps, nullptr, 0u, 1u}, want_q);
+}
+
+cudaError_t launch_finalize_row(Lattice& lat, uint32_t row_off, uint64_t sweep_off, int want_q) {
+  return finalize_launch(
+      lat, FinalizeOut{lat.ser_E, lat.ser_M, lat.ser_Q, lat.ser_sweep, sweep_off, lat.t_dev, row_off, lat.cap}, want_q);
 }
 
 cudaError_t launch_pt_swap(Lattice& lat) {

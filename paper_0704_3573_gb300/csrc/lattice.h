@@ -155,7 +155,7 @@ struct Lattice {
   uint32_t block_words;      // words per block of the bit-sliced sweep; 0 = heuristic
   // CUDA graphs of sweep blocks: the kernels of B sweeps and a counter
   // advance, captured once on a private stream and replayed on `stream`.
-  uint64_t* t_dev;           // device sweep counter read by captured kernels
+  uint64_t* t_dev;           // device counters of sweeps and series rows, read by captured kernels
   bool capturing;            // launchers pass t_dev (and an offset) while true
   bool use_graphs;
   bool use_resident;         // resident mode for small I8 lattices (default on)
@@ -166,11 +166,13 @@ struct Lattice {
   // acc_mut) when acc_ok; mut counts changes of the state other than sweeps.
   uint64_t mut, acc_sweeps, acc_mut;
   bool acc_ok;
-  bool t_dev_valid;          // *t_dev == sweeps
+  bool t_dev_valid;          // t_dev == {sweeps, ser_count}
   cudaStream_t cap_stream;
-  cudaStream_t side_streams[kMaxChains - 1];  // the other chains of a captured block
+  cudaStream_t side_streams[kMaxChains];  // the other chains of a captured block, then its accumulators' stream
   int chain, chains;         // while capturing a graph of several chains: the one launched now
-  std::map<uint32_t, cudaGraphExec_t>* graphs;  // by block length
+  // by block length (sweeps only), or kCycleKey | sweeps << 8 | cycles (a null
+  // entry: wanted once, not built yet)
+  std::map<uint32_t, cudaGraphExec_t>* graphs;
 };
 
 // ---- host table builders (tables.cpp) ----
@@ -283,6 +285,12 @@ cudaError_t launch_dependent(const void* k, dim3 grid, dim3 block, void** args, 
 size_t sweep_bits_smem(int R);  // least shared memory of the per-lane-plane sweep for R replicas
 // energy_only: U of every configuration only (the PT swap needs no more)
 cudaError_t launch_measure_bits(Lattice& lat, int want_q, bool energy_only = false);
+// Its parts: the counts of the chain being captured (all configurations
+// otherwise) into zeroed accumulators, and the overlap where another kernel
+// takes it (overlap_apart), which reads every configuration.
+cudaError_t launch_measure_bits_counts(Lattice& lat, bool energy_only);
+bool overlap_apart(const Lattice& lat, int want_q);
+cudaError_t launch_overlap_bits(Lattice& lat);
 cudaError_t launch_build_planes(Lattice& lat);  // tp from thr and temp_of
 cudaError_t launch_get_spins_bits(Lattice& lat, int8_t* dev_out);
 cudaError_t launch_set_spins_bits(Lattice& lat, const int8_t* dev_in);
@@ -359,8 +367,11 @@ static_assert(perm_rows_differ(2) && perm_rows_differ(3) && perm_rows_differ(4),
 // shared (k_pt.cu)
 cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, uint64_t* sweep_out, int want_q);
 cudaError_t launch_pt_swap(Lattice& lat);
-cudaError_t launch_set_tick(Lattice& lat, uint64_t value);
-cudaError_t launch_advance_tick(Lattice& lat, uint64_t by);
+// The same into the series row that the device counters name, row_off rows and
+// sweep_off sweeps further (captured graphs).
+cudaError_t launch_finalize_row(Lattice& lat, uint32_t row_off, uint64_t sweep_off, int want_q);
+cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows);
+cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows);
 // Independent chains a captured block of sweeps is split into (1 .. kMaxChains):
 // configurations that never meet: the lane-queue sweep's block rows, the
 // Potts sweep's quads and replicas, the plain bit-sliced tiles' groups.  Passes of fewer than kChainSites threads
