@@ -1166,10 +1166,15 @@ ianus_status ianus_segment_state(ianus_lattice* h, int32_t group, int32_t lane0,
   return IANUS_OK;
 }
 
-static int fused_sweep_once(Lattice* lat) {
-  CK(launch_sweep_fused(*lat, 0));
-  CK(launch_sweep_fused(*lat, 1));
-  CK(launch_advance_segments(*lat));
+// n sweeps of a pool's segments, whose counters advance at the end.  Inside a
+// capture nothing but the sweeps runs between them, so all but the first pass
+// stage their tables early.
+static int fused_sweeps(Lattice* lat, uint32_t n, bool captured) {
+  for (uint32_t k = 0; k < n; ++k) {
+    CK(launch_sweep_fused(*lat, 0, k, captured && k > 0));
+    CK(launch_sweep_fused(*lat, 1, k, captured));
+  }
+  CK(launch_advance_segments(*lat, n));
   return IANUS_OK;
 }
 
@@ -1184,10 +1189,8 @@ ianus_status ianus_sweep_segments(ianus_lattice* h, uint64_t nsweeps) {
     if (resident) {
       CK(launch_resident_fused(*lat, B));
     } else if (B < 4 || !lat->use_graphs || !lat->graphs) {
-      for (uint32_t k = 0; k < B; ++k) {
-        int st = fused_sweep_once(lat);
-        if (st) return (ianus_status)st;
-      }
+      const int st = fused_sweeps(lat, B, false);
+      if (st) return (ianus_status)st;
     } else {
       const uint32_t key = (1u << 31) | B;
       auto it = lat->graphs->find(key);
@@ -1198,7 +1201,7 @@ ianus_status ianus_sweep_segments(ianus_lattice* h, uint64_t nsweeps) {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(lat->cap_stream, cudaStreamCaptureModeThreadLocal);
         int st = IANUS_OK;
-        for (uint32_t k = 0; e == cudaSuccess && st == IANUS_OK && k < B; ++k) st = fused_sweep_once(lat);
+        if (e == cudaSuccess) st = fused_sweeps(lat, B, true);
         cudaError_t e2 = cudaStreamEndCapture(lat->cap_stream, &g);
         lat->stream = user;
         cudaGraphExec_t ex = nullptr;

@@ -316,49 +316,121 @@ __global__ void k_set_sites_bits(uint64_t* hbits, uint64_t* xbits, const int8_t*
 // ---- fused serving: several jobs in the lanes of one group ----
 //
 // One block per (word range, group).  The block stages the group's per-lane
-// threshold planes and its segment table.  Per plane pair, every segment
-// that still has undecided lanes draws one Philox block from its own stream
-// (key of the job's seed, counter of the job's sweep t, group 0, slot 0) and
-// contributes its bits 0..n-1 shifted to its lanes.  Heat-bath lanes flip on
-// "not less" (inv lanes), Metropolis lanes on "less"; lanes of no live
-// segment never flip.
-template <int D, bool P2>
-__global__ void __launch_bounds__(kBlock) k_sweep_fused(const BitsParams p, const Segment* __restrict__ segs,
-                                                        const uint32_t* __restrict__ nseg) {
-  __shared__ uint64_t tpa[kPlanes * kMaxClasses];
-  __shared__ uint64_t s_mask[kMaxSegs];
-  __shared__ uint32_t s_klo[kMaxSegs], s_khi[kMaxSegs];
-  __shared__ Tick s_t[kMaxSegs];
-  __shared__ uint32_t s_lane0[kMaxSegs], s_c2[kMaxSegs];
-  __shared__ int s_n;
-  __shared__ uint64_t s_live, s_inv;
-  const int g = blockIdx.y;
-  for (int k = threadIdx.x; k < kPlanes * kMaxClasses; k += kBlock)
-    tpa[k] = p.tp[(size_t)g * kPlanes * kMaxClasses + k];
-  if (threadIdx.x == 0) {
-    const uint32_t ns = min(nseg[g], (uint32_t)kMaxSegs);
+// threshold planes, its segment table and, per running segment and plane
+// pair, the part of Philox rounds 0 and 1 that its sites share
+// (plane_uniform).  Per plane pair every segment that still has undecided
+// lanes draws one Philox block from its own stream (key of the job's seed,
+// counter of the job's sweep) and contributes its bits 0..n-1 shifted to its
+// lanes.  Heat-bath lanes flip on "not less" (inv lanes), Metropolis lanes on
+// "less"; lanes of no live segment never flip.
+//
+// T neighbouring threads share a word: thread j of them draws pairs m + j of
+// all segments, the T pairs' random words then pass through shuffles and every
+// thread does the compare.  A word's blocks are otherwise a serial chain (four
+// pairs times its segments): with few words T = 4 is the faster, with many the
+// repeated compare costs more than it hides.  L=16, 4 groups, 9 jobs: 6.5 us
+// per colour pass and a launch per sweep to advance the counters -> 3.6 us.
+constexpr int kFusedBlock = 128;
+
+struct FusedParams {
+  BitsParams b;          // t_lo: sweeps since the segments' counters were advanced
+  const Segment* segs;
+  const uint32_t* nseg;
+  int early;             // the tables were last written before the previous kernel started
+};
+
+struct FusedShared {
+  uint64_t tpa[kPlanes * kMaxClasses];
+  uint4 u[kMaxSegs * 16];              // shared part of rounds 0 and 1 per (segment, pair)
+  uint64_t mask[kMaxSegs];
+  uint32_t klo[kMaxSegs], khi[kMaxSegs], lane0[kMaxSegs], thi[kMaxSegs];
+  uint64_t live, inv;
+  int n;
+};
+
+__device__ __forceinline__ void stage_fused(FusedShared& sh, const FusedParams& fp, int g) {
+  const BitsParams& p = fp.b;
+  for (int k = threadIdx.x; k < kPlanes * kMaxClasses; k += kFusedBlock)
+    sh.tpa[k] = p.tp[(size_t)g * kPlanes * kMaxClasses + k];
+  if (threadIdx.x < 32u) {  // one warp packs the running segments, two candidates a thread
+    const uint32_t lane = threadIdx.x, ns = min(fp.nseg[g], (uint32_t)kMaxSegs);
     uint64_t live = 0, inv = 0;
     int n = 0;
-    for (uint32_t j = 0; j < ns; ++j) {
-      const Segment sg = segs[(size_t)g * kMaxSegs + j];
-      if (sg.t >= sg.t_end || sg.mask == 0ull) continue;
-      s_mask[n] = sg.mask;
-      s_klo[n] = sg.key_lo;
-      s_khi[n] = sg.key_hi;
-      s_t[n] = Tick{(uint32_t)sg.t, (uint32_t)(sg.t >> 32)};
-      s_lane0[n] = sg.lane0;
-      s_c2[n] = (TAG_SPIN << 28) | sg.jgroup;  // slot 0, the job's own group
-      live |= sg.mask;
-      if (sg.inv) inv |= sg.mask;
-      ++n;
+    for (uint32_t j0 = 0; j0 < ns; j0 += 32u) {
+      const uint32_t j = j0 + lane;
+      Segment sg{};
+      if (j < ns) sg = fp.segs[(size_t)g * kMaxSegs + j];
+      const uint64_t t = sg.t + p.t_lo;
+      const bool run = j < ns && sg.mask != 0ull && t < sg.t_end;
+      const uint32_t bal = __ballot_sync(0xffffffffu, run);
+      if (run) {
+        const int i = n + __popc(bal & ((1u << lane) - 1u));
+        sh.mask[i] = sg.mask;
+        sh.klo[i] = sg.key_lo;
+        sh.khi[i] = sg.key_hi;
+        sh.lane0[i] = sg.lane0;
+        sh.thi[i] = (uint32_t)(t >> 32) ^ sg.key_hi;
+        // plane_uniform of every pair: counter word c2 = slot 0 of the job's own group
+#pragma unroll
+        for (uint32_t m = 0; m < 16u; ++m) {
+          const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((TAG_SPIN << 28) | (m << 24) | sg.jgroup);
+          const uint32_t c0 = (uint32_t)(p1 >> 32) ^ (uint32_t)t ^ sg.key_lo;
+          const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
+          sh.u[i * 16 + (int)m] = make_uint4((uint32_t)p1 ^ (sg.key_lo + 0x9E3779B9u),
+                                             (uint32_t)(p0 >> 32) ^ (sg.key_hi + 0xBB67AE85u), (uint32_t)p0, 0u);
+        }
+        live |= sg.mask;
+        if (sg.inv) inv |= sg.mask;
+      }
+      n += __popc(bal);
     }
-    s_n = n;
-    s_live = live;
-    s_inv = inv;
+    const uint32_t ll = __reduce_or_sync(0xffffffffu, (uint32_t)live);
+    const uint32_t lh = __reduce_or_sync(0xffffffffu, (uint32_t)(live >> 32));
+    const uint32_t il = __reduce_or_sync(0xffffffffu, (uint32_t)inv);
+    const uint32_t ih = __reduce_or_sync(0xffffffffu, (uint32_t)(inv >> 32));
+    if (lane == 0) {
+      sh.n = n;
+      sh.live = (uint64_t)ll | ((uint64_t)lh << 32);
+      sh.inv = (uint64_t)il | ((uint64_t)ih << 32);
+    }
   }
   __syncthreads();
-  const uint64_t live = s_live, inv = s_inv;
-  const int nsg = s_n;
+}
+
+// Segment i's Philox block of plane pair m for a site: rounds 0 and 1 from
+// their parts, rounds 2..9 with the job's bumped key.
+__device__ __forceinline__ uint4 fused_block(const FusedShared& sh, int i, uint32_t m, uint32_t site) {
+  const uint64_t q0 = (uint64_t)0xD2511F53u * site;
+  const uint64_t q1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(q0 >> 32) ^ sh.thi[i]);
+  const uint4 u = sh.u[i * 16 + (int)m];
+  uint32_t c0 = (uint32_t)(q1 >> 32) ^ u.x, c1 = (uint32_t)q1, c2 = u.y ^ (uint32_t)q0, c3 = u.z;
+  uint32_t k0 = sh.klo[i] + 2u * 0x9E3779B9u, k1 = sh.khi[i] + 2u * 0xBB67AE85u;
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
+    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
+    c1 = (uint32_t)p1;
+    c3 = (uint32_t)p0;
+    c0 = n0;
+    c2 = n2;
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+  }
+  return make_uint4(c0, c1, c2, c3);
+}
+
+template <int D, bool P2, int T>
+__global__ void __launch_bounds__(kFusedBlock) k_sweep_fused(const FusedParams fp) {
+  __shared__ FusedShared sh;
+  const BitsParams& p = fp.b;
+  const int g = blockIdx.y;
+  if (fp.early) stage_fused(sh, fp, g);
+  dependent_launch_entry();
+  if (!fp.early) stage_fused(sh, fp, g);
+  const uint64_t live = sh.live, inv = sh.inv;
+  const int nsg = sh.n;
   if (live == 0ull) return;
   const Geom geom = p.geom;
   const uint32_t N = geom.N;
@@ -366,8 +438,11 @@ __global__ void __launch_bounds__(kBlock) k_sweep_fused(const BitsParams p, cons
   uint64_t* sp = p.spins + (size_t)g * N;  // one slot per group
   const uint32_t w_begin = blockIdx.x * p.words_per_block;
   const uint32_t w_end = min(w_begin + p.words_per_block, geom.half);
-  for (uint32_t w = w_begin + threadIdx.x; w < w_end; w += kBlock) {
-    const Nbr n = split_neighbours_t<P2>(geom, p.colour, w);
+  const uint32_t sub = threadIdx.x % T, first = threadIdx.x & 31u & ~(uint32_t)(T - 1);
+  for (uint32_t base = w_begin; base < w_end; base += kFusedBlock / T) {  // uniform across the block
+    const uint32_t w = base + threadIdx.x / T;
+    const bool valid = w < w_end;
+    const Nbr n = split_neighbours_t<P2>(geom, p.colour, valid ? w : w_begin);
     const uint64_t b = sp[n.self];
     uint64_t e[2 * D];
     e[0] = b ^ sp[n.xp] ^ __ldg(Jg + n.self);
@@ -381,31 +456,32 @@ __global__ void __launch_bounds__(kBlock) k_sweep_fused(const BitsParams p, cons
     uint64_t u0, u1, u2;
     count_unsat<D>(e, u0, u1, u2);
     // a segment's lanes may hold either algorithm's planes: select over all classes
-    const uint64_t always = class_select<D, 1>(tpa + 32 * kMaxClasses, u0, u1, u2);
+    const uint64_t always = class_select<D, 1>(sh.tpa + 32 * kMaxClasses, u0, u1, u2);
     uint64_t lt = always;
-    uint64_t und = ~always & live;
+    uint64_t und = valid ? ~always & live : 0ull;
 #pragma unroll 1
-    for (uint32_t mm = 0; mm < 16u && und != 0ull; ++mm) {
+    for (uint32_t m0 = 0; m0 < 16u && __any_sync(0xffffffffu, und != 0ull); m0 += T) {
       uint64_t r0 = 0, r1 = 0;
 #pragma unroll 1
       for (int j = 0; j < nsg; ++j) {
-        const uint64_t mk = s_mask[j];
+        const uint64_t mk = sh.mask[j];
         if (!(und & mk)) continue;
-        const uint4 x = philox10_key(n.site, s_t[j].lo, s_c2[j] | (mm << 24), s_t[j].hi, s_klo[j], s_khi[j]);
-        const uint32_t sh = s_lane0[j];
-        r0 |= (((uint64_t)x.x | ((uint64_t)x.y << 32)) << sh) & mk;
-        r1 |= (((uint64_t)x.z | ((uint64_t)x.w << 32)) << sh) & mk;
+        const uint4 x = fused_block(sh, j, m0 + sub, n.site);
+        const uint32_t s = sh.lane0[j];
+        r0 |= (((uint64_t)x.x | ((uint64_t)x.y << 32)) << s) & mk;
+        r1 |= (((uint64_t)x.z | ((uint64_t)x.w << 32)) << s) & mk;
       }
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const uint64_t r = q == 0 ? r0 : r1;
-        const uint64_t tb = class_select<D, 1>(tpa + (2u * mm + (uint32_t)q) * kMaxClasses, u0, u1, u2);
+      for (int q = 0; q < 2 * T; ++q) {
+        uint64_t r = (q & 1) ? r1 : r0;
+        if (T > 1) r = __shfl_sync(0xffffffffu, (unsigned long long)r, (int)first + (q >> 1));
+        const uint64_t tb = class_select<D, 1>(sh.tpa + (2u * m0 + (uint32_t)q) * kMaxClasses, u0, u1, u2);
         lt |= und & ~r & tb;
         und &= ~(r ^ tb);
       }
     }
     const uint64_t flip = (lt ^ inv) & live;
-    if (flip) sp[n.self] = b ^ flip;
+    if (valid && sub == 0u && flip) sp[n.self] = b ^ flip;
   }
 }
 
@@ -429,13 +505,13 @@ __global__ void k_load_segment(uint64_t* spins, uint64_t* J, Geom geom, int g, u
   }
 }
 
-__global__ void k_advance_segments(Segment* segs, const uint32_t* nseg, int G) {
+__global__ void k_advance_segments(Segment* segs, const uint32_t* nseg, int G, uint32_t by) {
   const int total = G * kMaxSegs;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
     const int g = idx / kMaxSegs, j = idx - g * kMaxSegs;
     if ((uint32_t)j >= nseg[g]) continue;
     Segment& sg = segs[idx];
-    if (sg.mask != 0ull && sg.t < sg.t_end) sg.t += 1;
+    if (sg.mask != 0ull && sg.t < sg.t_end) sg.t = min(sg.t_end, sg.t + by);
   }
 }
 
@@ -1461,13 +1537,14 @@ cudaError_t launch_load_segment(Lattice& lat, int group, uint32_t lane0, uint32_
   return cudaGetLastError();
 }
 
-cudaError_t launch_advance_segments(Lattice& lat) {
-  k_advance_segments<<<grid_for((uint64_t)lat.G * kMaxSegs, 128), 128, 0, lat.stream>>>(lat.segs, lat.nseg, lat.G);
+cudaError_t launch_advance_segments(Lattice& lat, uint32_t by) {
+  k_advance_segments<<<grid_for((uint64_t)lat.G * kMaxSegs, 128), 128, 0, lat.stream>>>(lat.segs, lat.nseg, lat.G, by);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_fused(Lattice& lat, int colour) {
-  BitsParams p;
+cudaError_t launch_sweep_fused(Lattice& lat, int colour, uint32_t off, bool early) {
+  FusedParams fp{};
+  BitsParams& p = fp.b;
   p.spins = (uint64_t*)lat.spins;
   p.J = (const uint64_t*)lat.J;
   p.tp = lat.tp;
@@ -1477,29 +1554,30 @@ cudaError_t launch_sweep_fused(Lattice& lat, int colour) {
   p.K = 1;
   p.slots = 1;
   p.colour = colour;
-  p.t_lo = p.t_hi = 0;
+  p.t_lo = off;
   p.keys = lat.keys;
-  p.t_dev = nullptr;
+  fp.segs = lat.segs;
+  fp.nseg = lat.nseg;
+  fp.early = early ? 1 : 0;
+  // threads a word, by 50 sweeps of 9 to 16 jobs: 8192 words (3D L=16, 4 groups)
+  // 393 us with four threads, 444 with two, 496 with one; 32768 (2D L=128) 635,
+  // 503, 656; 65536 (3D L=32) 926, 927, 682
   const uint32_t half = lat.geom.half;
-  uint32_t target_blocks = (152u * 8u + (uint32_t)lat.G - 1) / (uint32_t)lat.G;
+  const uint64_t words = (uint64_t)half * (uint64_t)lat.G;
+  const uint32_t T = words <= 152u * 96u ? 4u : words <= 152u * 300u ? 2u : 1u;
+  const uint32_t unit = kFusedBlock / T;  // words a block takes at a time
+  const uint32_t target_blocks = (152u * 12u + (uint32_t)lat.G - 1) / (uint32_t)lat.G;
   uint32_t wpb = (half + target_blocks - 1) / target_blocks;
-  wpb = ((wpb + kBlock - 1) / kBlock) * kBlock;
-  if (wpb < (uint32_t)kBlock) wpb = kBlock;
-  p.words_per_block = wpb;
-  dim3 grid((half + wpb - 1) / wpb, (unsigned)lat.G);
+  p.words_per_block = wpb = std::max(unit, (wpb + unit - 1) / unit * unit);
+  const dim3 grid((half + wpb - 1) / wpb, (unsigned)lat.G);
   const bool p2 = lat.geom.lL > 0;
-  if (lat.D == 3) {
-    if (p2)
-      k_sweep_fused<3, true><<<grid, kBlock, 0, lat.stream>>>(p, lat.segs, lat.nseg);
-    else
-      k_sweep_fused<3, false><<<grid, kBlock, 0, lat.stream>>>(p, lat.segs, lat.nseg);
-  } else {
-    if (p2)
-      k_sweep_fused<2, true><<<grid, kBlock, 0, lat.stream>>>(p, lat.segs, lat.nseg);
-    else
-      k_sweep_fused<2, false><<<grid, kBlock, 0, lat.stream>>>(p, lat.segs, lat.nseg);
-  }
-  return cudaGetLastError();
+  const void* k[2][2][3] = {
+      {{(const void*)k_sweep_fused<2, false, 1>, (const void*)k_sweep_fused<2, false, 2>, (const void*)k_sweep_fused<2, false, 4>},
+       {(const void*)k_sweep_fused<2, true, 1>, (const void*)k_sweep_fused<2, true, 2>, (const void*)k_sweep_fused<2, true, 4>}},
+      {{(const void*)k_sweep_fused<3, false, 1>, (const void*)k_sweep_fused<3, false, 2>, (const void*)k_sweep_fused<3, false, 4>},
+       {(const void*)k_sweep_fused<3, true, 1>, (const void*)k_sweep_fused<3, true, 2>, (const void*)k_sweep_fused<3, true, 4>}}};
+  void* args[] = {(void*)&fp};
+  return launch_dependent(k[lat.D - 2][p2 ? 1 : 0][T >> 1], grid, dim3(kFusedBlock), args, 0, lat.stream);
 }
 
 cudaError_t launch_build_field_planes(Lattice& lat) {

@@ -276,8 +276,10 @@ cudaError_t launch_build_field_planes(Lattice& lat);                 // ftp from
 // fused serving (k_msc.cu)
 cudaError_t launch_load_segment(Lattice& lat, int group, uint32_t lane0, uint32_t n, uint32_t jgroup,
                                 PhiloxKeys job_keys);
-cudaError_t launch_sweep_fused(Lattice& lat, int colour);
-cudaError_t launch_advance_segments(Lattice& lat);
+// Sweep `off` after the segments' counters; early: the tables were last
+// written before the previous kernel on the stream started.
+cudaError_t launch_sweep_fused(Lattice& lat, int colour, uint32_t off, bool early);
+cudaError_t launch_advance_segments(Lattice& lat, uint32_t by);
 cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv);
 // Launch with programmatic stream serialisation, for sweep kernels that
 // begin with dependent_launch_entry() (k_msc.cu)
