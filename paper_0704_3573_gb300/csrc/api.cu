@@ -141,7 +141,7 @@ int plan(const ianus_config* c, Sizes& z) {
   z.off_sM = take((size_t)z.cap * SKR * z.mq * 8);
   z.off_sQ = take((size_t)z.cap * z.S * z.K * 8);
   z.off_err = take(8);
-  z.off_tdev = take(16);
+  z.off_tdev = take(24);
   // progress flags of the persistent one-temperature bit-sliced sweep
   z.off_flags = take(layout == IANUS_LAYOUT_BITS64 && !field && z.K == 1 ? (size_t)kMaxPersistBlocks * 4 : 0);
   z.total = o;
@@ -394,6 +394,7 @@ int do_pt_swap(Lattice* lat) {
   }
   CK(launch_pt_swap(*lat));
   lat->steps += 1;
+  lat->t_dev_valid = false;
   if (lat->layout == IANUS_LAYOUT_BITS64) CK(launch_build_planes(*lat));
   return IANUS_OK;
 }
@@ -406,6 +407,24 @@ void drop_graphs(Lattice* lat) {
     if (kv.second) cudaGraphExecDestroy(kv.second);
   lat->graphs->clear();
 }
+
+// Resident sweep of a bit-sliced lattice for a run of n sweeps.
+enum class Resident { kNone, kBlock, kCluster };
+
+Resident resident_kind(Lattice* lat, uint64_t n) {
+  if (lat->layout != IANUS_LAYOUT_BITS64 || n < 2 || !lat->use_resident || lat->variant != 0) return Resident::kNone;
+  if (resident_cluster_bits(*lat)) return Resident::kCluster;
+  return resident_bits_fits(*lat) ? Resident::kBlock : Resident::kNone;
+}
+
+cudaError_t launch_resident(Lattice* lat, Resident kind, int inv, uint64_t t0, uint32_t n) {
+  return kind == Resident::kCluster ? launch_resident_cluster_bits(*lat, inv, t0, n)
+                                    : launch_resident_bits(*lat, inv, t0, n);
+}
+
+// What ends a captured cycle: a series row, a series row and a swap step, or a
+// swap step on energies measured for it alone.
+enum class Swap : uint32_t { kNone = 0, kMeasured = 1, kOnly = 2 };
 
 // One colour pass of the chain being captured.
 cudaError_t launch_pass(Lattice* lat, int colour, uint64_t t, int inv) {
@@ -425,11 +444,16 @@ cudaError_t launch_pass(Lattice* lat, int colour, uint64_t t, int inv) {
 // the other chains (but for the overlap, which reads them all), and the
 // accumulators are cleared and turned into the series row on another stream
 // beside the next sweeps (L=20, 100 x 4 replicas, 100 sweeps with 10
-// measurements: 1344 -> 1204 us).
-int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, cudaGraphExec_t* out) {
+// measurements: 1344 -> 1204 us).  With a swap each cycle ends in a
+// parallel-tempering step, which needs every energy; its cycles follow one
+// another.
+int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, Swap swap, cudaGraphExec_t* out) {
   const bool bits = lat->layout == IANUS_LAYOUT_BITS64;
+  const Resident kind = cycles > 0 ? resident_kind(lat, B) : Resident::kNone;
   int chains = 1;
-  if (bits) {
+  if (kind != Resident::kNone) {
+    chains = 1;
+  } else if (bits) {
     prepare_sweep_bits(*lat, inv);  // compile before capturing
     chains = sweep_chains_bits(*lat, inv);
   } else if (lat->layout == IANUS_LAYOUT_U8X4) {
@@ -459,6 +483,10 @@ int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, cudaGraphExe
   auto sweeps = [&](int k, uint32_t s0) {
     lat->chain = k;
     lat->stream = stream_of(k);
+    if (kind != Resident::kNone && e == cudaSuccess) {
+      e = launch_resident(lat, kind, inv, s0, B);
+      return;
+    }
     for (uint32_t s = s0; e == cudaSuccess && s < s0 + B; ++s)
       for (int c = 0; e == cudaSuccess && c < 2; ++c) e = launch_pass(lat, c, s, inv);
   };
@@ -477,7 +505,21 @@ int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, cudaGraphExe
       for (int k = 0; k < chains; ++k) {
         sweeps(k, n * B);
         after(stream_of(k), aux);  // cleared accumulators
-        if (e == cudaSuccess) e = launch_measure_bits_counts(*lat, false);
+        if (e == cudaSuccess) e = launch_measure_bits_counts(*lat, swap == Swap::kOnly);
+      }
+      if (swap != Swap::kNone) {
+        for (int k = 1; k < chains; ++k) after(main, stream_of(k));
+        lat->stream = main;
+        if (swap == Swap::kMeasured) {
+          if (e == cudaSuccess && overlap_apart(*lat, want_q)) e = launch_overlap_bits(*lat);
+          if (e == cudaSuccess) e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
+        }
+        if (e == cudaSuccess) e = launch_pt_swap(*lat, n);
+        if (e == cudaSuccess) e = launch_build_planes(*lat);
+        after(aux, main);
+        if (n + 1 < cycles) clear();
+        for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+        continue;
       }
       if (overlap_apart(*lat, want_q)) {
         for (int k = 1; k < chains; ++k) after(main, stream_of(k));
@@ -498,17 +540,22 @@ int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, cudaGraphExe
       for (int k = 1; k < chains; ++k) after(main, stream_of(k));
       lat->stream = main;
       lat->chain = lat->chains = 0;
+      const int q = swap == Swap::kOnly ? 0 : want_q;
       if (e == cudaSuccess)
-        e = lat->layout == IANUS_LAYOUT_I8 ? launch_measure_i8(*lat, want_q) : launch_measure_potts(*lat, want_q);
+        e = lat->layout == IANUS_LAYOUT_I8 ? launch_measure_i8(*lat, q) : launch_measure_potts(*lat, q);
       lat->chains = chains;
       if (n + 1 < cycles)
         for (int k = 1; k < chains; ++k) after(stream_of(k), main);
-      if (e == cudaSuccess) e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
+      if (e == cudaSuccess && swap != Swap::kOnly)
+        e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
+      if (e == cudaSuccess && swap != Swap::kNone) e = launch_pt_swap(*lat, n);
     }
   }
   lat->stream = main;
   lat->chain = lat->chains = 0;
-  if (e == cudaSuccess) e = launch_advance_tick(*lat, (uint64_t)B * std::max(cycles, 1u), cycles);
+  if (e == cudaSuccess)
+    e = launch_advance_tick(*lat, (uint64_t)B * std::max(cycles, 1u), swap == Swap::kOnly ? 0u : cycles,
+                            swap == Swap::kNone ? 0u : cycles);
   cudaError_t e2 = cudaStreamEndCapture(main, &g);
   cudaEventDestroy(ev);
   lat->stream = user;
@@ -532,10 +579,10 @@ constexpr uint32_t kResidentBlock = 4096;
 int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
   // small bit-sliced lattices under the automatic variant: resident sweeps,
   // many per launch, the lattice in shared memory
-  if (n >= 2 && lat->use_resident && lat->variant == 0 && resident_bits_fits(*lat)) {
+  if (const Resident kind = resident_kind(lat, n); kind != Resident::kNone) {
     while (n > 0) {
       const uint32_t B = (uint32_t)std::min<uint64_t>(n, kResidentBlock);
-      CK(launch_resident_bits(*lat, inv, lat->sweeps, B));
+      CK(launch_resident(lat, kind, inv, lat->sweeps, B));
       lat->sweeps += B;
       lat->t_dev_valid = false;
       n -= B;
@@ -571,11 +618,11 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
     auto it = lat->graphs->find(B);
     if (it == lat->graphs->end()) {
       cudaGraphExec_t ex = nullptr;
-      int st = build_graph(lat, inv, B, 0, &ex);
+      int st = build_graph(lat, inv, B, 0, Swap::kNone, &ex);
       if (st) return st;
       it = lat->graphs->emplace(B, ex).first;
     }
-    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count));
+    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count, lat->steps));
     CK(cudaGraphLaunch(it->second, lat->stream));
     lat->sweeps += B;
     lat->t_dev_valid = true;  // the graph advanced the counter by B
@@ -584,20 +631,17 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
   return IANUS_OK;
 }
 
-// Runs up to `left` measured cycles of B sweeps through a captured graph and
-// returns how many it ran (0: the caller goes on launch by launch).  Small
+// Runs up to `left` cycles of B sweeps through a captured graph and returns how
+// many it ran (0: the caller goes on launch by launch).  Small
 // lattices take several cycles a graph.  A graph is captured when this call
 // replays it six times or more (a first pass should not wait for captures that
 // it hardly uses), or when an earlier call wanted it.
 constexpr uint32_t kCycleKey = 1u << 30, kCycleSweeps = 64, kCycleMost = 16;
 
-int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, uint32_t* ran) {
+int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, Swap swap, uint32_t* ran) {
   *ran = 0;
   if (!lat->use_graphs || !lat->graphs || B > kCycleSweeps) return IANUS_OK;
-  if (lat->layout == IANUS_LAYOUT_BITS64 &&
-      (persistent_variant(*lat) ||
-       (B >= 2 && lat->use_resident && lat->variant == 0 && resident_bits_fits(*lat))))
-    return IANUS_OK;
+  if (lat->layout == IANUS_LAYOUT_BITS64 && persistent_variant(*lat)) return IANUS_OK;
   // a graph's start costs about 6 us: hidden by 16 sweeps of a large lattice,
   // by 64 of a small one (one measured sweep a graph: L=64, 58 samples 1.4 ms
   // for 44 against 1.2 ms launched one by one)
@@ -605,8 +649,8 @@ int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, uint32_t* r
   const uint32_t most = std::min(kCycleMost, std::max(1u, (large ? 16u : kCycleSweeps) / B));
   uint32_t n = 1;
   while (2u * n <= most && 2u * n <= left) n *= 2u;
-  for (; n > 0; n /= 2u) {
-    const uint32_t key = kCycleKey | B << 8 | n;
+  for (; n > 0 && n * B >= 4u; n /= 2u) {  // shorter ones: launch by launch
+    const uint32_t key = kCycleKey | (uint32_t)swap << 16 | B << 8 | n;
     auto it = lat->graphs->find(key);
     if (it == lat->graphs->end() && left < 6ull * n) {
       lat->graphs->emplace(key, nullptr);  // wanted: built when it is asked for again
@@ -614,15 +658,16 @@ int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, uint32_t* r
     }
     if (it == lat->graphs->end() || !it->second) {
       cudaGraphExec_t ex = nullptr;
-      const int st = build_graph(lat, inv, B, n, &ex);
+      const int st = build_graph(lat, inv, B, n, swap, &ex);
       if (st) return st;
       (*lat->graphs)[key] = ex;
       it = lat->graphs->find(key);
     }
-    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count));
+    if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count, lat->steps));
     CK(cudaGraphLaunch(it->second, lat->stream));
     lat->sweeps += (uint64_t)B * n;
-    lat->ser_count += n;
+    if (swap != Swap::kOnly) lat->ser_count += n;
+    if (swap != Swap::kNone) lat->steps += n;
     lat->t_dev_valid = true;  // the graph advanced the counters
     acc_fresh(lat);
     *ran = n;
@@ -839,7 +884,7 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
   while (left > 0) {
     if (measure_every && lat->sweeps % measure_every == 0 && left >= measure_every) {
       uint32_t ran = 0;
-      int st = cycles_graphed(lat, inv, measure_every, left / measure_every, &ran);
+      int st = cycles_graphed(lat, inv, measure_every, left / measure_every, Swap::kNone, &ran);
       if (st) return (ianus_status)st;
       left -= (uint64_t)ran * measure_every;
       if (ran) continue;
@@ -872,6 +917,19 @@ ianus_status ianus_sweep_pt(ianus_lattice* h, int32_t algo, const double* beta, 
   if (lat->K < 2) return IANUS_EINVAL;
   if (lat->model != IANUS_EA_PM_J || lat->field) return IANUS_EUNSUPPORTED;
   for (uint64_t n = 0; n < nsweeps; n += swap_every) {
+    // cycles that end in a measurement (or none) and a swap, once the first
+    // has checked the arguments and brought the tables up to date
+    if (n > 0 && swap_every <= kCycleSweeps &&
+        (measure_every == 0 || (measure_every == swap_every && lat->sweeps % swap_every == 0))) {
+      uint32_t ran = 0;
+      const int st = cycles_graphed(lat, algo == IANUS_HEATBATH, swap_every, (nsweeps - n) / swap_every,
+                                    measure_every ? Swap::kMeasured : Swap::kOnly, &ran);
+      if (st) return (ianus_status)st;
+      if (ran) {
+        n += (uint64_t)(ran - 1u) * swap_every;
+        continue;
+      }
+    }
     ianus_status st = ianus_sweep(h, algo, beta, swap_every, measure_every);
     if (st) return st;
     st = ianus_pt_swap(h);

@@ -65,14 +65,23 @@ __global__ void k_finalize(const int64_t* __restrict__ acc, const int32_t* __res
   if (o.sweep_out && blockIdx.x == 0 && threadIdx.x == 0) *o.sweep_out = o.sweep;
 }
 
+// The absolute swap step: the parameter, or in a captured graph the device
+// counter tick[2] plus the offset in it.
+__device__ __forceinline__ Tick swap_step(const Tick& tau, const uint64_t* tick) {
+  if (!tick) return tau;
+  const uint64_t t = tick[2] + tau.lo;
+  return Tick{(uint32_t)t, (uint32_t)(t >> 32)};
+}
+
 // One thread per chain (sample s, replica a): pairs k = 0..K-2 in order.
 // Swap iff db*d <= 0, else iff r < T_PT(|d|/4); d = E_B - E_A is a multiple
 // of 4 in the +-J model (checked: a violation sets ERR_PT_PARITY and rejects).
 __global__ void k_pt_swap(const int64_t* __restrict__ acc, int32_t* slot_at, int32_t* temp_of,
                           uint64_t* accepted, const uint64_t* __restrict__ pttab, const int8_t* __restrict__ pt_sign,
                           uint32_t pt_len, int S, int R, int K, int slots, int mode, int D, uint32_t N,
-                          uint32_t tau_lo, uint32_t tau_hi, PhiloxKeys keys, uint32_t* err) {
+                          Tick tau, const uint64_t* tick, PhiloxKeys keys, uint32_t* err) {
   const int total = S * R;
+  tau = swap_step(tau, tick);
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
     const int s = idx / R, a = idx - s * R;
     int32_t* sa = slot_at + (size_t)idx * K;
@@ -95,7 +104,7 @@ __global__ void k_pt_swap(const int64_t* __restrict__ acc, int32_t* slot_at, int
         } else {
           const unsigned long long m = ad >> 2;
           const uint64_t T = (m <= pt_len) ? pttab[(size_t)k * pt_len + (m - 1)] : 0ull;
-          const uint4 x = philox10((uint32_t)k, tau_lo, c2, tau_hi, keys);
+          const uint4 x = philox10((uint32_t)k, tau.lo, c2, tau.hi, keys);
           const uint32_t sel = (uint32_t)s & 3u;
           const uint32_t r = sel == 0 ? x.x : sel == 1 ? x.y : sel == 2 ? x.z : x.w;
           swap = (uint64_t)r < T;
@@ -123,11 +132,12 @@ __global__ void k_pt_swap(const int64_t* __restrict__ acc, int32_t* slot_at, int
 __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at, int32_t* temp_of,
                                uint64_t* accepted, const uint64_t* __restrict__ pttab,
                                const int8_t* __restrict__ pt_sign, uint32_t pt_len, int S, int R, int K, int slots,
-                               int mode, int D, uint32_t N, uint32_t tau_lo, uint32_t tau_hi, PhiloxKeys keys,
+                               int mode, int D, uint32_t N, Tick tau, const uint64_t* tick, PhiloxKeys keys,
                                uint32_t* err) {
   const int lane = (int)(threadIdx.x & 31u);
   const int idx = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // uniform across the warp
   if (idx >= S * R) return;
+  tau = swap_step(tau, tick);
   const int s = idx / R, a = idx - s * R;
   int32_t* sa = slot_at + (size_t)idx * K;
   int32_t* ta = temp_of + (size_t)idx * K;
@@ -142,7 +152,7 @@ __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at
   int my_sg = 0;
   if (lane + 1 < K) {
     const uint32_t c2 = (TAG_PT << 28) | ((uint32_t)a << 16) | ((uint32_t)s >> 2);
-    const uint4 x = philox10((uint32_t)lane, tau_lo, c2, tau_hi, keys);
+    const uint4 x = philox10((uint32_t)lane, tau.lo, c2, tau.hi, keys);
     const uint32_t sel = (uint32_t)s & 3u;
     const uint32_t r = sel == 0 ? x.x : sel == 1 ? x.y : sel == 2 ? x.z : x.w;
     my_sg = pt_sign[lane];
@@ -196,14 +206,16 @@ __global__ void k_pt_swap_warp(const int64_t* __restrict__ acc, int32_t* slot_at
   if (lane + 1 < K && my_acc) accepted[(size_t)idx * (K - 1) + lane] += my_acc;
 }
 
-// tick[0] = sweeps done, tick[1] = series rows recorded
-__global__ void k_set_tick(uint64_t* t, uint64_t sweeps, uint64_t rows) {
+// tick: sweeps done, series rows recorded, swap steps done
+__global__ void k_set_tick(uint64_t* t, uint64_t sweeps, uint64_t rows, uint64_t steps) {
   t[0] = sweeps;
   t[1] = rows;
+  t[2] = steps;
 }
-__global__ void k_advance_tick(uint64_t* t, uint64_t by, uint64_t rows) {
+__global__ void k_advance_tick(uint64_t* t, uint64_t by, uint64_t rows, uint64_t steps) {
   t[0] += by;
   t[1] += rows;
+  t[2] += steps;
 }
 
 cudaError_t finalize_launch(Lattice& lat, const FinalizeOut& o, int want_q) {
@@ -216,13 +228,13 @@ cudaError_t finalize_launch(Lattice& lat, const FinalizeOut& o, int want_q) {
 
 }  // namespace
 
-cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows) {
-  k_set_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, sweeps, rows);
+cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows, uint64_t steps) {
+  k_set_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, sweeps, rows, steps);
   return cudaGetLastError();
 }
 
-cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows) {
-  k_advance_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, by, rows);
+cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows, uint64_t steps) {
+  k_advance_tick<<<1, 1, 0, lat.stream>>>(lat.t_dev, by, rows, steps);
   return cudaGetLastError();
 }
 
@@ -235,21 +247,22 @@ cudaError_t launch_finalize_row(Lattice& lat, uint32_t row_off, uint64_t sweep_o
       lat, FinalizeOut{lat.ser_E, lat.ser_M, lat.ser_Q, lat.ser_sweep, sweep_off, lat.t_dev, row_off, lat.cap}, want_q);
 }
 
-cudaError_t launch_pt_swap(Lattice& lat) {
+cudaError_t launch_pt_swap(Lattice& lat, uint32_t off) {
   const int total = lat.S * lat.R;
+  // while capturing: the device's step counter plus the cycle's offset
+  const uint64_t* tick = lat.capturing ? lat.t_dev : nullptr;
+  const Tick tau = tick ? Tick{off, 0u} : Tick{(uint32_t)lat.steps, (uint32_t)(lat.steps >> 32)};
   if (lat.K <= 32 && lat.pt_falls) {  // one warp per chain
     const unsigned grid = (unsigned)((total + 3) / 4);
-    k_pt_swap_warp<<<grid, 128, 0, lat.stream>>>(
-        lat.acc, lat.slot_at, lat.temp_of, lat.accepted, lat.pttab, lat.pt_sign, lat.pt_len, lat.S, lat.R, lat.K,
-        lat.slots, lat.layout, lat.D, lat.N, (uint32_t)(lat.steps & 0xffffffffu), (uint32_t)(lat.steps >> 32),
-        lat.keys, lat.err);
+    k_pt_swap_warp<<<grid, 128, 0, lat.stream>>>(lat.acc, lat.slot_at, lat.temp_of, lat.accepted, lat.pttab,
+                                                 lat.pt_sign, lat.pt_len, lat.S, lat.R, lat.K, lat.slots, lat.layout,
+                                                 lat.D, lat.N, tau, tick, lat.keys, lat.err);
     return cudaGetLastError();
   }
   const unsigned grid = (unsigned)((total + 127) / 128);
   k_pt_swap<<<grid, 128, 0, lat.stream>>>(lat.acc, lat.slot_at, lat.temp_of, lat.accepted, lat.pttab, lat.pt_sign,
-                                          lat.pt_len, lat.S, lat.R, lat.K, lat.slots, lat.layout, lat.D, lat.N,
-                                          (uint32_t)(lat.steps & 0xffffffffu), (uint32_t)(lat.steps >> 32), lat.keys,
-                                          lat.err);
+                                          lat.pt_len, lat.S, lat.R, lat.K, lat.slots, lat.layout, lat.D, lat.N, tau,
+                                          tick, lat.keys, lat.err);
   return cudaGetLastError();
 }
 

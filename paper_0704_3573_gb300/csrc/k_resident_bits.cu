@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident_bits(const BitsPara
   for (uint32_t i = threadIdx.x; i < (uint32_t)D * N; i += blockDim.x) s_J[i] = __ldg(g_J + i);
   for (uint32_t i = threadIdx.x; i < R * kPlanes * kMaxClasses; i += blockDim.x) s_tp[i] = g_tp[i];
   __syncthreads();
-  const uint64_t t0 = ((uint64_t)p.t_hi << 32) | p.t_lo;
+  const Tick first = sweep_tick(p.t_lo, p.t_hi, p.t_dev);
+  const uint64_t t0 = ((uint64_t)first.hi << 32) | first.lo;
 #pragma unroll 1
   for (uint32_t s = 0; s < nsweeps; ++s) {
     const uint64_t t = t0 + s;
@@ -239,7 +240,7 @@ size_t resident_fused_smem(const Lattice& lat) {
 }
 
 BitsParams resident_params(const Lattice& lat, uint64_t t0) {
-  BitsParams p;
+  BitsParams p{};
   p.spins = (uint64_t*)lat.spins;
   p.J = (const uint64_t*)lat.J;
   p.tp = lat.tp;
@@ -253,7 +254,7 @@ BitsParams resident_params(const Lattice& lat, uint64_t t0) {
   p.t_hi = (uint32_t)(t0 >> 32);
   p.words_per_block = 0;
   p.keys = lat.keys;
-  p.t_dev = nullptr;
+  p.t_dev = lat.capturing ? lat.t_dev : nullptr;
   return p;
 }
 

@@ -155,23 +155,25 @@ struct Lattice {
   uint32_t block_words;      // words per block of the bit-sliced sweep; 0 = heuristic
   // CUDA graphs of sweep blocks: the kernels of B sweeps and a counter
   // advance, captured once on a private stream and replayed on `stream`.
-  uint64_t* t_dev;           // device counters of sweeps and series rows, read by captured kernels
+  uint64_t* t_dev;           // device counters of sweeps, series rows and swap steps, read by captured kernels
   bool capturing;            // launchers pass t_dev (and an offset) while true
   bool use_graphs;
   bool use_resident;         // resident mode for small I8 lattices (default on)
   int cluster_size;          // blocks per configuration of the resident plain sweep (when cluster_known)
   bool cluster_known;
+  uint32_t bits_cluster;     // the same of the bit-sliced cluster sweep
+  int bits_cluster_mode;     // the resident mode it was chosen for (0: not yet)
   int resident_mode;         // 1 = clusters when few configurations, 2 = one block each, 3 = clusters
   // The accumulators hold the measurement of the state at (acc_sweeps,
   // acc_mut) when acc_ok; mut counts changes of the state other than sweeps.
   uint64_t mut, acc_sweeps, acc_mut;
   bool acc_ok;
-  bool t_dev_valid;          // t_dev == {sweeps, ser_count}
+  bool t_dev_valid;          // t_dev == {sweeps, ser_count, steps}
   cudaStream_t cap_stream;
   cudaStream_t side_streams[kMaxChains];  // the other chains of a captured block, then its accumulators' stream
   int chain, chains;         // while capturing a graph of several chains: the one launched now
-  // by block length (sweeps only), or kCycleKey | sweeps << 8 | cycles (a null
-  // entry: wanted once, not built yet)
+  // by block length (sweeps only), or kCycleKey | swap << 16 | sweeps << 8 | cycles
+  // (a null entry: wanted once, not built yet)
   std::map<uint32_t, cudaGraphExec_t>* graphs;
 };
 
@@ -262,6 +264,11 @@ bool resident_fused_fits(const Lattice& lat);
 cudaError_t launch_resident_bits(Lattice& lat, int inv, uint64_t t0, uint32_t nsweeps);
 // nsweeps sweeps of a pool, each advancing its running segments by one.
 cudaError_t launch_resident_fused(Lattice& lat, uint32_t nsweeps);
+// The same split over a cluster (k_resident_cluster.cu): blocks per cluster
+// where it can run and is the faster one (resident_mode 3: wherever it can
+// run), 0 otherwise.
+uint32_t resident_cluster_bits(Lattice& lat);
+cudaError_t launch_resident_cluster_bits(Lattice& lat, int inv, uint64_t t0, uint32_t nsweeps);
 cudaError_t launch_resident_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t measure_every);
 cudaError_t launch_get_spins_i8(Lattice& lat, int8_t* dev_out);       // [S][slots][N]
 cudaError_t launch_set_spins_i8(Lattice& lat, const int8_t* dev_in);
@@ -368,12 +375,12 @@ static_assert(perm_rows_differ(2) && perm_rows_differ(3) && perm_rows_differ(4),
               "two reachable counts share a table row");
 // shared (k_pt.cu)
 cudaError_t launch_finalize(Lattice& lat, int64_t* E, int64_t* M, int64_t* Q, uint64_t* sweep_out, int want_q);
-cudaError_t launch_pt_swap(Lattice& lat);
+cudaError_t launch_pt_swap(Lattice& lat, uint32_t off = 0);  // off: steps after the counter, while capturing
 // The same into the series row that the device counters name, row_off rows and
 // sweep_off sweeps further (captured graphs).
 cudaError_t launch_finalize_row(Lattice& lat, uint32_t row_off, uint64_t sweep_off, int want_q);
-cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows);
-cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows);
+cudaError_t launch_set_tick(Lattice& lat, uint64_t sweeps, uint64_t rows, uint64_t steps);
+cudaError_t launch_advance_tick(Lattice& lat, uint64_t by, uint64_t rows, uint64_t steps);
 // Independent chains a captured block of sweeps is split into (1 .. kMaxChains):
 // configurations that never meet: the lane-queue sweep's block rows, the
 // Potts sweep's quads and replicas, the plain bit-sliced tiles' groups.  Passes of fewer than kChainSites threads

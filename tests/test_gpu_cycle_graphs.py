@@ -45,3 +45,24 @@ def test_measured_blocks_equal_launches(ianus, kw):
     assert np.array_equal(a.spins(), b.spins())
     if a.K > 1:
         assert all(np.array_equal(x, y) for x, y in zip(a.pt_state()[:2], b.pt_state()[:2]))
+
+
+@pytest.mark.parametrize("layout", ["bits64", "i8"])
+@pytest.mark.parametrize("L,S,R,K,every", [(6, 5, 2, 4, 1), (8, 70, 1, 3, 2), (32, 70, 2, 4, 5), (12, 3, 3, 33, 3)])
+def test_tempering_blocks_equal_calls(ianus, L, S, R, K, every, layout):
+    if layout == "i8" and S * L > 1000:
+        S = 3
+    beta = [1.3 - 0.9 * k / K for k in range(K)]
+    a, b = (ianus.Lattice(dim=3, L=L, n_samples=S, n_replicas=R, n_temps=K, seed=SEED, layout=layout,
+                          series_capacity=60) for _ in range(2))
+    b.set_graphs(False)
+    for n, m in ((8, every), (24, every), (24, every), (24, 0), (24, 0), (7, 1), (24, every)):
+        a.sweep_pt("metropolis", beta, n * every, every, m)
+        for _ in range(n):
+            b.sweep("metropolis", beta, every, m)
+            b.pt_swap()
+    for x, y in zip(a.series(), b.series()):
+        assert (x is None) == (y is None) and (x is None or np.array_equal(x, y))
+    assert np.array_equal(a.spins(), b.spins())
+    assert all(np.array_equal(x, y) for x, y in zip(a.pt_state()[:2], b.pt_state()[:2]))
+    assert a.pt_state()[2] == b.pt_state()[2]
