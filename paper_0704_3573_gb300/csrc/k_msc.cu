@@ -1454,11 +1454,18 @@ cudaKernel_t specialised_sweep_kernel(const Lattice& lat, const UniformLut& u, i
   return jit_kernel(lat, u, algo, js.mode, js.phase_a, js.min_blocks, js.group, js.jreload, js.ufirst, js.block);
 }
 
+// Whether random fields are swept by the kernel specialised at run time:
+// variants 0 (large lattices) and 2..; else by the precompiled ones.
+bool field_specialised(const Lattice& lat) {
+  return lat.flut_ok && lat.variant != 1 &&
+         (lat.variant != 0 || (uint64_t)lat.G * lat.slots * lat.N >= (1ull << 20));
+}
+
 void prepare_sweep_bits(Lattice& lat, int inv) {
   const int algo = inv ? 1 : 0;
   if (lat.field) {
     const bool lq = lane_queue(lat);
-    if (lat.flut_ok && lat.variant != 1 && (lat.jitf_algo != algo || lat.jitf_lq != lq)) {
+    if (field_specialised(lat) && (lat.jitf_algo != algo || lat.jitf_lq != lq)) {
       lat.jitf = lq ? jit_lt_field_kernel(lat, algo, field_blocks(lat), kLtBlock)
                     : jit_field_kernel(lat, algo, lat.dilute && lat.R == 2 ? 2 : 3);
       lat.jitf_algo = algo;
@@ -1488,7 +1495,7 @@ int sweep_chains_bits(const Lattice& lat, int inv) {
   if (!lane_queue(lat)) return 1;
   uint64_t rows;
   if (lat.field) {
-    if (!lat.jitf) return 1;
+    if (!field_specialised(lat) || !lat.jitf) return 1;
     rows = (uint64_t)lat.G;
   } else {
     const int v = jit_variant_for(lat);
@@ -1650,10 +1657,8 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
   const int algo = inv ? 1 : 0;
   if (lat.field) {
     // one temperature: the field kernel specialised at run time for the
-    // lattice's tables (variants 0 (large lattices) and 2..); else per-lane planes
-    const uint64_t words = (uint64_t)lat.G * lat.slots * lat.N;
-    const bool want_jit = lat.flut_ok && lat.variant != 1 && (lat.variant != 0 || words >= (1ull << 20));
-    if (want_jit) {
+    // lattice's tables; else per-lane planes
+    if (field_specialised(lat)) {
       prepare_sweep_bits(lat, inv);
       if (lat.jitf && lane_queue(lat)) return launch_lt(lat, lat.jitf, p, (uint32_t)lat.G, field_blocks(lat), kLtBlock);
       if (lat.jitf) {

@@ -19,6 +19,7 @@ LATTICES = [dict(dim=3, L=10, n_samples=70, n_replicas=2),
             dict(model="potts_perm", dim=2, L=8, n_samples=5, n_replicas=3),
             # several chains
             dict(dim=3, L=40, n_samples=130, n_replicas=2),
+            dict(dim=3, L=30, n_samples=156, n_replicas=1, disorder="daff", field=0.6, occupation=0.7),
             dict(dim=3, L=32, n_samples=64, n_replicas=3, n_temps=3),
             dict(dim=3, L=32, n_samples=130, n_replicas=1, layout="i8"),
             dict(model="potts", dim=3, L=24, n_samples=40, n_replicas=2)]
