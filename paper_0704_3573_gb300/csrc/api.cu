@@ -404,7 +404,7 @@ int do_pt_swap(Lattice* lat) {
 void drop_graphs(Lattice* lat) {
   if (!lat->graphs) return;
   for (auto& kv : *lat->graphs)
-    if (kv.second) cudaGraphExecDestroy(kv.second);
+    if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   lat->graphs->clear();
 }
 
@@ -570,13 +570,37 @@ int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, Swap swap, c
   return e == cudaSuccess ? IANUS_OK : fail(lat, IANUS_ECUDA);
 }
 
-// Runs n sweeps (no measurement inside) through cached graphs of blocks of
-// up to 64 sweeps; short runs (< 4 sweeps) launch eagerly.
+// Lattices whose passes take longer than their launches.
+bool large_lattice(const Lattice& lat) { return (uint64_t)lat.S * lat.slots * lat.N >= (1u << 22); }
+
+// The slot of `key` when its graph exists or should be captured now, null when
+// the caller should launch its kernels one by one; `uses`: times that the rest
+// of this call would replay it.  Capturing costs about 3 us a node, as much as
+// the launches, so a call launches what it asks for first, and a graph is
+// captured when an earlier call asked for it or this one still replays it three
+// times; two times where the first block of a large lattice keeps the GPU busy
+// meanwhile.  First calls on a new state, against capturing at once: 154 x 154,
+// 253 samples x 2, 99 sweeps 2226 -> 1148 us; L=20, 73 samples, 53 sweeps with
+// 26 measurements 927 -> 646; three-dimensional Potts L=78 1508 -> 472.
+GraphSlot* graph_slot(Lattice* lat, uint32_t key, uint64_t uses) {
+  GraphSlot& s = (*lat->graphs)[key];  // {null, 0} when new
+  if (s.exec) return &s;
+  const bool large = large_lattice(*lat);
+  if (s.asked == lat->calls) return uses >= (large ? 2u : 3u) ? &s : nullptr;
+  if (s.asked != 0 && (!large || uses < 3)) return &s;
+  s.asked = lat->calls;
+  return nullptr;
+}
+
 // Sweeps per launch of the resident bit-sliced sweep: long enough that the
 // launch costs nothing, short enough that no launch runs for long.
 constexpr uint32_t kResidentBlock = 4096;
 
-int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
+// Runs n sweeps (no measurement inside) through cached graphs of blocks of up
+// to 64 sweeps, 16 of a large lattice (whose chains have as many nodes and whose
+// graph starts are hidden); runs of less than 4 launch by launch.  The call has
+// `reps` such runs left.
+int sweeps_graphed(Lattice* lat, int inv, uint64_t n, uint64_t reps) {
   // small bit-sliced lattices under the automatic variant: resident sweeps,
   // many per launch, the lattice in shared memory
   if (const Resident kind = resident_kind(lat, n); kind != Resident::kNone) {
@@ -604,9 +628,12 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
     }
     if (n == 0) return IANUS_OK;
   }
+  const uint32_t most = large_lattice(*lat) ? 16u : 64u;
   while (n > 0) {
-    const uint32_t B = (uint32_t)std::min<uint64_t>(n, 64);
-    if (B < 4 || !lat->use_graphs || !lat->graphs) {
+    const uint32_t B = (uint32_t)std::min<uint64_t>(n, most);
+    GraphSlot* slot = nullptr;
+    if (B >= 4 && lat->use_graphs && lat->graphs) slot = graph_slot(lat, B, n / B * reps);
+    if (!slot) {
       for (uint32_t s = 0; s < B; ++s) {
         int st = one_sweep(lat, inv);
         if (st) return st;
@@ -615,15 +642,12 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
       n -= B;
       continue;
     }
-    auto it = lat->graphs->find(B);
-    if (it == lat->graphs->end()) {
-      cudaGraphExec_t ex = nullptr;
-      int st = build_graph(lat, inv, B, 0, Swap::kNone, &ex);
+    if (!slot->exec) {
+      const int st = build_graph(lat, inv, B, 0, Swap::kNone, &slot->exec);
       if (st) return st;
-      it = lat->graphs->emplace(B, ex).first;
     }
     if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count, lat->steps));
-    CK(cudaGraphLaunch(it->second, lat->stream));
+    CK(cudaGraphLaunch(slot->exec, lat->stream));
     lat->sweeps += B;
     lat->t_dev_valid = true;  // the graph advanced the counter by B
     n -= B;
@@ -632,10 +656,8 @@ int sweeps_graphed(Lattice* lat, int inv, uint64_t n) {
 }
 
 // Runs up to `left` cycles of B sweeps through a captured graph and returns how
-// many it ran (0: the caller goes on launch by launch).  Small
-// lattices take several cycles a graph.  A graph is captured when this call
-// replays it six times or more (a first pass should not wait for captures that
-// it hardly uses), or when an earlier call wanted it.
+// many it ran (0: the caller goes on launch by launch).  Small lattices take
+// several cycles a graph.
 constexpr uint32_t kCycleKey = 1u << 30, kCycleSweeps = 64, kCycleMost = 16;
 
 int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, Swap swap, uint32_t* ran) {
@@ -645,26 +667,19 @@ int cycles_graphed(Lattice* lat, int inv, uint32_t B, uint64_t left, Swap swap, 
   // a graph's start costs about 6 us: hidden by 16 sweeps of a large lattice,
   // by 64 of a small one (one measured sweep a graph: L=64, 58 samples 1.4 ms
   // for 44 against 1.2 ms launched one by one)
-  const bool large = (uint64_t)lat->S * lat->slots * lat->N >= (1u << 22);
-  const uint32_t most = std::min(kCycleMost, std::max(1u, (large ? 16u : kCycleSweeps) / B));
+  const uint32_t most = std::min(kCycleMost, std::max(1u, (large_lattice(*lat) ? 16u : kCycleSweeps) / B));
   uint32_t n = 1;
   while (2u * n <= most && 2u * n <= left) n *= 2u;
   for (; n > 0 && n * B >= 4u; n /= 2u) {  // shorter ones: launch by launch
     const uint32_t key = kCycleKey | (uint32_t)swap << 16 | B << 8 | n;
-    auto it = lat->graphs->find(key);
-    if (it == lat->graphs->end() && left < 6ull * n) {
-      lat->graphs->emplace(key, nullptr);  // wanted: built when it is asked for again
-      continue;
-    }
-    if (it == lat->graphs->end() || !it->second) {
-      cudaGraphExec_t ex = nullptr;
-      const int st = build_graph(lat, inv, B, n, swap, &ex);
+    GraphSlot* slot = graph_slot(lat, key, left / n);
+    if (!slot) continue;
+    if (!slot->exec) {
+      const int st = build_graph(lat, inv, B, n, swap, &slot->exec);
       if (st) return st;
-      (*lat->graphs)[key] = ex;
-      it = lat->graphs->find(key);
     }
     if (!lat->t_dev_valid) CK(launch_set_tick(*lat, lat->sweeps, lat->ser_count, lat->steps));
-    CK(cudaGraphLaunch(it->second, lat->stream));
+    CK(cudaGraphLaunch(slot->exec, lat->stream));
     lat->sweeps += (uint64_t)B * n;
     if (swap != Swap::kOnly) lat->ser_count += n;
     if (swap != Swap::kNone) lat->steps += n;
@@ -801,7 +816,7 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   lat->use_graphs = true;
   lat->use_resident = true;
   lat->resident_mode = 1;
-  lat->graphs = new (std::nothrow) std::map<uint32_t, cudaGraphExec_t>();
+  lat->graphs = new (std::nothrow) std::map<uint32_t, GraphSlot>();
 
   auto bail = [&](int code) {
     if (lat->owns_buffer) cudaFree(lat->base);
@@ -853,9 +868,15 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   if (!lat) return IANUS_EINVAL;                            \
   if (lat->sticky) return (ianus_status)lat->sticky;
 
-ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uint64_t nsweeps,
-                         uint32_t measure_every) {
-  GET_LAT(h);
+// Whether a run of n sweeps of a small plain lattice is resident.
+static bool resident_i8_run(Lattice& lat, uint64_t n, uint32_t measure_every) {
+  return lat.use_resident && resident_i8_fits(lat) && (lat.R == 1 || measure_every == 0) && n >= 2 &&
+         (lat.resident_mode != 1 || resident_i8_pays(lat, measure_every));
+}
+
+// ianus_sweep within a call that makes `reps` more of the same.
+static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
+                              uint32_t measure_every, uint64_t reps) {
   if (lat->pool) return IANUS_EINVAL;  // a pool is driven by ianus_sweep_segments
   if (!beta || (algo != IANUS_METROPOLIS && algo != IANUS_HEATBATH)) return IANUS_EINVAL;
   if (!beta_ok(beta, lat->K)) return IANUS_EINVAL;
@@ -865,8 +886,7 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
     if (st) return (ianus_status)st;
   }
   const int inv = algo == IANUS_HEATBATH;
-  if (lat->use_resident && resident_i8_fits(*lat) && (lat->R == 1 || measure_every == 0) && nsweeps >= 2 &&
-      (lat->resident_mode != 1 || resident_i8_pays(*lat, measure_every))) {
+  if (resident_i8_run(*lat, nsweeps, measure_every)) {
     // small plain lattice: whole configurations in shared memory, many sweeps per launch
     uint64_t left = nsweeps;
     while (left > 0) {
@@ -891,7 +911,7 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
     }
     uint64_t chunk = left;  // sweeps up to the next measurement point
     if (measure_every) chunk = std::min<uint64_t>(chunk, measure_every - lat->sweeps % measure_every);
-    int st = sweeps_graphed(lat, inv, chunk);
+    int st = sweeps_graphed(lat, inv, chunk, measure_every ? reps * std::max<uint64_t>(1, left / measure_every) : reps);
     if (st) return (ianus_status)st;
     left -= chunk;
     if (measure_every && lat->sweeps % measure_every == 0) {
@@ -900,6 +920,13 @@ ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uin
     }
   }
   return IANUS_OK;
+}
+
+ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uint64_t nsweeps,
+                         uint32_t measure_every) {
+  GET_LAT(h);
+  lat->calls += 1;
+  return sweep_run(lat, algo, beta, nsweeps, measure_every, 1);
 }
 
 ianus_status ianus_pt_swap(ianus_lattice* h) {
@@ -916,10 +943,11 @@ ianus_status ianus_sweep_pt(ianus_lattice* h, int32_t algo, const double* beta, 
   if (swap_every == 0 || nsweeps % swap_every != 0) return IANUS_EINVAL;
   if (lat->K < 2) return IANUS_EINVAL;
   if (lat->model != IANUS_EA_PM_J || lat->field) return IANUS_EUNSUPPORTED;
+  lat->calls += 1;
   for (uint64_t n = 0; n < nsweeps; n += swap_every) {
     // cycles that end in a measurement (or none) and a swap, once the first
     // has checked the arguments and brought the tables up to date
-    if (n > 0 && swap_every <= kCycleSweeps &&
+    if (n > 0 && swap_every <= kCycleSweeps && !resident_i8_run(*lat, swap_every, measure_every) &&
         (measure_every == 0 || (measure_every == swap_every && lat->sweeps % swap_every == 0))) {
       uint32_t ran = 0;
       const int st = cycles_graphed(lat, algo == IANUS_HEATBATH, swap_every, (nsweeps - n) / swap_every,
@@ -930,7 +958,7 @@ ianus_status ianus_sweep_pt(ianus_lattice* h, int32_t algo, const double* beta, 
         continue;
       }
     }
-    ianus_status st = ianus_sweep(h, algo, beta, swap_every, measure_every);
+    ianus_status st = sweep_run(lat, algo, beta, swap_every, measure_every, (nsweeps - n) / swap_every);
     if (st) return st;
     st = ianus_pt_swap(h);
     if (st) return st;
@@ -1240,19 +1268,20 @@ ianus_status ianus_sweep_segments(ianus_lattice* h, uint64_t nsweeps) {
   GET_LAT(h);
   lat->mut += 1;  // the state changes other than by sweeps
   if (!lat->segs) return IANUS_EUNSUPPORTED;
+  lat->calls += 1;
   uint64_t left = nsweeps;
   const bool resident = nsweeps >= 2 && lat->use_resident && resident_fused_fits(*lat);
   while (left > 0) {
     const uint32_t B = (uint32_t)std::min<uint64_t>(left, resident ? kResidentBlock : 64);
+    GraphSlot* slot = nullptr;
+    if (!resident && B >= 4 && lat->use_graphs && lat->graphs) slot = graph_slot(lat, (1u << 31) | B, left / B);
     if (resident) {
       CK(launch_resident_fused(*lat, B));
-    } else if (B < 4 || !lat->use_graphs || !lat->graphs) {
+    } else if (!slot) {
       const int st = fused_sweeps(lat, B, false);
       if (st) return (ianus_status)st;
     } else {
-      const uint32_t key = (1u << 31) | B;
-      auto it = lat->graphs->find(key);
-      if (it == lat->graphs->end()) {
+      if (!slot->exec) {
         if (!lat->cap_stream) CK(cudaStreamCreateWithFlags(&lat->cap_stream, cudaStreamNonBlocking));
         cudaStream_t user = lat->stream;
         lat->stream = lat->cap_stream;
@@ -1262,17 +1291,15 @@ ianus_status ianus_sweep_segments(ianus_lattice* h, uint64_t nsweeps) {
         if (e == cudaSuccess) st = fused_sweeps(lat, B, true);
         cudaError_t e2 = cudaStreamEndCapture(lat->cap_stream, &g);
         lat->stream = user;
-        cudaGraphExec_t ex = nullptr;
         if (e != cudaSuccess || e2 != cudaSuccess || st != IANUS_OK || !g ||
-            cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) {
+            cudaGraphInstantiate(&slot->exec, g, 0) != cudaSuccess) {
           if (g) cudaGraphDestroy(g);
           cudaGetLastError();
           return IANUS_ECUDA;
         }
         cudaGraphDestroy(g);
-        it = lat->graphs->emplace(key, ex).first;
       }
-      CK(cudaGraphLaunch(it->second, lat->stream));
+      CK(cudaGraphLaunch(slot->exec, lat->stream));
     }
     // the host copy follows the device counters: every live segment advances
     for (int g = 0; g < lat->G; ++g)

@@ -61,6 +61,12 @@ constexpr int kMaxSegs = 64;  // per group
 
 constexpr int kMaxChains = 4;
 
+// A captured graph (null: not captured yet) and the call that last asked for it.
+struct GraphSlot {
+  cudaGraphExec_t exec;
+  uint64_t asked;
+};
+
 struct Lattice {
   ianus_config cfg;
   int model, D, L, S, R, K, slots, layout;
@@ -173,8 +179,8 @@ struct Lattice {
   cudaStream_t side_streams[kMaxChains];  // the other chains of a captured block, then its accumulators' stream
   int chain, chains;         // while capturing a graph of several chains: the one launched now
   // by block length (sweeps only), or kCycleKey | swap << 16 | sweeps << 8 | cycles
-  // (a null entry: wanted once, not built yet)
-  std::map<uint32_t, cudaGraphExec_t>* graphs;
+  std::map<uint32_t, GraphSlot>* graphs;
+  uint64_t calls;            // sweep calls so far
 };
 
 // ---- host table builders (tables.cpp) ----
