@@ -31,7 +31,8 @@ struct Sizes {
   bool poolable;
   size_t off_segs, off_nseg;
   size_t off_spins, off_J, off_thr, off_tp, off_fthr, off_ftp, off_sites, off_ptab, off_pttab, off_ptsign, off_slot,
-      off_temp, off_acc_pt, off_acc, off_oE, off_oM, off_oQ, off_sw, off_sE, off_sM, off_sQ, off_err, off_tdev, off_flags, total;
+      off_temp, off_acc_pt, off_acc, off_oE, off_oM, off_oQ, off_sw, off_sE, off_sM, off_sQ, off_err, off_tdev, off_flags, least, total;
+  size_t off_masks, mask_bytes;
   size_t spins_bytes, J_bytes, sites_bytes;
 };
 
@@ -144,6 +145,11 @@ int plan(const ianus_config* c, Sizes& z) {
   z.off_tdev = take(24);
   // progress flags of the persistent one-temperature bit-sliced sweep
   z.off_flags = take(layout == IANUS_LAYOUT_BITS64 && !field && z.K == 1 ? (size_t)kMaxPersistBlocks * 4 : 0);
+  z.least = o;  // a smaller buffer is refused; the rest only makes sweeps faster
+  z.mask_bytes = layout == IANUS_LAYOUT_I8 && !field && c->rng == IANUS_RNG_PHILOX && z.K == 1
+                     ? packed_mask_bytes(z.N, (uint64_t)z.S * z.R)
+                     : 0;
+  z.off_masks = take(z.mask_bytes);
   z.total = o;
   return IANUS_OK;
 }
@@ -761,9 +767,9 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   lat->jitf_algo = -1;
   lat->mut = 0;
   lat->acc_ok = false;
-  lat->bytes = z.total;
+  lat->bytes = cfg->device_buffer && cfg->device_buffer_bytes < z.total ? z.least : z.total;
   if (cfg->device_buffer) {
-    if (cfg->device_buffer_bytes < z.total || ((uintptr_t)cfg->device_buffer & 255u)) {
+    if (cfg->device_buffer_bytes < z.least || ((uintptr_t)cfg->device_buffer & 255u)) {
       delete lat;
       return IANUS_EINVAL;
     }
@@ -813,6 +819,8 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   lat->err = (uint32_t*)(b + z.off_err);
   lat->flags = (z.layout == IANUS_LAYOUT_BITS64 && !z.field && z.K == 1) ? (uint32_t*)(b + z.off_flags) : nullptr;
   lat->t_dev = (uint64_t*)(b + z.off_tdev);
+  lat->mask_bytes = lat->bytes == z.total ? z.mask_bytes : 0;
+  lat->masks = lat->mask_bytes ? (uint4*)(b + z.off_masks) : nullptr;
   lat->use_graphs = true;
   lat->use_resident = true;
   lat->resident_mode = 1;
@@ -835,7 +843,7 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
       return bail(IANUS_ENOMEM);
     }
   }
-  if (cudaMemsetAsync(lat->base, 0, z.total, lat->stream) != cudaSuccess) return bail(IANUS_ECUDA);
+  if (cudaMemsetAsync(lat->base, 0, z.least, lat->stream) != cudaSuccess) return bail(IANUS_ECUDA);
   {
     std::vector<int32_t> perm((size_t)z.S * z.R * z.K);
     for (size_t c = 0; c < perm.size(); ++c) perm[c] = (int32_t)(c % z.K);
@@ -871,7 +879,7 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
 // Whether a run of n sweeps of a small plain lattice is resident.
 static bool resident_i8_run(Lattice& lat, uint64_t n, uint32_t measure_every) {
   return lat.use_resident && resident_i8_fits(lat) && (lat.R == 1 || measure_every == 0) && n >= 2 &&
-         (lat.resident_mode != 1 || resident_i8_pays(lat, measure_every));
+         (lat.resident_mode != 1 || packed_i8_pays(lat, n) || resident_i8_pays(lat, measure_every));
 }
 
 // ianus_sweep within a call that makes `reps` more of the same.
@@ -891,7 +899,10 @@ static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, ui
     uint64_t left = nsweeps;
     while (left > 0) {
       const uint32_t n = (uint32_t)std::min<uint64_t>(left, 65536);
-      CK(launch_resident_i8(*lat, inv, n, measure_every));
+      if (lat->resident_mode == 1 && packed_i8_pays(*lat, n))
+        CK(launch_packed_i8(*lat, inv, n, measure_every));
+      else
+        CK(launch_resident_i8(*lat, inv, n, measure_every));
       if (measure_every)  // measured sweeps t+1 in (sweeps, sweeps + n] with (t+1) % every == 0
         lat->ser_count += (lat->sweeps + n) / measure_every - lat->sweeps / measure_every;
       lat->sweeps += n;

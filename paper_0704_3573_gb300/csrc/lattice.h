@@ -181,6 +181,8 @@ struct Lattice {
   // by block length (sweeps only), or kCycleKey | swap << 16 | sweeps << 8 | cycles
   std::map<uint32_t, GraphSlot>* graphs;
   uint64_t calls;            // sweep calls so far
+  uint4* masks;              // packed resident sweeps (k_packed.cu): a run's random decisions; null: not used
+  size_t mask_bytes;
 };
 
 // ---- host table builders (tables.cpp) ----
@@ -311,6 +313,13 @@ cudaError_t launch_get_spins_bits(Lattice& lat, int8_t* dev_out);
 cudaError_t launch_set_spins_bits(Lattice& lat, const int8_t* dev_in);
 cudaError_t launch_get_couplings_bits(Lattice& lat, int8_t* dev_out);
 cudaError_t launch_set_couplings_bits(Lattice& lat, const int8_t* dev_in);
+// Resident sweeps of small plain lattices, 32 sites a word (k_packed.cu): bytes
+// of the random decisions kept (0: not for this lattice), whether such a run is
+// the faster one, the run.
+constexpr size_t kPackedBytes = 8u << 20;
+size_t packed_mask_bytes(uint32_t N, uint64_t configs);
+bool packed_i8_pays(const Lattice& lat, uint64_t nsweeps);
+cudaError_t launch_packed_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t measure_every);
 // U8X4 Potts (k_potts.cu)
 cudaError_t launch_init_potts(Lattice& lat, int jmode);
 cudaError_t launch_sweep_potts(Lattice& lat, int colour, uint64_t t);
