@@ -248,6 +248,11 @@ typedef struct {
  * tables, series).  Returns 0 for an invalid configuration.  Host only. */
 size_t ianus_required_bytes(const ianus_config* cfg);
 
+/* The same with the room that its fastest sweep uses (small plain lattices: up
+ * to 8 MiB of random decisions drawn ahead).  A device buffer between the two
+ * sizes is used without it; the results do not depend on it.  Host only. */
+size_t ianus_preferred_bytes(const ianus_config* cfg);
+
 /* Validates cfg, takes device memory (cfg->device_buffer if non-NULL, which
  * the caller keeps alive until ianus_destroy; else cudaMalloc), and fills
  * the couplings and the initial configuration from the seed on the device

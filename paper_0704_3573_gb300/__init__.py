@@ -43,7 +43,7 @@ EXPORTS = [
     "ianus_table_pt", "ianus_measure_bits64_noalloc", "ianus_set_variant", "ianus_set_block_words",
     "ianus_set_graphs", "ianus_set_resident", "ianus_get_sites_i8", "ianus_set_sites_i8", "ianus_table_field",
     "ianus_table_potts_counts", "ianus_segment_load", "ianus_segment_release", "ianus_segment_state",
-    "ianus_sweep_segments", "ianus_set_persistent_wait", "ianus_prepare_sweep",
+    "ianus_sweep_segments", "ianus_set_persistent_wait", "ianus_prepare_sweep", "ianus_preferred_bytes",
 ]
 
 
@@ -96,6 +96,7 @@ def lib(build_if_missing: bool = True):
     cfgp = C.POINTER(IanusConfig)
     sig = {
         "ianus_required_bytes": (sz, [cfgp]),
+        "ianus_preferred_bytes": (sz, [cfgp]),
         "ianus_lattice_create": (i32, [cfgp, C.POINTER(vp)]),
         "ianus_sweep": (i32, [vp, i32, dp, u64, u32]),
         "ianus_pt_swap": (i32, [vp]),
@@ -231,7 +232,7 @@ class Lattice:
         cfg.rng = _RNGS[rng] if isinstance(rng, str) else int(rng)
         cfg.series_capacity = series_capacity
         cfg.seed = seed & 0xFFFFFFFFFFFFFFFF
-        nbytes = self._lib.ianus_required_bytes(C.byref(cfg))
+        nbytes = self._lib.ianus_preferred_bytes(C.byref(cfg))
         if nbytes == 0:
             # invalid configuration: ianus_lattice_create validates it the
             # same way (before any allocation) and names the reason

@@ -145,7 +145,7 @@ int plan(const ianus_config* c, Sizes& z) {
   z.off_tdev = take(24);
   // progress flags of the persistent one-temperature bit-sliced sweep
   z.off_flags = take(layout == IANUS_LAYOUT_BITS64 && !field && z.K == 1 ? (size_t)kMaxPersistBlocks * 4 : 0);
-  z.least = o;  // a smaller buffer is refused; the rest only makes sweeps faster
+  z.least = o;  // the rest only makes sweeps faster
   z.mask_bytes = layout == IANUS_LAYOUT_I8 && !field && c->rng == IANUS_RNG_PHILOX && z.K == 1
                      ? packed_mask_bytes(z.N, (uint64_t)z.S * z.R)
                      : 0;
@@ -709,6 +709,12 @@ struct StateHeader {
 extern "C" {
 
 size_t ianus_required_bytes(const ianus_config* cfg) {
+  Sizes z;
+  if (plan(cfg, z) != IANUS_OK) return 0;
+  return z.least;
+}
+
+size_t ianus_preferred_bytes(const ianus_config* cfg) {
   Sizes z;
   if (plan(cfg, z) != IANUS_OK) return 0;
   return z.total;

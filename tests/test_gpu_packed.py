@@ -54,7 +54,8 @@ def test_a_smaller_buffer_sweeps_without_the_decisions(ianus):
     lib = a._lib
     cfg = type(a.cfg)()
     C.memmove(C.byref(cfg), C.byref(a.cfg), C.sizeof(cfg))
-    least = cfg.device_buffer_bytes - 1024 * 2 * 512  # a byte a site and sweep
+    least = lib.ianus_required_bytes(C.byref(cfg))
+    assert cfg.device_buffer_bytes == lib.ianus_preferred_bytes(C.byref(cfg)) == least + 1024 * 2 * 512
     buf = torch.empty(least, dtype=torch.uint8, device="cuda")
     cfg.device_buffer, cfg.device_buffer_bytes = buf.data_ptr(), least
     h = C.c_void_p()
