@@ -8,6 +8,7 @@
 #include <functional>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -706,6 +707,118 @@ struct StateHeader {
 
 }  // namespace
 
+// ---- reads of results ----
+
+namespace {
+
+// Page-locked memory that small results pass through on their way to the
+// caller's arrays: a copy straight into pageable memory waits for the stream and
+// for the driver's own staging each time, about 8 us an array, one into
+// page-locked memory is queued with the others (measure() of L=8, 64 samples x
+// 2: 55 -> 38 us).  Blocks belong to one call at a time; the process keeps up to
+// kPinnedMost of them, and a call that finds none copies directly.  Large arrays
+// are copied directly (3.5 MB: 160 us less than staged) once their pages exist:
+// the copy engine spends some 500 us on each MB of new ones, so the host touches
+// them first, while the GPU is still at work (11 MB of series into new arrays,
+// with the 48 swap steps that filled it: 8.7 -> 2.4 ms).
+constexpr size_t kPinnedBytes = 1u << 20;
+constexpr int kPinnedMost = 4;
+constexpr size_t kStagedMost = 512u << 10;  // bytes of an array that is staged
+constexpr size_t kPage = 4096;
+
+class PinnedBlock {
+ public:
+  PinnedBlock() {
+    std::lock_guard<std::mutex> lock(mutex());
+    if (!idle().empty()) {
+      p_ = idle().back();
+      idle().pop_back();
+    } else if (count() < kPinnedMost) {
+      if (cudaHostAlloc(&p_, kPinnedBytes, cudaHostAllocPortable) == cudaSuccess) {
+        ++count();
+      } else {
+        cudaGetLastError();
+        p_ = nullptr;
+      }
+    }
+  }
+  ~PinnedBlock() {
+    if (!p_) return;
+    std::lock_guard<std::mutex> lock(mutex());
+    idle().push_back(p_);  // its room was reserved below
+  }
+  PinnedBlock(const PinnedBlock&) = delete;
+  PinnedBlock& operator=(const PinnedBlock&) = delete;
+  uint8_t* data() const { return (uint8_t*)p_; }
+
+ private:
+  static std::mutex& mutex() {
+    static std::mutex m;
+    return m;
+  }
+  static int& count() {
+    static int n = 0;
+    return n;
+  }
+  static std::vector<void*>& idle() {  // never destroyed: the driver may go first
+    static std::vector<void*>* v = [] {
+      auto* w = new std::vector<void*>();
+      w->reserve(kPinnedMost);
+      return w;
+    }();
+    return *v;
+  }
+  void* p_ = nullptr;
+};
+
+struct Read {
+  void* dst;  // host; null: skipped
+  const void* src;
+  size_t bytes;
+};
+
+// Whether a host array is pageable (others are copied to directly).
+bool pageable(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeUnregistered;
+}
+
+// Copies device ranges to the host and waits for them.
+int read_back(Lattice* lat, const Read* reads, int n) {
+  const PinnedBlock block;
+  uint8_t* const pin = block.data();
+  struct Part {
+    void* dst;
+    size_t at, bytes;
+  };
+  Part parts[8];
+  int np = 0;
+  size_t used = 0;
+  for (int i = 0; i < n; ++i) {
+    const Read& r = reads[i];
+    if (!r.dst || !r.bytes) continue;
+    const bool paged = pageable(r.dst);
+    if (pin && paged && r.bytes <= kStagedMost && used + r.bytes <= kPinnedBytes && np < 8) {
+      CK(cudaMemcpyAsync(pin + used, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream));
+      parts[np++] = Part{r.dst, used, r.bytes};
+      used += (r.bytes + 63) & ~(size_t)63;
+      continue;
+    }
+    if (paged && r.bytes > kStagedMost)
+      for (size_t o = 0; o < r.bytes; o += kPage) ((volatile uint8_t*)r.dst)[o] = 0;
+    CK(cudaMemcpyAsync(r.dst, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream));
+  }
+  CK(cudaStreamSynchronize(lat->stream));
+  for (int k = 0; k < np; ++k) std::memcpy(parts[k].dst, pin + parts[k].at, parts[k].bytes);
+  return IANUS_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 size_t ianus_required_bytes(const ianus_config* cfg) {
@@ -989,13 +1102,10 @@ ianus_status ianus_measure(ianus_lattice* h, int64_t* energy, int64_t* magnetisa
   int st = measure_into(lat, lat->out_E, lat->out_M, lat->out_Q, nullptr, overlap != nullptr);
   if (st) return (ianus_status)st;
   const size_t SKR = (size_t)lat->S * lat->K * lat->R;
-  if (energy) CK(cudaMemcpyAsync(energy, lat->out_E, SKR * 8, cudaMemcpyDeviceToHost, lat->stream));
-  if (magnetisation)
-    CK(cudaMemcpyAsync(magnetisation, lat->out_M, SKR * lat->mq * 8, cudaMemcpyDeviceToHost, lat->stream));
-  if (overlap)
-    CK(cudaMemcpyAsync(overlap, lat->out_Q, (size_t)lat->S * lat->K * 8, cudaMemcpyDeviceToHost, lat->stream));
-  CK(cudaStreamSynchronize(lat->stream));
-  return IANUS_OK;
+  const Read reads[] = {{energy, lat->out_E, SKR * 8},
+                        {magnetisation, lat->out_M, SKR * lat->mq * 8},
+                        {overlap, lat->out_Q, (size_t)lat->S * lat->K * 8}};
+  return (ianus_status)read_back(lat, reads, 3);
 }
 
 ianus_status ianus_read_series(ianus_lattice* h, uint64_t* sweep, int64_t* energy, int64_t* magnetisation,
@@ -1007,20 +1117,20 @@ ianus_status ianus_read_series(ianus_lattice* h, uint64_t* sweep, int64_t* energ
   const size_t SKR = (size_t)lat->S * lat->K * lat->R, SK = (size_t)lat->S * lat->K;
   // the rows are contiguous in the ring except where it wraps: at most two
   // copies per array
+  Read reads[8];
+  int nr = 0;
   for (uint64_t r = 0; r < n;) {
     const size_t pos = (size_t)((first + r) % lat->cap);
     const size_t m = (size_t)std::min<uint64_t>(n - r, lat->cap - pos);
-    if (sweep) CK(cudaMemcpyAsync(sweep + r, lat->ser_sweep + pos, m * 8, cudaMemcpyDeviceToHost, lat->stream));
-    if (energy)
-      CK(cudaMemcpyAsync(energy + r * SKR, lat->ser_E + pos * SKR, m * SKR * 8, cudaMemcpyDeviceToHost, lat->stream));
+    if (sweep) reads[nr++] = {sweep + r, lat->ser_sweep + pos, m * 8};
+    if (energy) reads[nr++] = {energy + r * SKR, lat->ser_E + pos * SKR, m * SKR * 8};
     if (magnetisation)
-      CK(cudaMemcpyAsync(magnetisation + r * SKR * lat->mq, lat->ser_M + pos * SKR * lat->mq,
-                         m * SKR * lat->mq * 8, cudaMemcpyDeviceToHost, lat->stream));
-    if (overlap && lat->R >= 2)
-      CK(cudaMemcpyAsync(overlap + r * SK, lat->ser_Q + pos * SK, m * SK * 8, cudaMemcpyDeviceToHost, lat->stream));
+      reads[nr++] = {magnetisation + r * SKR * lat->mq, lat->ser_M + pos * SKR * lat->mq, m * SKR * lat->mq * 8};
+    if (overlap && lat->R >= 2) reads[nr++] = {overlap + r * SK, lat->ser_Q + pos * SK, m * SK * 8};
     r += m;
   }
-  CK(cudaStreamSynchronize(lat->stream));
+  const int st = read_back(lat, reads, nr);
+  if (st) return (ianus_status)st;
   if (n_rows) *n_rows = (size_t)n;
   if (clear) lat->ser_first = lat->ser_count;
   return IANUS_OK;
@@ -1332,11 +1442,10 @@ ianus_status ianus_sweep_segments(ianus_lattice* h, uint64_t nsweeps) {
 ianus_status ianus_get_pt_state(ianus_lattice* h, int32_t* slot_at, uint64_t* accepted, uint64_t* swap_steps) {
   GET_LAT(h);
   const size_t n = (size_t)lat->S * lat->R * lat->K;
-  if (slot_at) CK(cudaMemcpyAsync(slot_at, lat->slot_at, n * 4, cudaMemcpyDeviceToHost, lat->stream));
-  if (accepted && lat->K > 1)
-    CK(cudaMemcpyAsync(accepted, lat->accepted, (size_t)lat->S * lat->R * (lat->K - 1) * 8, cudaMemcpyDeviceToHost,
-                       lat->stream));
-  CK(cudaStreamSynchronize(lat->stream));
+  const Read reads[] = {{slot_at, lat->slot_at, n * 4},
+                        {lat->K > 1 ? accepted : nullptr, lat->accepted, (size_t)lat->S * lat->R * (lat->K - 1) * 8}};
+  const int st = read_back(lat, reads, 2);
+  if (st) return (ianus_status)st;
   if (swap_steps) *swap_steps = lat->steps;
   return IANUS_OK;
 }
