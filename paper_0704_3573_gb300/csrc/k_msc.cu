@@ -1332,7 +1332,13 @@ int lanes_replicas(const Lattice& lat) { return lat.R % 2 == 0 ? 2 : 1; }
 
 // Launches a colour pass of a lane-queue kernel (jit_sweep_lt.cuh): ys block
 // rows, about min_blocks blocks per SM in all (one wave), whole warps of words.
-cudaError_t launch_lt(const Lattice& lat, cudaKernel_t k, BitsParams& p, uint32_t ys, int min_blocks, int block) {
+// Blocks that stage threshold rows (rows: per-lane planes) have at least a block
+// of words where they would have less than half of one: L=20, 100 samples x 4
+// replicas, blocks of 32 words 5.7 us a pass, of 128 or 256 3.8; L=14, 64
+// samples x 4 x 10 temperatures 6.2 (64 words) / 4.9 (128) / 4.3 (256); but L=20,
+// 64 x 2 x 20 temperatures 6.3 (192) / 6.8 (256).
+cudaError_t launch_lt(const Lattice& lat, cudaKernel_t k, BitsParams& p, uint32_t ys, int min_blocks, int block,
+                      bool rows = false) {
   uint32_t w;
   if (lat.block_words) {
     w = (lat.block_words + 31u) / 32u * 32u;
@@ -1340,6 +1346,7 @@ cudaError_t launch_lt(const Lattice& lat, cudaKernel_t k, BitsParams& p, uint32_
     const uint32_t per_row = std::max<uint32_t>(1u, 152u * (uint32_t)min_blocks / ys);
     w = (lat.geom.half + per_row - 1u) / per_row;
     w = std::max<uint32_t>(32u, (w + 31u) / 32u * 32u);
+    if (rows && w <= (uint32_t)block / 2u) w = (uint32_t)block;
   }
   p.words_per_block = w;
   // the rows of this chain (all of them but inside a graph of several)
@@ -1698,7 +1705,7 @@ cudaError_t launch_sweep_bits(Lattice& lat, int colour, uint64_t t, int inv) {
     const cudaKernel_t k = lat.jitp[algo][lane_queue(lat) ? 1 : 0];
     if (k && lane_queue(lat)) {
       const uint64_t ys = (uint64_t)gts * (uint64_t)(lat.R / lanes_replicas(lat));
-      if (ys <= 65535u) return launch_lt(lat, k, p, (uint32_t)ys, kLtBlocks, kLtBlock);
+      if (ys <= 65535u) return launch_lt(lat, k, p, (uint32_t)ys, kLtBlocks, kLtBlock, true);
     } else if (k) {
       const bool q = algo == 1 && bits_sweep_smem(lat.R, true) <= 227u * 1024u;
       void* args[] = {(void*)&p};

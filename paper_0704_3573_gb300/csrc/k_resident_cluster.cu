@@ -23,7 +23,7 @@
 // Bound: latency, about 0.8 us a pass and 0.6 ns a word and SM.  us per sweep,
 // heat bath, 64 samples (launched / one block / cluster): 3D L=8, one replica
 // 3.9 / 3.7 / 1.9; L=8 x 2 4.6 / 6.3 / 2.1; L=12 x 2 4.8 / 19 / 3.6; L=16 x 2
-// 5.0 / 41 / 6.5 (not taken); L=8 x 2 x 32 temperatures 9.3 / 6.3 / 3.5.
+// 5.1 / 41 / 6.5 (not taken); L=8 x 2 x 32 temperatures 7.3 / 6.3 / 3.5.
 #include "lattice.h"
 #include "sweep_planes.cuh"
 
@@ -312,9 +312,10 @@ double block_us(const Lattice& lat) { return 1.8 + 7.6e-3 * lat.R * lat.geom.hal
 
 double launched_us(const Lattice& lat) {
   const double words = (double)lat.G * lat.K * lat.R * lat.geom.half;
-  const double base = 3.7 + (lat.R >= 2 ? 0.9 : 0.0);
-  if (lat.K == 1 && lat.R <= 2) return base + 0.1e-3 * words;
-  return base + 1.3 + std::min(0.2e-3 * words, 4.1 + 0.05e-3 * words);
+  if (lat.K == 1 && lat.R <= 2)
+    return (lat.R == 1 ? 4.2 : 4.8) + std::min(0.08e-3 * words, 0.5 + 0.02e-3 * words);
+  const bool two = lat.R % 2 == 0;  // replicas a thread
+  return (lat.D == 3 ? (two ? 7.0 : 5.8) : (two ? 6.2 : 5.2)) + 0.03e-3 * words;
 }
 
 // Blocks of a cluster: the fastest of 16, 8, 4 and 2 that fit; 0 if there is
