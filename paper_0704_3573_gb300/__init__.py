@@ -240,7 +240,11 @@ class Lattice:
             st = self._lib.ianus_lattice_create(C.byref(cfg), C.byref(h))
             raise IanusError(st if st != OK else EINVAL, "ianus_lattice_create")
         with torch.cuda.device(dev):
-            self.buffer = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+            try:
+                self.buffer = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+            except torch.OutOfMemoryError:
+                nbytes = self._lib.ianus_required_bytes(C.byref(cfg))
+                self.buffer = torch.empty(nbytes, dtype=torch.uint8, device=dev)
         cfg.device_buffer = self.buffer.data_ptr()
         cfg.device_buffer_bytes = nbytes
         cfg.cuda_stream = stream.cuda_stream

@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libianus.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 
 SOURCES = ["api.cu", "k_plain.cu", "k_msc.cu", "k_potts.cu", "k_pt.cu", "k_perm.cu", "tables.cpp", "noalloc.cu", "jit.cu",
-           "k_resident_bits.cu", "k_resident_cluster.cu", "k_packed.cu"]
+           "k_resident_bits.cu", "k_resident_cluster.cu", "k_packed.cu", "k_words.cu"]
 PROBE_SOURCES = ["probe.cu"]
 PROBE_LIB = os.path.join(HERE, "libianus_probe.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

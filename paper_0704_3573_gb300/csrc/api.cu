@@ -33,7 +33,8 @@ struct Sizes {
   size_t off_segs, off_nseg;
   size_t off_spins, off_J, off_thr, off_tp, off_fthr, off_ftp, off_sites, off_ptab, off_pttab, off_ptsign, off_slot,
       off_temp, off_acc_pt, off_acc, off_oE, off_oM, off_oQ, off_sw, off_sE, off_sM, off_sQ, off_err, off_tdev, off_flags, least, total;
-  size_t off_masks, mask_bytes;
+  size_t off_masks, mask_bytes, off_wspins, off_wJ, off_wtp;
+  bool words;  // room for the lattice in words
   size_t spins_bytes, J_bytes, sites_bytes;
 };
 
@@ -151,6 +152,14 @@ int plan(const ianus_config* c, Sizes& z) {
                      ? packed_mask_bytes(z.N, (uint64_t)z.S * z.R)
                      : 0;
   z.off_masks = take(z.mask_bytes);
+  // the same lattice in words: from 8 samples on, at most 2 GiB
+  const size_t wspins = (size_t)z.G * z.slots * z.N * 8, wJ = (size_t)z.G * z.D * z.N * 8;
+  const size_t wtp = (size_t)z.G * z.slots * kPlanes * kMaxClasses * 8;
+  z.words = layout == IANUS_LAYOUT_I8 && !field && c->rng == IANUS_RNG_PHILOX && z.K == 1 && z.S >= 8 &&
+            wspins + wJ + wtp <= (size_t)2 << 30;
+  z.off_wspins = take(z.words ? wspins : 0);
+  z.off_wJ = take(z.words ? wJ : 0);
+  z.off_wtp = take(z.words ? wtp : 0);
   z.total = o;
   return IANUS_OK;
 }
@@ -897,6 +906,11 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   } else {
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, z.total);
+    if (e == cudaErrorMemoryAllocation && z.least < z.total) {
+      cudaGetLastError();
+      lat->bytes = z.least;
+      e = cudaMalloc(&p, z.least);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       delete lat;
@@ -947,6 +961,8 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
 
   auto bail = [&](int code) {
     if (lat->owns_buffer) cudaFree(lat->base);
+    if (lat->words) delete lat->words->graphs;
+    delete lat->words;
     delete lat->graphs;
     delete lat;
     return (ianus_status)code;
@@ -986,6 +1002,22 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
                                        : launch_init_sites_bits(*lat, cfg->occupation);
   if (e == cudaSuccess && lat->wheels) e = launch_init_wheels(*lat);
   if (e != cudaSuccess || cudaStreamSynchronize(lat->stream) != cudaSuccess) return bail(IANUS_ECUDA);
+  if (z.words && lat->bytes == z.total) {
+    // everything but the spins, the couplings and the planes is shared
+    lat->words = new (std::nothrow) Lattice(*lat);
+    if (lat->words) {
+      Lattice* w = lat->words;
+      w->layout = IANUS_LAYOUT_BITS64;
+      w->spins = b + z.off_wspins;
+      w->J = b + z.off_wJ;
+      w->tp = (uint64_t*)(b + z.off_wtp);
+      w->masks = nullptr;
+      w->mask_bytes = 0;
+      w->owns_buffer = false;
+      w->variant = 1;  // no run-time compiler: plain sweeps take new temperatures as they come
+      w->graphs = new (std::nothrow) std::map<uint32_t, GraphSlot>();
+    }
+  }
   *out = reinterpret_cast<ianus_lattice*>(lat);
   return IANUS_OK;
 }
@@ -1000,6 +1032,9 @@ static bool resident_i8_run(Lattice& lat, uint64_t n, uint32_t measure_every) {
   return lat.use_resident && resident_i8_fits(lat) && (lat.R == 1 || measure_every == 0) && n >= 2 &&
          (lat.resident_mode != 1 || packed_i8_pays(lat, n) || resident_i8_pays(lat, measure_every));
 }
+
+static ianus_status sweep_words(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
+                                uint32_t measure_every);
 
 // ianus_sweep within a call that makes `reps` more of the same.
 static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
@@ -1030,6 +1065,8 @@ static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, ui
     }
     return IANUS_OK;
   }
+  if (lat->words && lat->use_resident && lat->resident_mode == 1 && lat->variant == 0 && words_pay(*lat, nsweeps))
+    return sweep_words(lat, algo, beta, nsweeps, measure_every);
   uint64_t left = nsweeps;
   while (left > 0) {
     if (measure_every && lat->sweeps % measure_every == 0 && left >= measure_every) {
@@ -1049,6 +1086,36 @@ static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, ui
       if (st) return (ianus_status)st;
     }
   }
+  return IANUS_OK;
+}
+
+// A plain lattice's sweeps in words: the counters and the series are the
+// lattice's own.
+static ianus_status sweep_words(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
+                                uint32_t measure_every) {
+  Lattice* w = lat->words;
+  if (lat->words_mut != lat->mut + 1) {
+    CK(launch_pack_couplings(*lat));
+    lat->words_mut = lat->mut + 1;
+  }
+  CK(launch_pack_spins(*lat));
+  w->use_graphs = lat->use_graphs;
+  w->sweeps = lat->sweeps;
+  w->ser_count = lat->ser_count;
+  w->steps = lat->steps;
+  w->t_dev_valid = false;
+  w->acc_ok = false;
+  w->calls += 1;
+  const ianus_status st = sweep_run(w, algo, beta, nsweeps, measure_every, 1);
+  lat->sweeps = w->sweeps;
+  lat->ser_count = w->ser_count;
+  lat->t_dev_valid = false;
+  lat->acc_ok = false;
+  if (st) {
+    lat->sticky = w->sticky;
+    return st;
+  }
+  CK(launch_unpack_spins(*lat));
   return IANUS_OK;
 }
 
@@ -1651,6 +1718,14 @@ ianus_status ianus_destroy(ianus_lattice* h) {
   cudaStreamSynchronize(lat->stream);
   drop_graphs(lat);
   delete lat->graphs;
+  if (Lattice* w = lat->words) {
+    drop_graphs(w);
+    delete w->graphs;
+    if (w->cap_stream) cudaStreamDestroy(w->cap_stream);
+    for (cudaStream_t s : w->side_streams)
+      if (s) cudaStreamDestroy(s);
+    delete w;
+  }
   delete lat->segs_host;
   delete lat->nseg_host;
   delete lat->tp_host;

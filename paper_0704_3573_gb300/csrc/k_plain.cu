@@ -2052,6 +2052,8 @@ PlainChoice plain_choice(const Lattice& lat) {
   return best;
 }
 
+double plain_us(const Lattice& lat) { return plain_choice(lat).us; }
+
 PlainPath plain_path(const Lattice& lat) {
   // with the small-lattice sweeps switched off, the large-lattice choice
   if (lat.variant == 0 && !lat.use_resident) return i8_sliced_fits(lat) ? PlainPath::kSliced : PlainPath::kShared;

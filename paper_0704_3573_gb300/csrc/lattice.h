@@ -183,6 +183,8 @@ struct Lattice {
   uint64_t calls;            // sweep calls so far
   uint4* masks;              // packed resident sweeps (k_packed.cu): a run's random decisions; null: not used
   size_t mask_bytes;
+  Lattice* words;            // the same lattice in words (k_words.cu); null: not used
+  uint64_t words_mut;        // mut + 1 when its couplings were packed
 };
 
 // ---- host table builders (tables.cpp) ----
@@ -320,6 +322,13 @@ constexpr size_t kPackedBytes = 8u << 20;
 size_t packed_mask_bytes(uint32_t N, uint64_t configs);
 bool packed_i8_pays(const Lattice& lat, uint64_t nsweeps);
 cudaError_t launch_packed_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t measure_every);
+// Plain lattices swept in words (k_words.cu): between lat's bytes and
+// lat.words', and whether a run of n sweeps is faster so.
+cudaError_t launch_pack_spins(Lattice& lat);
+cudaError_t launch_pack_couplings(Lattice& lat);
+cudaError_t launch_unpack_spins(Lattice& lat);
+bool words_pay(const Lattice& lat, uint64_t n);
+double plain_us(const Lattice& lat);  // estimated us of a plain sweep
 // U8X4 Potts (k_potts.cu)
 cudaError_t launch_init_potts(Lattice& lat, int jmode);
 cudaError_t launch_sweep_potts(Lattice& lat, int colour, uint64_t t);
