@@ -66,11 +66,6 @@ TRAFFIC_SOURCE_HASH = "0b06d535be286e49"
 POTTS_TRAFFIC = {"l1_global_load_bytes": 179127744, "l2_bytes": 73770400, "dram_bytes": 21049344,
                  "l1_hit_rate_pct": 78.5}
 POTTS_SOURCE_HASH = "ab9e8badae2a5729"
-# DRAM traffic of one colour launch of the plain-layout sweep
-# (k_sweep_i8_sliced) on the bench workload, from one ncu capture, valid
-# while its sources are unchanged.
-PLAIN_TRAFFIC = {"dram_read_bytes": 337867008, "dram_write_bytes": 94819584}
-PLAIN_SOURCE_HASH = "69d32de33006c0d7"
 # The kernel variant and launch shape the bench runs by default: the
 # lane-queue kernel in its one-wave launch (the automatic choice for one
 # temperature), fixed so that the profile above describes the timed kernel.
@@ -376,40 +371,26 @@ def run_gpu(args, ws, rank, local):
         torch.cuda.synchronize()
         ps = p0.elapsed_time(p1) / 1e3
         pv = S * R * L ** 3 * nps / (ps * 1e9)
-        # roofline of the plain form: the smaller of two bounds.  HBM: per
-        # update the site's byte read and written and its share of the other
-        # colour's bytes (3 B) and the 6 coupling bytes each configuration
-        # streams (9 B, the couplings larger than L2).  Issue: the kernel
-        # updates 64-lane words built in shared memory, so per update the
-        # per-lane-plane word update of the bit-sliced form / 64 (e-words 12,
-        # adder tree 16, "always" and undecided masks 16, per plane the
-        # threshold multiplexers 6 + compare 4, per pair Philox 21 + merge 2,
-        # 3.92 pairs; 20 mad.wide per Philox block) plus the layout's own
-        # work: the sign packing (9 ops per 32 bytes and lane) and the 32 x 32
-        # bit transposes (5 ops per stage, 5 stages) of the bytes read and
-        # written, about 13.5 B per update
+        # roofline of the plain form: the smaller of two bounds.  HBM: the
+        # spins read as bytes and written as words before the run and back
+        # after it.  Issue: the per-lane-plane word update of the bit-sliced
+        # form / 64 (e-words 12, adder tree 16, "always" and undecided masks
+        # 16, per plane the threshold multiplexers 6 + compare 4, per pair
+        # Philox 18 + merge 2, 3.92 pairs; 16 mad.wide per Philox block)
         hbm = MEASURED.get("hbm_gbs")
-        b_upd = 9.0
+        b_upd = 2.25 / nps
         npp = expected_plane_pairs()
-        ops_upd = (44 + npp * (2 * 10 + 23) + npp * 20) / 64 + 13.5 * (9 + 25) / 32
+        ops_upd = (44 + npp * (2 * 10 + 20) + npp * 16) / 64
         pk = _issue_peak()
         bounds = {"hbm": hbm / b_upd if hbm else None, "alu": pk * 1e3 / ops_upd if pk else None}
         binding = min((v, k) for k, v in bounds.items() if v)[1] if any(bounds.values()) else None
-        traffic = None
-        if kernel_source_hash(("common.cuh", "sweep_planes.cuh", "k_plain.cu")) == PLAIN_SOURCE_HASH:
-            upd_pass = S * R * L ** 3 // 2
-            traffic = {"dram_bytes_per_update": (PLAIN_TRAFFIC["dram_read_bytes"] + PLAIN_TRAFFIC["dram_write_bytes"])
-                       / upd_pass, **PLAIN_TRAFFIC,
-                       "what": "ncu, one colour launch; below the 9 B algorithmic figure because one block sweeps "
-                               "both replicas of a tile and reads their shared couplings once"}
         plain = {"value": pv, "unit": UNIT, "layout": "i8 (one byte per spin)", "sweeps": nps,
-                 "kernel": "k_sweep_i8_sliced (tiles of the 64-sample group, both replicas, turned into 64-lane "
-                           "words in shared memory by warp bit transposes, updated bit-sliced, written back as bytes)",
+                 "kernel": "k_sweep_bits: spins packed into 64-sample words for the run of sweeps and unpacked after it "
+                           "(k_words.cu), swept by the precompiled per-lane-plane kernel, measured in words",
                  "speedup_bitsliced_over_plain": value / ws / pv,
                  "roofline": {"bound": binding, "bytes_per_update": b_upd, "ops_per_update": ops_upd,
                               "bound_updates_per_ns": bounds,
                               "frac": pv / bounds[binding] if binding else None,
-                              "traffic": traffic,
                               "peaks": {"hbm_gbs": hbm, "issue_tops": pk}}}
         del pl
 
@@ -428,7 +409,11 @@ def run_gpu(args, ws, rank, local):
     serving = run_serving(args) if (rank == 0 and args.serve_jobs > 0) else None
     others = run_other_configs(args) if (rank == 0 and not args.no_others) else None
 
-    launches = args.steps * (2 * SWEEPS_PER_STEP + 2 * (SWEEPS_PER_STEP // MEASURE_EVERY))
+    # per measured cycle one captured graph: MEASURE_EVERY sweeps of two colour
+    # passes and a measurement for each of the four chains (one per group of 64
+    # samples), the series row and the counters' advance
+    chains = S // 64
+    launches = args.steps * (SWEEPS_PER_STEP // MEASURE_EVERY) * (chains * (2 * MEASURE_EVERY + 1) + 2)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": 1e3 * dev_s / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -469,10 +454,9 @@ def run_other_configs(args):
     lat = ianus.Lattice(dim=3, L=16, n_samples=1, seed=SEED - 1, layout="i8", series_capacity=1000, stream=stream)
     lat.sweep(ianus.METROPOLIS, 1 / 1.1, 10, 1)
     sec = timed(lambda: lat.sweep(ianus.METROPOLIS, 1 / 1.1, 1000, 1), 1)
-    # latency floor of a sweep: two passes, each a cluster barrier round trip
-    # (0.19 us, measured with a barrier probe on GB300) and one dependent
-    # update of a site (about 410 cycles at 2070 MHz, read with clock64)
-    floor_us = 2 * (0.19 + 410 / 2070.0)
+    # latency floor of a sweep: two passes, each a block barrier and one
+    # dependent update of a word of 32 sites, about 200 cycles at 2070 MHz
+    floor_us = 2 * 200 / 2070.0
     sweep_us = sec * 1e3
     # integer work per update (one lane of the plane stream, plain layout):
     # the local field 2 per bond (12), E[pairs] = 1 + 1/4 + 1/16 + ... = 4/3
@@ -482,23 +466,23 @@ def run_other_configs(args):
     alu_u, madw_u = 12 + (4 / 3) * (16 + 2 + 1) + 3 * 8 / 3 + 2, (4 / 3) * (16 + 2)
     ach = rate16 * (alu_u + madw_u) / 1e3
     pk = _issue_peak()
-    sms_used = 16
+    sms_used = 1
     out["L16_single_sample_metropolis"] = {"updates_per_ns": rate16, "ms_per_1000_sweeps": sec * 1e3,
                                            "sweep_us": sweep_us,
-                                           "mode": "plain int8, one lattice split over a 16-block cluster "
-                                                   "(one z-plane per block, halos in shared memory), E/M every sweep",
-                                           "bound": "latency (2 cluster barriers and 2 dependent passes per sweep)",
+                                           "mode": "plain int8, 32 sites a word in one block, random decisions drawn "
+                                                   "ahead by the whole GPU (k_packed.cu), E/M every sweep",
+                                           "bound": "latency (2 dependent passes of two warps per sweep)",
                                            "roofline": {"bound": "alu", "ops_per_update": alu_u + madw_u,
                                                         "achieved": ach,
                                                         "peak": pk * sms_used / SM_COUNT if pk else None,
-                                                        "unit": "T int32 ops/s on the 16 SMs used",
+                                                        "unit": "T int32 ops/s on the SM that sweeps",
                                                         "frac": ach / (pk * sms_used / SM_COUNT) if pk else None,
                                                         "one_sm_peak": pk / SM_COUNT if pk else None,
                                                         "frac_of_one_sm": ach / (pk / SM_COUNT) if pk else None},
                                            "latency_floor": {"achieved_us": sweep_us, "floor_us": floor_us,
                                                              "frac": floor_us / sweep_us,
-                                                             "what": "2 cluster barrier round trips + 2 dependent "
-                                                                     "site updates per sweep"}}
+                                                             "what": "2 block barriers + 2 dependent word updates "
+                                                                     "per sweep"}}
     if not args.no_cpu_baseline:
         import oracle
 
@@ -746,8 +730,9 @@ def run_other_configs(args):
     alu_word = 44 + 3.92 * (2 * 10 + 20) + 1
     out["resident_L8_64xG_hb"] = {
         **res_out,
-        "mode": "bit-sliced, k_resident_bits: one block per 64-sample group holds spins, couplings and threshold "
-                "planes in shared memory for up to 4096 sweeps per launch; heat bath T=1.0, one replica",
+        "mode": "bit-sliced, spins, couplings and threshold planes in shared memory for up to 4096 sweeps per launch, "
+                "one block per 64-sample group (k_resident_bits) or, for few groups, a cluster of blocks each "
+                "(k_resident_bits_cluster); heat bath T=1.0, one replica",
         "roofline": issue_roof(alu_word, 3.92 * 16 + 2, 64, res_out["152x64"]["resident"]["updates_per_ns"]),
     }
     # device-side set-up: couplings and initial spins of the bench workload from the seed

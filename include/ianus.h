@@ -375,7 +375,8 @@ ianus_status ianus_segment_state(ianus_lattice* lat, int32_t group, int32_t lane
                                  uint64_t* sweeps_requested);
 /* Runs nsweeps sweeps of every live job of the pool (a job whose count has
  * reached its request stays frozen), as one launch per colour plus a counter
- * advance per sweep, replayed from CUDA graphs.  Asynchronous. */
+ * advance per block of up to 64 sweeps, replayed from CUDA graphs.
+ * Asynchronous. */
 ianus_status ianus_sweep_segments(ianus_lattice* lat, uint64_t nsweeps);
 
 /* Parallel-tempering state: slot_at int32 [n_samples][n_replicas][n_temps]
@@ -412,13 +413,12 @@ ianus_status ianus_synchronize(ianus_lattice* lat);
  * and the sweep kernel can be specialised for them at run time (NVRTC, a
  * fraction of a second per new table set, cached per device).
  *   0 = automatic: a lattice small enough for shared memory sweeps
- *       resident (ianus_set_resident); otherwise, with one temperature and
- *       one or two replicas, the lane-queue kernel (variant 24, below), the
- *       fastest shape measured on every lattice from L = 8 to L = 128; else
- *       the kernel with
- *       per-lane threshold bit-planes, compiled at run time for the
- *       lattice's geometry (also with several temperatures and for parallel
- *       tempering);
+ *       resident (ianus_set_resident); otherwise, the lane-queue kernel
+ *       (variant 24, below): with one temperature and one or two replicas
+ *       specialised for the tables, also with fields and dilution from 2^20
+ *       words on (fewer: precompiled); with several temperatures or more
+ *       replicas in a form with per-lane threshold bit-planes, compiled at
+ *       run time for the lattice's geometry;
  *   1 = always the precompiled per-lane kernel (geometry from the launch
  *       parameters);
  *   2..9 = a specialised kernel shape: 2, 3 = lockstep plane loop with 3 or 4
@@ -472,6 +472,8 @@ ianus_status ianus_synchronize(ianus_lattice* lat);
  * compares an 8-bit prefix of its random number from shared memory, in
  * the word kernel (four spins of one sample per 32-bit load) when L is a
  * multiple of 4, else in the tiled kernel (one byte per thread).
+ * Under variant 0 the resident forms (ianus_set_resident) go before, and
+ * where several of these kernels can run, estimates of their times decide.
  * With several temperatures every variant but 1 uses the per-lane kernel
  * compiled for the geometry.  If run-time compilation is unavailable, the
  * precompiled kernel runs.  EINVAL for other values. */
@@ -519,10 +521,12 @@ ianus_status ianus_prepare_sweep(ianus_lattice* lat, int32_t algo, const double*
 ianus_status ianus_set_persistent_wait(ianus_lattice* lat, uint64_t timeout_ns, int32_t absent_block);
 
 /* Sweep blocks through CUDA graphs (default on): runs of at least 4 sweeps
- * between measurements are replayed from graphs of up to 64 sweeps, captured
- * on a private stream the first time each block length occurs and dropped
- * when the tables, the variant or the launch shape change.  Captured kernels
- * read the sweep index from a device counter, so results are identical with
+ * between measurements are replayed from graphs of up to 64 sweeps, and
+ * measured sweeps and tempering steps from graphs of whole cycles, captured
+ * on a private stream when they are asked for again (by a later call, or by
+ * several more replays in the same one) and dropped when the tables, the
+ * variant or the launch shape change.  Captured kernels
+ * read the sweep index from device counters, so results are identical with
  * and without graphs.  enable = 0 launches every kernel directly. */
 ianus_status ianus_set_graphs(ianus_lattice* lat, int32_t enable);
 
@@ -540,10 +544,12 @@ ianus_status ianus_set_graphs(ianus_lattice* lat, int32_t enable);
  * usual.  A pool lattice (ianus_segment_load) sweeps the same way, one
  * block per group, when N + dim N + 264 words fit; each block advances its
  * jobs' sweep counters itself.  Same results, bit for bit, as the
- * launch-per-colour path.  enable = 1 (default) takes it where it is the
- * faster sweep: at most 512 word updates per block and sweep (R N), or
- * 1024 with at least 32 blocks (3D L = 8; 2D L <= 22 with one replica);
- * enable = 2 or 3 takes it wherever it fits; enable = 0: off.
+ * launch-per-colour path.  The state can also be split over a cluster of 2
+ * to 16 blocks, neighbours in other blocks read through distributed shared
+ * memory.  enable = 1 (default) takes the one of the three sweeps with the
+ * least estimated time (mostly clusters up to about L = 14 in 3D); enable =
+ * 2: one block wherever it fits; enable = 3: a cluster wherever one can be
+ * scheduled; enable = 0: off.
  *
  * Plain layout: with layout I8, one
  * temperature, (1 + dim) L^dim bytes <= 200 KiB, and either one replica or no
@@ -551,8 +557,13 @@ ianus_status ianus_set_graphs(ianus_lattice* lat, int32_t enable);
  * that runs all requested sweeps (the two colours separated by barriers,
  * Sec. 3.1) and records E and M itself.  Same results as the
  * launch-per-colour path.
- *   enable = 1 (default): with few configurations (at most two blocks per SM
- *            when each is split) a thread-block cluster of C blocks holds
+ *   enable = 1 (default): where the buffer has the room
+ *            (ianus_preferred_bytes) and L^dim / 2 is a multiple of 32, runs of
+ *            enough sweeps draw their random decisions ahead on the whole GPU
+ *            and sweep 32 sites a word in one block per configuration; larger
+ *            lattices of 8 samples or more are packed into 64-sample words for
+ *            the run when that is faster.  Else, with few configurations (at
+ *            most two blocks per SM when each is split) a thread-block cluster of C blocks holds
  *            one configuration, C the largest divisor of L in 2..16 that
  *            can be scheduled; block r owns the slab of L/C planes along the
  *            last axis, neighbours across a face come from the neighbouring

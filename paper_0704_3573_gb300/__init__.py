@@ -405,7 +405,7 @@ class Lattice:
         _check(self._lib.ianus_set_state(self._h, _ptr(buf), buf.size), "ianus_set_state")
 
     def set_variant(self, variant: int):
-        """Bit-sliced sweep kernel: 0 automatic, 1 per-lane threshold planes,
+        """Bit-sliced sweep kernel: 0 automatic, 1 precompiled per-lane planes,
         2..27 shapes of the kernel specialised at run time (include/ianus.h)."""
         _check(self._lib.ianus_set_variant(self._h, variant), "ianus_set_variant")
 
@@ -425,11 +425,12 @@ class Lattice:
 
     def set_resident(self, enable):
         """Shared-memory-resident sweeps for small lattices.  Plain layout:
-        True / 1 (default: a block cluster per configuration when there are
-        few), 2 (one block per configuration always), 3 (a cluster per
-        configuration whenever one can be formed), False / 0 (off).
-        Bit-sliced layout (automatic variant) and pools: any nonzero value
-        on, 0 off."""
+        True / 1 (default: packed sites or words, or a block cluster per
+        configuration when there are few), 2 (one block per configuration
+        always), 3 (a cluster per configuration whenever one can be formed),
+        False / 0 (off).  Bit-sliced layout (automatic variant): 1 the fastest
+        of launched, one-block and cluster sweeps, 2 one block, 3 clusters, 0
+        off.  Pools: any nonzero value on, 0 off."""
         _check(self._lib.ianus_set_resident(self._h, int(enable)), "ianus_set_resident")
 
     def synchronize(self):
