@@ -535,9 +535,10 @@ def run_other_configs(args):
     sec = timed(lambda: po.sweep(ianus.HEATBATH, 1 / 0.8, 100, 10), reps)
     upd = 128 * 2 * 32 ** 3 * 100 * reps
     rate = upd / (sec * 1e9)
-    # per 4-sample word: Philox 21 ALU; per sample 6 neighbours x (state,
-    # coupling, shift, add: 4) + 3 compares with "always" flags (6) + pack (3)
-    alu_word = 21 + 4 * (24 + 6 + 3)
+    # per 4-sample word: Philox rounds 2..9 16 + merge 3 (and 16 mad.wide); the
+    # counts of the 4 samples as bytes of one word, 4 ops a neighbour; table rows
+    # 8; per sample 3 compares and selects (6) + pack (1)
+    alu_word = 19 + 6 * 4 + 8 + 4 * 7
     upd_launch = 128 * 2 * 32 ** 3 // 2
     potts_traffic = None
     if kernel_source_hash(("common.cuh", "k_potts.cu")) == POTTS_SOURCE_HASH:
@@ -548,7 +549,7 @@ def run_other_configs(args):
     out["potts_L32_128x2"] = {
         "updates_per_ns": rate, "ms_per_100_sweeps": sec * 1e3 / reps,
         "mode": "4 samples per uint32 word, heat bath, E/Q every 10 sweeps",
-        "roofline": issue_roof(alu_word, 20, 4, rate),
+        "roofline": issue_roof(alu_word, 16, 4, rate),
         "table_traffic_per_launch": potts_traffic,
     }
     if not args.no_cpu_baseline:
@@ -684,14 +685,14 @@ def run_other_configs(args):
         sec = timed(lambda: pp.sweep(ianus.HEATBATH, bp, 100, 10), reps)
         upd = 256 * 2 * Lp ** dim * 100 * reps
         rate = upd / (sec * 1e9)
-        # per 4-sample word: Philox 21; per sample and bond ~7 (state and code
-        # fields, target state, nibble increment), table index 4, selection 6,
-        # pack 2
-        alu_word = 21 + 4 * (2 * dim * 7 + 12)
+        # per 4-sample word: Philox 19 (and 16 mad.wide); per bond 7 for the 4
+        # samples at once (target states by byte permutes, counts); table rows 8;
+        # per sample selection 6, pack 1
+        alu_word = 19 + 2 * dim * 7 + 8 + 4 * 7
         out[key] = {
             "updates_per_ns": rate, "ms_per_100_sweeps": sec * 1e3 / reps,
             "mode": f"4 samples per uint32 word, {dim}D, heat bath beta={bp}, E/Q every 10 sweeps",
-            "roofline": issue_roof(alu_word, 20, 4, rate),
+            "roofline": issue_roof(alu_word, 16, 4, rate),
         }
         if not args.no_cpu_baseline:
             import oracle
