@@ -2046,7 +2046,8 @@ PlainChoice plain_choice(const Lattice& lat) {
   const double shared = 6.0 + 1.1 * std::min(lat.S, 8) + k / 150.0;
   if (shared < best.us) best = PlainChoice{PlainPath::kShared, shared};
   if (i8_sliced_fits(lat)) {
-    const double sliced = (lat.L == 128 ? 16.0 : lat.D == 2 ? 8.5 : 12.0) + k / 400.0;
+    // the tiles of a part-filled group take as long as of a full one
+    const double sliced = (lat.L == 128 ? 16.0 : lat.D == 2 ? 8.5 : 12.0) + k / 400.0 * (64.0 * lat.G / lat.S);
     if (sliced < best.us) best = PlainChoice{PlainPath::kSliced, sliced};
   }
   return best;
