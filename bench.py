@@ -466,7 +466,7 @@ def run_other_configs(args):
     alu_u, madw_u = 12 + (4 / 3) * (16 + 2 + 1) + 3 * 8 / 3 + 2, (4 / 3) * (16 + 2)
     ach = rate16 * (alu_u + madw_u) / 1e3
     pk = _issue_peak()
-    sms_used = 1
+    sms_used = SM_COUNT  # the random decisions are drawn on all of them
     out["L16_single_sample_metropolis"] = {"updates_per_ns": rate16, "ms_per_1000_sweeps": sec * 1e3,
                                            "sweep_us": sweep_us,
                                            "mode": "plain int8, 32 sites a word in one block, random decisions drawn "
@@ -475,10 +475,8 @@ def run_other_configs(args):
                                            "roofline": {"bound": "alu", "ops_per_update": alu_u + madw_u,
                                                         "achieved": ach,
                                                         "peak": pk * sms_used / SM_COUNT if pk else None,
-                                                        "unit": "T int32 ops/s on the SM that sweeps",
-                                                        "frac": ach / (pk * sms_used / SM_COUNT) if pk else None,
-                                                        "one_sm_peak": pk / SM_COUNT if pk else None,
-                                                        "frac_of_one_sm": ach / (pk / SM_COUNT) if pk else None},
+                                                        "unit": "T int32 ops/s",
+                                                        "frac": ach / (pk * sms_used / SM_COUNT) if pk else None},
                                            "latency_floor": {"achieved_us": sweep_us, "floor_us": floor_us,
                                                              "frac": floor_us / sweep_us,
                                                              "what": "2 block barriers + 2 dependent word updates "
