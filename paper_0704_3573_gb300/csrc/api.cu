@@ -560,11 +560,19 @@ int build_graph(Lattice* lat, int inv, uint32_t B, uint32_t cycles, Swap swap, c
       if (e == cudaSuccess)
         e = lat->layout == IANUS_LAYOUT_I8 ? launch_measure_i8(*lat, q) : launch_measure_potts(*lat, q);
       lat->chains = chains;
-      if (n + 1 < cycles)
-        for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+      // the next cycle's sweeps read the spins only after the measurement has,
+      // and the temperatures only after the swap step has written them
+      auto go_on = [&]() {
+        if (n + 1 < cycles)
+          for (int k = 1; k < chains; ++k) after(stream_of(k), main);
+      };
+      if (swap == Swap::kNone) go_on();
       if (e == cudaSuccess && swap != Swap::kOnly)
         e = launch_finalize_row(*lat, n, (uint64_t)(n + 1) * B, want_q);
-      if (e == cudaSuccess && swap != Swap::kNone) e = launch_pt_swap(*lat, n);
+      if (swap != Swap::kNone) {
+        if (e == cudaSuccess) e = launch_pt_swap(*lat, n);
+        go_on();
+      }
     }
   }
   lat->stream = main;
