@@ -1,0 +1,40 @@
+"""Plain lattices at the limits of their sweep in words (k_words.cu): many
+replicas, rows beyond a launch's limit, a buffer without the room.  Integer
+work: bit-exact against the plain kernels."""
+
+import ctypes as C
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SEED = 0x0704357300001800
+
+
+def _pair(ianus, **kw):
+    a, b = (ianus.Lattice(layout="i8", seed=SEED, series_capacity=8, **kw) for _ in range(2))
+    b.set_resident(0)
+    return a, b
+
+
+def _words_used(ianus, lat):
+    """Whether a sweep since the room was cleared wrote the words."""
+    return bool(lat.buffer[lat._lib.ianus_required_bytes(C.byref(lat.cfg)):].any())
+
+
+def _equal(a, b):
+    assert np.array_equal(a.spins(), b.spins())
+    for x, y in zip(a.series(), b.series()):
+        assert (x is None and y is None) or np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("L,S,R,words", [(40, 8, 128, False), (16, 64, 128, False), (16, 64, 110, True)])
+def test_many_replicas(ianus, L, S, R, words):
+    a, b = _pair(ianus, dim=3, L=L, n_samples=S, n_replicas=R)
+    a.buffer[a._lib.ianus_required_bytes(C.byref(a.cfg)):].zero_()
+    for algo, n, every in (("heatbath", 2, 0), ("metropolis", 4, 1), ("heatbath", 12, 5)):
+        for lat in (a, b):
+            lat.sweep(algo, 0.8, n, every)
+    assert _words_used(ianus, a) == words
+    _equal(a, b)
