@@ -153,11 +153,12 @@ int plan(const ianus_config* c, Sizes& z) {
                      : 0;
   z.off_masks = take(z.mask_bytes);
   // the same lattice in words: from 8 samples on, at most 2 GiB, replicas whose
-  // threshold planes fit one block of the word sweep (up to 110)
+  // threshold planes fit one block of the word sweep (up to 110), and no more
+  // (group, replica) rows than a launch of the measurement takes
   const size_t wspins = (size_t)z.G * z.slots * z.N * 8, wJ = (size_t)z.G * z.D * z.N * 8;
   const size_t wtp = (size_t)z.G * z.slots * kPlanes * kMaxClasses * 8;
   z.words = layout == IANUS_LAYOUT_I8 && !field && c->rng == IANUS_RNG_PHILOX && z.K == 1 && z.S >= 8 &&
-            sweep_bits_smem(z.R) <= kMaxSmemPerBlock && wspins + wJ + wtp <= (size_t)2 << 30;
+            sweep_bits_smem(z.R) <= kMaxSmemPerBlock && (z.R <= 2 || (size_t)z.G * z.slots <= 65535) && wspins + wJ + wtp <= (size_t)2 << 30;
   z.off_wspins = take(z.words ? wspins : 0);
   z.off_wJ = take(z.words ? wJ : 0);
   z.off_wtp = take(z.words ? wtp : 0);

@@ -38,3 +38,13 @@ def test_many_replicas(ianus, L, S, R, words):
             lat.sweep(algo, 0.8, n, every)
     assert _words_used(ianus, a) == words
     _equal(a, b)
+
+
+@pytest.mark.parametrize("R,words", [(17, False), (16, True), (2, True)])
+def test_many_rows(ianus, R, words):
+    a, b = _pair(ianus, dim=3, L=4, n_samples=64 * 4095, n_replicas=R)
+    a.buffer[a._lib.ianus_required_bytes(C.byref(a.cfg)):].zero_()
+    for lat in (a, b):
+        lat.sweep("heatbath", 0.8, 6, 3)
+    assert _words_used(ianus, a) == words
+    _equal(a, b)

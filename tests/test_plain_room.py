@@ -23,3 +23,11 @@ def test_no_words_beyond_the_replicas_their_sweep_takes():
     assert _words_room(40, 8, 111) == 0
     assert _words_room(16, 64, 128) == 0
     assert _words_room(16, 64, 4000) == 0
+
+
+def test_no_words_beyond_the_rows_their_measurement_takes():
+    """The counts of three replicas and more are launched with a row of blocks
+    per (group, replica), 65535 at most; one or two replicas are a row a group."""
+    assert _words_room(4, 64 * 4095, 16) > 0
+    assert _words_room(4, 64 * 4095, 17) == 0
+    assert _words_room(4, 64 * 4095, 2) > 0
