@@ -1116,17 +1116,19 @@ static ianus_status sweep_words(Lattice* lat, int32_t algo, const double* beta, 
   w->t_dev_valid = false;
   w->acc_ok = false;
   w->calls += 1;
+  w->sticky = 0;
   const ianus_status st = sweep_run(w, algo, beta, nsweeps, measure_every, 1);
-  lat->sweeps = w->sweeps;
-  lat->ser_count = w->ser_count;
   lat->t_dev_valid = false;
   lat->acc_ok = false;
-  if (st) {
+  if (w->sticky) {  // a refused launch inside a sweep: the state is lost
     lat->sticky = w->sticky;
     return st;
   }
+  // also after a capture that failed: the words hold the sweeps counted so far
   CK(launch_unpack_spins(*lat));
-  return IANUS_OK;
+  lat->sweeps = w->sweeps;
+  lat->ser_count = w->ser_count;
+  return st;
 }
 
 ianus_status ianus_sweep(ianus_lattice* h, int32_t algo, const double* beta, uint64_t nsweeps,

@@ -12,7 +12,7 @@ import paper_0704_3573_gb300 as ianus
 from paper_0704_3573_gb300 import build as b
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CUDA_OK, STATE = 0, 6
+ECUDA, ESTATE = 3, 6
 
 
 @pytest.fixture(scope="module")
@@ -106,3 +106,36 @@ def test_swaps_are_ordered_against_every_sweep(fake, lattice, layout, measured, 
                     assert m in before, (name, n, "does not wait for", other, m)
                 elif other in ("sweep", "sweep_bits") and m > n:
                     assert n in theirs, (other, m, "does not wait for", name, n)
+
+
+def sweeps_done(lib, h):
+    n = C.c_uint64()
+    assert lib.ianus_get_sweeps(h, C.byref(n)) == 0
+    return n.value
+
+
+def test_a_capture_that_fails_in_words_leaves_spins_and_counters_together(fake, lattice):
+    """2 sweeps, then 23 with measurements: 3 + 5 of those run before the capture of
+    the rest is refused.  The bytes get the 8, and the lattice goes on."""
+    h = lattice()
+    fake.fake_set(b"words", 1)
+    assert fake.ianus_sweep(h, 0, betas(1), 2, 0) == 0
+    fake.fake_forget()
+    fake.fake_set(b"fail_capture", 1)
+    assert fake.ianus_sweep(h, 0, betas(1), 23, 5) == ECUDA
+    names = [o[1] for o in record(fake)]
+    assert names.count("sweep_bits") == 2 * 8 and sweeps_done(fake, h) == 10
+    assert names[-1] == "unpack_spins"
+    fake.fake_forget()
+    assert fake.ianus_sweep(h, 0, betas(1), 15, 5) == 0
+    names = [o[1] for o in record(fake)]
+    assert "capture" in names and sweeps_done(fake, h) == 25
+    assert names.index("pack_spins") < names.index("capture") and names[-1] == "unpack_spins"
+
+
+def test_a_launch_refused_in_words_closes_the_lattice(fake, lattice):
+    h = lattice()
+    fake.fake_set(b"words", 1)
+    fake.fake_set(b"fail_sweep", 3)
+    assert fake.ianus_sweep(h, 0, betas(1), 3, 0) == ECUDA
+    assert fake.ianus_sweep(h, 0, betas(1), 3, 0) == ESTATE
