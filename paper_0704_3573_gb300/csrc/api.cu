@@ -1719,6 +1719,8 @@ ianus_status ianus_set_graphs(ianus_lattice* h, int32_t enable) {
 ianus_status ianus_set_resident(ianus_lattice* h, int32_t enable) {
   GET_LAT(h);
   if (enable < 0 || enable > 3) return IANUS_EINVAL;
+  // captured cycles hold the resident sweep that was chosen for them
+  if (lat->use_resident != (enable != 0) || (enable && lat->resident_mode != enable)) drop_graphs(lat);
   lat->use_resident = enable != 0;
   if (enable) lat->resident_mode = enable;
   return IANUS_OK;

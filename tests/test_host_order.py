@@ -139,3 +139,23 @@ def test_a_launch_refused_in_words_closes_the_lattice(fake, lattice):
     fake.fake_set(b"fail_sweep", 3)
     assert fake.ianus_sweep(h, 0, betas(1), 3, 0) == ECUDA
     assert fake.ianus_sweep(h, 0, betas(1), 3, 0) == ESTATE
+
+
+@pytest.mark.parametrize("layout", [1, 2])
+def test_a_resident_mode_reaches_captured_cycles(fake, lattice, layout):
+    """Cycles captured under one mode are not replayed under another; setting the
+    mode that is set keeps them."""
+    h = lattice(layout=layout)
+
+    def replays():
+        fake.fake_forget()
+        assert fake.ianus_sweep(h, 0, betas(1), 10, 5) == 0
+        return [o[1] for o in record(fake)].count("graph")
+
+    for _ in range(3):
+        before = replays()
+    assert before > 0
+    assert fake.ianus_set_resident(h, 1) == 0 and replays() == before
+    for mode in (0, 2, 3, 1):
+        assert fake.ianus_set_resident(h, mode) == 0 and replays() == 0
+        assert replays() + replays() > 0
