@@ -1104,10 +1104,7 @@ static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, ui
 static ianus_status sweep_words(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
                                 uint32_t measure_every) {
   Lattice* w = lat->words;
-  if (lat->words_mut != lat->mut + 1) {
-    CK(launch_pack_couplings(*lat));
-    lat->words_mut = lat->mut + 1;
-  }
+  CK(launch_pack_couplings(*lat));
   CK(launch_pack_spins(*lat));
   w->use_graphs = lat->use_graphs;
   w->sweeps = lat->sweeps;

@@ -3,9 +3,10 @@
 //
 // A plain sweep moves and counts one byte a spin; the bit-sliced one updates 64
 // samples with each instruction, from the same random numbers.  A run of sweeps
-// of a plain lattice therefore packs the spins into words, sweeps those
-// (api.cu, sweep_words) and unpacks them: two passes over the bytes for the run
-// instead of two for every sweep.  The couplings are packed when they changed.
+// of a plain lattice therefore packs the spins and the couplings into words,
+// sweeps those (api.cu, sweep_words) and unpacks the spins: three passes over
+// bytes for the run instead of several for every sweep.  Nothing is kept from
+// one run to the next, since a program may write either in the lattice's buffer.
 //
 // The sweep is the precompiled per-lane-plane kernel, which needs no run-time
 // compiler for a new temperature.  us per colour pass, 3D, heat bath (plain /

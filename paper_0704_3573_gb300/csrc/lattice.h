@@ -184,7 +184,6 @@ struct Lattice {
   uint4* masks;              // packed resident sweeps (k_packed.cu): a run's random decisions; null: not used
   size_t mask_bytes;
   Lattice* words;            // the same lattice in words (k_words.cu); null: not used
-  uint64_t words_mut;        // mut + 1 when its couplings were packed
 };
 
 // ---- host table builders (tables.cpp) ----

@@ -48,3 +48,26 @@ def test_many_rows(ianus, R, words):
         lat.sweep("heatbath", 0.8, 6, 3)
     assert _words_used(ianus, a) == words
     _equal(a, b)
+
+
+def test_couplings_written_in_the_buffer(ianus):
+    """Spins and couplings changed in place, without a call, between two runs."""
+    import torch
+
+    a, b = _pair(ianus, dim=3, L=32, n_samples=70, n_replicas=2)
+    nspins, ncouplings = 70 * 2 * 32 ** 3, 70 * 3 * 32 ** 3
+    at = (nspins + 255) // 256 * 256
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    a.buffer[a._lib.ianus_required_bytes(C.byref(a.cfg)):].zero_()
+    for run in range(3):
+        signs = torch.randint(0, 2, (ncouplings,), generator=gen, device="cuda", dtype=torch.int8) * 2 - 1
+        flips = torch.randint(0, 2, (nspins,), generator=gen, device="cuda", dtype=torch.int8) * 2 - 1
+        for lat in (a, b):
+            lat.sweep("heatbath", 0.9, 20, 5)
+            lat.buffer[at:at + ncouplings].view(torch.int8).mul_(signs)
+            lat.buffer[:nspins].view(torch.int8).mul_(flips)
+    for lat in (a, b):
+        lat.sweep("heatbath", 0.9, 20, 5)
+    assert _words_used(ianus, a)
+    assert np.array_equal(a.couplings(), b.couplings())
+    _equal(a, b)

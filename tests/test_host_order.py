@@ -159,3 +159,14 @@ def test_a_resident_mode_reaches_captured_cycles(fake, lattice, layout):
     for mode in (0, 2, 3, 1):
         assert fake.ianus_set_resident(h, mode) == 0 and replays() == 0
         assert replays() + replays() > 0
+
+
+def test_every_run_in_words_packs_spins_and_couplings(fake, lattice):
+    """Both may have been written in the lattice's buffer since the last run."""
+    h = lattice()
+    fake.fake_set(b"words", 1)
+    for _ in range(3):
+        fake.fake_forget()
+        assert fake.ianus_sweep(h, 0, betas(1), 20, 0) == 0
+        names = [o[1] for o in record(fake)]
+        assert {"pack_spins", "pack_couplings"} <= set(names[:4]) and names[-1] == "unpack_spins"
