@@ -817,21 +817,25 @@ int read_back(Lattice* lat, const Read* reads, int n) {
   Part parts[8];
   int np = 0;
   size_t used = 0;
-  for (int i = 0; i < n; ++i) {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
     const Read& r = reads[i];
     if (!r.dst || !r.bytes) continue;
     const bool paged = pageable(r.dst);
     if (pin && paged && r.bytes <= kStagedMost && used + r.bytes <= kPinnedBytes && np < 8) {
-      CK(cudaMemcpyAsync(pin + used, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream));
+      e = cudaMemcpyAsync(pin + used, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream);
       parts[np++] = Part{r.dst, used, r.bytes};
       used += (r.bytes + 63) & ~(size_t)63;
       continue;
     }
     if (paged && r.bytes > kStagedMost)
       for (size_t o = 0; o < r.bytes; o += kPage) ((volatile uint8_t*)r.dst)[o] = 0;
-    CK(cudaMemcpyAsync(r.dst, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream));
+    e = cudaMemcpyAsync(r.dst, r.src, r.bytes, cudaMemcpyDeviceToHost, lat->stream);
   }
-  CK(cudaStreamSynchronize(lat->stream));
+  // also after a refused copy: the ones before it write the block until they are done
+  const cudaError_t waited = cudaStreamSynchronize(lat->stream);
+  CK(e);
+  CK(waited);
   for (int k = 0; k < np; ++k) std::memcpy(parts[k].dst, pin + parts[k].at, parts[k].bytes);
   return IANUS_OK;
 }

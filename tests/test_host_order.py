@@ -170,3 +170,16 @@ def test_every_run_in_words_packs_spins_and_couplings(fake, lattice):
         assert fake.ianus_sweep(h, 0, betas(1), 20, 0) == 0
         names = [o[1] for o in record(fake)]
         assert {"pack_spins", "pack_couplings"} <= set(names[:4]) and names[-1] == "unpack_spins"
+
+
+@pytest.mark.parametrize("nth", [1, 2, 3])
+def test_a_refused_read_waits_for_the_copies_before_it(fake, lattice, nth):
+    """The page-locked block that small results pass through goes to other calls
+    only when no copy writes it any more."""
+    h = lattice(S=8, R=2)
+    out = [(C.c_int64 * 16)() for _ in range(3)]
+    fake.fake_set(b"fail_read", nth)
+    assert fake.ianus_measure(h, *out) == ECUDA
+    names = [o[1] for o in record(fake)]
+    assert names.count("read") == nth - 1 and names[-1] == "synchronize"
+    assert fake.ianus_measure(h, *out) == ESTATE
