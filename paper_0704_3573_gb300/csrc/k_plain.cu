@@ -504,6 +504,30 @@ struct WheelWarp {
   uint64_t T[kFieldClasses];
 };
 
+// Row of T for the sum v of a site's bond terms, -2D .. 2D, with f = [s h > 0]
+// in the field models.  Spin bytes that are not +-1 (a program may write the
+// lattice's buffer) give other sums; they get the last row, never one past it.
+template <int D, bool FIELD>
+__host__ __device__ constexpr uint32_t wheel_row(int v, int f) {
+  const uint32_t row = FIELD ? (uint32_t)((v + 2 * D) * 2 + f) : (uint32_t)(2 * D - v) >> 1;
+  const uint32_t last = (FIELD ? kFieldClasses : kMaxClasses) - 1;
+  return row < last ? row : last;
+}
+
+template <int D, bool FIELD>
+constexpr bool wheel_rows_hold() {
+  for (int v = -2 * D * 128; v <= 2 * D * 128; ++v)
+    for (int f = 0; f < 2; ++f) {
+      const uint32_t row = wheel_row<D, FIELD>(v, f);
+      if (row >= (uint32_t)(FIELD ? kFieldClasses : kMaxClasses)) return false;
+      if (v >= -2 * D && v <= 2 * D && (int)row != (FIELD ? (v + 2 * D) * 2 + f : (2 * D - v) >> 1)) return false;
+    }
+  return true;
+}
+static_assert(wheel_rows_hold<2, false>() && wheel_rows_hold<3, false>() && wheel_rows_hold<2, true>() &&
+                  wheel_rows_hold<3, true>(),
+              "a wheel sweep's threshold row");
+
 // Words of kWheelUnroll items of one warp's rows: see k_sweep_wheel_i8 (W).
 // Bits 1..7 of a +-1 byte all equal its sign, so the class u = (u2 u1 u0) of a
 // byte can be read off any three of them: bits 3, 4, 5 give 8 u, the byte
@@ -718,7 +742,7 @@ __global__ void __launch_bounds__(32 * kWheelWarps, FIELD ? 6 : 8) k_sweep_wheel
 #pragma unroll
         for (int c = 0; c < kWheelUnroll; ++c) {
           if (!live[c]) continue;
-          const uint64_t T = w.T[FIELD ? (v[c] + 2 * D) * 2 + f[c] : (2 * D - v[c]) >> 1];
+          const uint64_t T = w.T[wheel_row<D, FIELD>(v[c], f[c])];
           const bool less = (uint64_t)rr[c] < T;
           if (less != (p.inv != 0)) sp[ix[c]] = (int8_t)(-si[c]);
         }
