@@ -1244,8 +1244,9 @@ template <int D, int ALGO, int RT, bool P2, bool Q>
 cudaError_t sweep_launch(Lattice& lat, const BitsParams& p, dim3 grid) {
   const size_t smem = bits_sweep_smem(lat.R, Q);
   if (smem > 48 * 1024) {  // many replicas: opt in to more than 48 KiB of planes and queues
+    // the most that any lattice needs: other threads may be launching theirs
     cudaError_t e = cudaFuncSetAttribute(k_sweep_bits<D, ALGO, RT, P2, Q>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
   }
   k_sweep_bits<D, ALGO, RT, P2, Q><<<grid, kBlock, smem, lat.stream>>>(p);

@@ -71,3 +71,37 @@ def test_couplings_written_in_the_buffer(ianus):
     assert _words_used(ianus, a)
     assert np.array_equal(a.couplings(), b.couplings())
     _equal(a, b)
+
+
+def test_threads_with_different_replicas(ianus):
+    """Two threads whose word sweeps ask for different amounts of shared memory."""
+    import threading
+
+    import torch
+
+    pairs, failed = [], []
+    for R in (108, 28):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            pairs.append(_pair(ianus, dim=3, L=8, n_samples=200, n_replicas=R))
+
+    def run(lat):
+        try:
+            for _ in range(60):
+                lat.sweep("metropolis", 0.8, 20)
+        except Exception as e:
+            failed.append(e)
+
+    for a, _ in pairs:
+        a.set_graphs(False)
+        a.buffer[a._lib.ianus_required_bytes(C.byref(a.cfg)):].zero_()
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=run, args=(a,)) for a, _ in pairs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    for a, b in pairs:
+        run(b)
+        assert _words_used(ianus, a)
+        _equal(a, b)
