@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kBlock) k_measure(const MeasParams p) {
   // per warp and sample: sites, overlap, then good, bad, lo, hi, both of each
   // replica; the block's sums by one thread per (replica, sample) and value
   constexpr int NV = 2 + 5 * RT;
-  __shared__ int red[kBlock / 32][NV][4];
+  __shared__ __align__(16) int red[kBlock / 32][NV][4];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   {
     int v[NV][4];
