@@ -248,9 +248,15 @@ typedef struct {
  * tables, series).  Returns 0 for an invalid configuration.  Host only. */
 size_t ianus_required_bytes(const ianus_config* cfg);
 
-/* The same with the room that its fastest sweep uses (small plain lattices: up
- * to 8 MiB of random decisions drawn ahead).  A device buffer between the two
- * sizes is used without it; the results do not depend on it.  Host only. */
+/* The same with the room that its fastest sweeps use: for plain lattices of one
+ * temperature, without fields, on the Philox stream, up to 8 MiB of random
+ * decisions drawn ahead (small lattices), and with 8 samples or more and up to
+ * 110 replicas the lattice in 64-sample words beside its bytes (8 bytes a site
+ * for each 64 samples begun, replica and dimension, at most 2 GiB; with 8
+ * samples as much again as the bytes).  The lattices of a process hold up to
+ * 8 GiB of such room; beyond that, and for all other lattices, this is
+ * ianus_required_bytes.  A device buffer below this size is used as one of
+ * ianus_required_bytes.  The results do not depend on it.  Host only. */
 size_t ianus_preferred_bytes(const ianus_config* cfg);
 
 /* Validates cfg, takes device memory (cfg->device_buffer if non-NULL, which

@@ -4,6 +4,7 @@
 // uploads (Sec. 3.2), measurements (Sec. 4.1), parallel tempering,
 // checkpoints and error reporting.  Host logic only; all per-site work runs
 // in the kernels of k_plain.cu, k_msc.cu, k_potts.cu and k_pt.cu.
+#include <atomic>
 #include <cmath>
 #include <functional>
 #include <cstdlib>
@@ -840,6 +841,15 @@ int read_back(Lattice* lat, const Read* reads, int n) {
   return IANUS_OK;
 }
 
+// What a lattice's buffer holds beyond its least only makes sweeps faster, and it
+// can double a plain lattice of few samples.  The lattices of a process take up
+// to kRoomMost of it, 3 % of the memory, so that a program whose lattices fill
+// the GPU fits as it did without; the ones made after that do without.
+constexpr size_t kRoomMost = (size_t)8 << 30;
+std::atomic<size_t> room_held{0};
+
+size_t wanted_bytes(const Sizes& z) { return z.total - z.least + room_held <= kRoomMost ? z.total : z.least; }
+
 }  // namespace
 
 extern "C" {
@@ -853,7 +863,7 @@ size_t ianus_required_bytes(const ianus_config* cfg) {
 size_t ianus_preferred_bytes(const ianus_config* cfg) {
   Sizes z;
   if (plan(cfg, z) != IANUS_OK) return 0;
-  return z.total;
+  return wanted_bytes(z);
 }
 
 ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) {
@@ -909,7 +919,7 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
   lat->jitf_algo = -1;
   lat->mut = 0;
   lat->acc_ok = false;
-  lat->bytes = cfg->device_buffer && cfg->device_buffer_bytes < z.total ? z.least : z.total;
+  lat->bytes = !cfg->device_buffer ? wanted_bytes(z) : cfg->device_buffer_bytes < z.total ? z.least : z.total;
   if (cfg->device_buffer) {
     if (cfg->device_buffer_bytes < z.least || ((uintptr_t)cfg->device_buffer & 255u)) {
       delete lat;
@@ -919,8 +929,8 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
     lat->owns_buffer = false;
   } else {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, z.total);
-    if (e == cudaErrorMemoryAllocation && z.least < z.total) {
+    cudaError_t e = cudaMalloc(&p, lat->bytes);
+    if (e == cudaErrorMemoryAllocation && z.least < lat->bytes) {
       cudaGetLastError();
       lat->bytes = z.least;
       e = cudaMalloc(&p, z.least);
@@ -1032,6 +1042,8 @@ ianus_status ianus_lattice_create(const ianus_config* cfg, ianus_lattice** out) 
       w->graphs = new (std::nothrow) std::map<uint32_t, GraphSlot>();
     }
   }
+  lat->room = lat->bytes - z.least;
+  room_held += lat->room;
   *out = reinterpret_cast<ianus_lattice*>(lat);
   return IANUS_OK;
 }
@@ -1747,6 +1759,7 @@ ianus_status ianus_destroy(ianus_lattice* h) {
   if (lat->cap_stream) cudaStreamDestroy(lat->cap_stream);
   for (cudaStream_t s : lat->side_streams)
     if (s) cudaStreamDestroy(s);
+  room_held -= lat->room;
   if (lat->owns_buffer) cudaFree(lat->base);
   delete lat;
   return IANUS_OK;

@@ -183,6 +183,7 @@ struct Lattice {
   uint64_t calls;            // sweep calls so far
   uint4* masks;              // packed resident sweeps (k_packed.cu): a run's random decisions; null: not used
   size_t mask_bytes;
+  size_t room;               // bytes of the buffer beyond the least
   Lattice* words;            // the same lattice in words (k_words.cu); null: not used
 };
 

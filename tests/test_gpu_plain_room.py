@@ -105,3 +105,27 @@ def test_threads_with_different_replicas(ianus):
         run(b)
         assert _words_used(ianus, a)
         _equal(a, b)
+
+
+@pytest.mark.parametrize("short", [0, 1])
+def test_a_buffer_without_room_for_the_words(ianus, short):
+    """The least buffer, and one byte less than the preferred, sweep by bytes."""
+    import torch
+
+    a, b = _pair(ianus, dim=3, L=32, n_samples=70, n_replicas=2)
+    lib = a._lib
+    cfg = type(a.cfg)()
+    C.memmove(C.byref(cfg), C.byref(a.cfg), C.sizeof(cfg))
+    least, most = lib.ianus_required_bytes(C.byref(cfg)), lib.ianus_preferred_bytes(C.byref(cfg))
+    size = most - 1 if short else least
+    buf = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    cfg.device_buffer, cfg.device_buffer_bytes = buf.data_ptr(), size
+    h = C.c_void_p()
+    assert lib.ianus_lattice_create(C.byref(cfg), C.byref(h)) == 0
+    beta = (C.c_double * 1)(0.9)
+    assert lib.ianus_sweep(h, 1, beta, 30, 0) == 0
+    b.sweep("heatbath", 0.9, 30)
+    out = np.empty(b.spins().shape, dtype=np.int8)
+    assert lib.ianus_get_spins_i8(h, out.ctypes.data) == 0
+    assert np.array_equal(out, b.spins()) and not buf[least:].any()
+    lib.ianus_destroy(h)

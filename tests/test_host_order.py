@@ -57,6 +57,11 @@ def lattice(fake):
         fake.fake_forget()
         return h
 
+    def destroy(h):
+        made.remove(h)
+        fake.ianus_destroy(h)
+
+    make.destroy = destroy
     yield make
     for h in made:
         fake.ianus_destroy(h)
@@ -183,3 +188,31 @@ def test_a_refused_read_waits_for_the_copies_before_it(fake, lattice, nth):
     names = [o[1] for o in record(fake)]
     assert names.count("read") == nth - 1 and names[-1] == "synchronize"
     assert fake.ianus_measure(h, *out) == ESTATE
+
+
+def test_the_room_beyond_the_least_is_bounded_and_given_back(fake, lattice):
+    """Lattices that fill the GPU's memory still fit: those of a process take 8 GiB
+    at most beyond what they need."""
+    kw = dict(L=128, S=8, R=100, rows=1)  # 1.7 GB of words each
+    fake.fake_set(b"words", 1)
+
+    def room():
+        c = config(**kw)
+        return fake.ianus_preferred_bytes(C.byref(c)) - fake.ianus_required_bytes(C.byref(c))
+
+    def in_words(h):
+        fake.fake_forget()
+        assert fake.ianus_sweep(h, 0, betas(1), 2, 0) == 0
+        return "pack_spins" in [o[1] for o in record(fake)]
+
+    each = room()
+    assert each > 1.6e9
+    held = [lattice(**kw) for _ in range((8 << 30) // each)]
+    assert all(in_words(h) for h in held)
+    assert room() == 0
+    late = [lattice(**kw) for _ in range(2)]
+    assert not any(in_words(h) for h in late)
+    lattice.destroy(late.pop(0))  # held none: gives none back
+    assert room() == 0
+    lattice.destroy(held.pop())
+    assert room() == each and in_words(lattice(**kw)) and room() == 0
