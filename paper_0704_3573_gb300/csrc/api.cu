@@ -1120,8 +1120,7 @@ static ianus_status sweep_run(Lattice* lat, int32_t algo, const double* beta, ui
 static ianus_status sweep_words(Lattice* lat, int32_t algo, const double* beta, uint64_t nsweeps,
                                 uint32_t measure_every) {
   Lattice* w = lat->words;
-  CK(launch_pack_couplings(*lat));
-  CK(launch_pack_spins(*lat));
+  CK(launch_pack_words(*lat));
   w->use_graphs = lat->use_graphs;
   w->sweeps = lat->sweeps;
   w->ser_count = lat->ser_count;

@@ -13,8 +13,10 @@
 // words): L=64, 256 samples x 2 149 / 38; L=40, 100 x 2 33 / 8.7; L=100, 64 x 2
 // 288 / 39; L=16, 256 x 2 10.2 / 6.1; L=24, 20 samples 8.2 / 4.5.
 //
-// Bound: HBM, a byte and an eighth a spin: 134 M spins 46 us with sixteen loads
-// under way a thread (121 one by one).
+// Bound: HBM, a byte and an eighth a spin or coupling.  L=64, 256 x 2: packing 134 M
+// spins and 201 M couplings 75 us in one launch of 4 bytes a thread and sample,
+// sixteen loads under way (5 TB/s; 46 + 66 us in two launches of 2 bytes),
+// unpacking the spins 44 us.
 #include <algorithm>
 
 #include "lattice.h"
@@ -23,12 +25,17 @@ namespace ianus {
 
 namespace {
 
-struct WordsParams {
+// Bytes and words of the spins or the couplings.
+struct WordsPart {
   int8_t* bytes;    // sample s, unit u: s sample_stride + u unit_stride + site
   uint64_t* words;  // [G][units][N], split layout
   uint64_t sample_stride, unit_stride;
-  Geom geom;
   uint32_t units;   // slots or dimensions
+};
+
+struct WordsParams {
+  WordsPart part[2];  // spins, couplings: blockIdx.y counts the units of both
+  Geom geom;
   int S;
 };
 
@@ -40,48 +47,54 @@ __device__ __forceinline__ void pair_words(const Geom& g, uint32_t q, uint32_t& 
   odd = (2u * row + 1u - c) * h + k;
 }
 
-// Thread: two neighbouring sites of a group's 64 samples, 2 bytes a sample, so
-// that a warp's access to a sample is 64 contiguous bytes.
+// Thread: four neighbouring sites of a group's 64 samples, 4 bytes a sample (N
+// is a multiple of 4), so that a warp's access to a sample is 128 contiguous bytes.
 __global__ void __launch_bounds__(256) k_bytes_to_words(const WordsParams p) {
-  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x, u = blockIdx.y, g = blockIdx.z;
-  if (q >= p.geom.half) return;
-  const int8_t* in = p.bytes + (uint64_t)g * 64u * p.sample_stride + u * p.unit_stride + 2u * q;
+  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x, g = blockIdx.z;
+  if (q >= p.geom.N / 4u) return;
+  const bool couplings = blockIdx.y >= p.part[0].units;
+  const WordsPart t = couplings ? p.part[1] : p.part[0];
+  const uint32_t u = couplings ? blockIdx.y - p.part[0].units : blockIdx.y;
+  const int8_t* in = t.bytes + (uint64_t)g * 64u * t.sample_stride + u * t.unit_stride + 4u * q;
   const int n = min(64, p.S - 64 * (int)g);
-  uint32_t e[2] = {0u, 0u}, o[2] = {0u, 0u};
+  uint32_t w[2][4] = {};  // half, site
 #pragma unroll
-  for (int w = 0; w < 2; ++w)
+  for (int hf = 0; hf < 2; ++hf)
 #pragma unroll 1
     for (int l0 = 0; l0 < 32; l0 += 16) {
       uint32_t v[16];  // 16 loads under way
 #pragma unroll
       for (int l = 0; l < 16; ++l) {
-        const int s = 32 * w + l0 + l;
-        v[l] = s < n ? *(const uint16_t*)(in + (uint64_t)s * p.sample_stride) : 0u;
+        const int s = 32 * hf + l0 + l;
+        v[l] = s < n ? *(const uint32_t*)(in + (uint64_t)s * t.sample_stride) : 0u;
       }
-      uint32_t be = 0, bo = 0;
 #pragma unroll
-      for (int l = 0; l < 16; ++l) {
-        be |= (v[l] >> 7 & 1u) << l;
-        bo |= (v[l] >> 15) << l;
+      for (int i = 0; i < 4; ++i) {
+        uint32_t b = 0;
+#pragma unroll
+        for (int l = 0; l < 16; ++l) b |= (v[l] >> (8 * i + 7) & 1u) << l;
+        w[hf][i] |= b << l0;
       }
-      e[w] |= be << l0;
-      o[w] |= bo << l0;
     }
-  uint32_t ie, io;
-  pair_words(p.geom, q, ie, io);
-  uint64_t* out = p.words + ((uint64_t)g * p.units + u) * p.geom.N;
-  out[ie] = (uint64_t)e[0] | (uint64_t)e[1] << 32;
-  out[io] = (uint64_t)o[0] | (uint64_t)o[1] << 32;
+  uint64_t* out = t.words + ((uint64_t)g * t.units + u) * p.geom.N;
+#pragma unroll
+  for (int i = 0; i < 4; i += 2) {
+    uint32_t ie, io;
+    pair_words(p.geom, 2u * q + (uint32_t)i / 2u, ie, io);
+    out[ie] = (uint64_t)w[0][i] | (uint64_t)w[1][i] << 32;
+    out[io] = (uint64_t)w[0][i + 1] | (uint64_t)w[1][i + 1] << 32;
+  }
 }
 
 __global__ void __launch_bounds__(256) k_words_to_bytes(const WordsParams p) {
   const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x, u = blockIdx.y, g = blockIdx.z;
   if (q >= p.geom.half) return;
+  const WordsPart& t = p.part[0];
   uint32_t ie, io;
   pair_words(p.geom, q, ie, io);
-  const uint64_t* in = p.words + ((uint64_t)g * p.units + u) * p.geom.N;
+  const uint64_t* in = t.words + ((uint64_t)g * t.units + u) * p.geom.N;
   const uint64_t we = in[ie], wo = in[io];
-  int8_t* out = p.bytes + (uint64_t)g * 64u * p.sample_stride + u * p.unit_stride + 2u * q;
+  int8_t* out = t.bytes + (uint64_t)g * 64u * t.sample_stride + u * t.unit_stride + 2u * q;
   const int n = min(64, p.S - 64 * (int)g);
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
@@ -91,52 +104,34 @@ __global__ void __launch_bounds__(256) k_words_to_bytes(const WordsParams p) {
       if (32 * w + l >= n) continue;
       // 1 or -1: 1 - 2 b in each byte
       const uint32_t v = (e >> l & 1u ? 0xFFu : 1u) | (o >> l & 1u ? 0xFF00u : 0x100u);
-      *(uint16_t*)(out + (uint64_t)(32 * w + l) * p.sample_stride) = (uint16_t)v;
+      *(uint16_t*)(out + (uint64_t)(32 * w + l) * t.sample_stride) = (uint16_t)v;
     }
   }
 }
 
-WordsParams params(const Lattice& lat, bool couplings) {
+WordsParams params(const Lattice& lat) {
   WordsParams p{};
   p.geom = lat.geom;
   p.S = lat.S;
-  if (couplings) {
-    p.bytes = (int8_t*)lat.J;
-    p.words = (uint64_t*)lat.words->J;
-    p.units = (uint32_t)lat.D;
-    p.sample_stride = (uint64_t)lat.D * lat.N;
-    p.unit_stride = lat.N;
-  } else {
-    p.bytes = (int8_t*)lat.spins;
-    p.words = (uint64_t*)lat.words->spins;
-    p.units = (uint32_t)lat.slots;
-    p.sample_stride = lat.N;
-    p.unit_stride = (uint64_t)lat.S * lat.N;
-  }
+  const uint64_t N = lat.N, S = (uint64_t)lat.S, D = (uint64_t)lat.D;
+  p.part[0] = WordsPart{(int8_t*)lat.spins, (uint64_t*)lat.words->spins, N, S * N, (uint32_t)lat.slots};
+  p.part[1] = WordsPart{(int8_t*)lat.J, (uint64_t*)lat.words->J, D * N, N, (uint32_t)lat.D};
   return p;
-}
-
-dim3 grid_of(const Lattice& lat, uint32_t units) {
-  return dim3((lat.geom.half + 255u) / 256u, units, (unsigned)(lat.S + 63) / 64u);
 }
 
 }  // namespace
 
-cudaError_t launch_pack_spins(Lattice& lat) {
-  const WordsParams p = params(lat, false);
-  k_bytes_to_words<<<grid_of(lat, p.units), 256, 0, lat.stream>>>(p);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pack_couplings(Lattice& lat) {
-  const WordsParams p = params(lat, true);
-  k_bytes_to_words<<<grid_of(lat, p.units), 256, 0, lat.stream>>>(p);
+cudaError_t launch_pack_words(Lattice& lat) {
+  const WordsParams p = params(lat);
+  const dim3 grid((lat.N / 4u + 255u) / 256u, p.part[0].units + p.part[1].units, (unsigned)(lat.S + 63) / 64u);
+  k_bytes_to_words<<<grid, 256, 0, lat.stream>>>(p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_spins(Lattice& lat) {
-  const WordsParams p = params(lat, false);
-  k_words_to_bytes<<<grid_of(lat, p.units), 256, 0, lat.stream>>>(p);
+  const WordsParams p = params(lat);
+  const dim3 grid((lat.geom.half + 255u) / 256u, p.part[0].units, (unsigned)(lat.S + 63) / 64u);
+  k_words_to_bytes<<<grid, 256, 0, lat.stream>>>(p);
   return cudaGetLastError();
 }
 

@@ -324,8 +324,7 @@ bool packed_i8_pays(const Lattice& lat, uint64_t nsweeps);
 cudaError_t launch_packed_i8(Lattice& lat, int inv, uint32_t nsweeps, uint32_t measure_every);
 // Plain lattices swept in words (k_words.cu): between lat's bytes and
 // lat.words', and whether a run of n sweeps is faster so.
-cudaError_t launch_pack_spins(Lattice& lat);
-cudaError_t launch_pack_couplings(Lattice& lat);
+cudaError_t launch_pack_words(Lattice& lat);  // spins and couplings
 cudaError_t launch_unpack_spins(Lattice& lat);
 bool words_pay(const Lattice& lat, uint64_t n);
 double plain_us(const Lattice& lat);  // estimated us of a plain sweep

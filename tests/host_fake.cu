@@ -192,12 +192,8 @@ cudaError_t launch_build_planes(Lattice& l) {
 }
 cudaError_t launch_set_tick(Lattice&, uint64_t, uint64_t, uint64_t) { return cudaSuccess; }
 cudaError_t launch_advance_tick(Lattice&, uint64_t, uint64_t, uint64_t) { return cudaSuccess; }
-cudaError_t launch_pack_spins(Lattice& l) {
-  op("pack_spins", l.stream);
-  return cudaSuccess;
-}
-cudaError_t launch_pack_couplings(Lattice& l) {
-  op("pack_couplings", l.stream);
+cudaError_t launch_pack_words(Lattice& l) {
+  op("pack_words", l.stream);
   return cudaSuccess;
 }
 cudaError_t launch_unpack_spins(Lattice& l) {
