@@ -63,9 +63,9 @@ TRAFFIC_SOURCE_HASH = "b79679f980ff4342"
 # on its L=32, 128 x 2 workload, from one ncu capture, valid while its
 # sources are unchanged: global loads through L1 (spin words, couplings, the
 # table once per block), L2 and DRAM bytes, L1 hit rate.
-POTTS_TRAFFIC = {"l1_global_load_bytes": 47693824, "l2_bytes": 52645728, "dram_bytes": 21001472,
+POTTS_TRAFFIC = {"l1_global_load_bytes": 47693824, "l2_bytes": 52665088, "dram_bytes": 21001472,
                  "l1_hit_rate_pct": 49.2}
-POTTS_SOURCE_HASH = "3db4924a81cef12c"
+POTTS_SOURCE_HASH = "c4977c8b45708dd1"
 # The kernel variant and launch shape the bench runs by default: the
 # lane-queue kernel in its one-wave launch (the automatic choice for one
 # temperature), fixed so that the profile above describes the timed kernel.
@@ -372,13 +372,13 @@ def run_gpu(args, ws, rank, local):
         ps = p0.elapsed_time(p1) / 1e3
         pv = S * R * L ** 3 * nps / (ps * 1e9)
         # roofline of the plain form: the smaller of two bounds.  HBM: the
-        # spins read as bytes and written as words before the run and back
-        # after it.  Issue: the per-lane-plane word update of the bit-sliced
+        # spins and couplings read as bytes and written as words before the run,
+        # the spins back after it.  Issue: the per-lane-plane word update of the bit-sliced
         # form / 64 (e-words 12, adder tree 16, "always" and undecided masks
         # 16, per plane the threshold multiplexers 6 + compare 4, per pair
         # Philox 18 + merge 2, 3.92 pairs; 16 mad.wide per Philox block)
         hbm = MEASURED.get("hbm_gbs")
-        b_upd = 2.25 / nps
+        b_upd = (2.25 + 1.125 * 3 / R) / nps
         npp = expected_plane_pairs()
         ops_upd = (44 + npp * (2 * 10 + 20) + npp * 16) / 64
         pk = _issue_peak()
@@ -534,9 +534,12 @@ def run_other_configs(args):
     upd = 128 * 2 * 32 ** 3 * 100 * reps
     rate = upd / (sec * 1e9)
     # per 4-sample word: Philox rounds 2..9 16 + merge 3 (and 16 mad.wide); the
-    # counts of the 4 samples as bytes of one word, 4 ops a neighbour; table rows
-    # 8; per sample 3 compares and selects (6) + pack (1)
-    alu_word = 19 + 6 * 4 + 8 + 4 * 7
+    # table rows as sums of digits: per direction the nibbles of both neighbours
+    # (2), their upper half (1) and 4 byte permutes, 4 three-input adds of the
+    # directions, the digits folded to 2 samples a word (16), masked (2) and taken
+    # apart (4); per sample 3 compares and selects (6) + pack (1); the largest of
+    # the 4 random words tested (4).  32-bit multiply-adds issue elsewhere
+    alu_word = 19 + 3 * 7 + 4 + 16 + 2 + 4 + 4 * 7 + 4
     upd_launch = 128 * 2 * 32 ** 3 // 2
     potts_traffic = None
     if kernel_source_hash(("common.cuh", "k_potts.cu", "potts_words.cuh")) == POTTS_SOURCE_HASH:
@@ -569,16 +572,17 @@ def run_other_configs(args):
     sec = timed(lambda: rf.sweep(ianus.HEATBATH, 1 / Tr, 100, 10), reps)
     upd = 256 * 64 ** 3 * 100 * reps
     rate = upd / (sec * 1e9)
-    # kernel specialised at run time for the field tables; per word: e-words
-    # 12, adder tree 16, f 2, "always"/"need" tables (u, f) 12, write-back 3;
-    # per plane: threshold bit 3 lop3 x 2 halves + compare 4; per pair Philox
-    # 21 ALU + merge 2; 3.92 plane pairs per word on average
-    alu_word = 45 + 3.92 * (2 * (6 + 4) + 23)
+    # lane-queue kernel specialised at run time for the field tables; per word:
+    # e-words 12, adder tree 16, f 2, flip 2; per plane: threshold bit 3 lop3 x 2
+    # halves + compare 4 (2 in plane 0, every lane undecided); per pair Philox
+    # rounds 2..9 16 ALU + 2 to merge the shared parts, and 16 mad.wide; the site
+    # key 1 ALU and 2 mad.wide; 3.92 plane pairs per word on average
+    alu_word = 12 + 16 + 2 + 2 - 2 + 1 + 3.92 * (2 * (6 + 4) + 18)
     out["rfim_L64_256_h1.5"] = {
         "updates_per_ns": rate, "ms_per_100_sweeps": sec * 1e3 / reps,
         "mode": "bit-sliced, field kernel specialised at run time ((u, f) tables as lop3 immediates), heat bath "
                 "T=2.0, |h|=1.5, E/M/F every 10 sweeps",
-        "roofline": issue_roof(alu_word, 3.92 * 20, 64, rate),
+        "roofline": issue_roof(alu_word, 3.92 * 16 + 2, 64, rate),
     }
     if not args.no_cpu_baseline:
         import oracle
@@ -599,17 +603,18 @@ def run_other_configs(args):
     sec = timed(lambda: da.sweep(ianus.METROPOLIS, 1 / Td, 100, 10), reps)
     upd = 256 * 64 ** 3 * 100 * reps
     rate = upd / (sec * 1e9)
-    # kernel specialised at run time; per word: e-words 12, occupied
-    # satisfied-bond words 12, occupation and bond count trees 32, the 4-bit
-    # sum t 10, f 2, "always"/"need" tables 28, write-back 4; per plane:
-    # threshold bit 7 lop3 x 2 halves + compare 4; per pair Philox 21 ALU +
-    # merge 2; 3.92 plane pairs per word on average (occupied lanes)
-    alu_word = 100 + 3.92 * (2 * (14 + 4) + 23)
+    # lane-queue kernel specialised at run time; per word: e-words 12, occupied
+    # satisfied-bond words 12, occupation and bond count trees 32, the 4-bit sum
+    # t 10, f 2, "always"/"need" tables 28 and occupation on both 4, flip 2; per
+    # plane: threshold bit 7 lop3 x 2 halves + compare 4; per pair Philox rounds
+    # 2..9 16 ALU + 2 to merge the shared parts, and 16 mad.wide; the site key 1
+    # ALU and 2 mad.wide; 3.92 plane pairs per word on average (occupied lanes)
+    alu_word = 12 + 12 + 32 + 10 + 2 + 28 + 4 + 2 + 1 + 3.92 * (2 * (14 + 4) + 18)
     out["daff_L64_256_occ0.7_h1.0"] = {
         "updates_per_ns": rate, "ms_per_100_sweeps": sec * 1e3 / reps,
         "mode": "bit-sliced with occupation words, kernel specialised at run time ((t, f) tables, t = v + 2D as "
                 "4 bit-planes), Metropolis T=1.5, |h|=1.0, occupation 0.7, E/M/F every 10 sweeps",
-        "roofline": issue_roof(alu_word, 3.92 * 20, 64, rate),
+        "roofline": issue_roof(alu_word, 3.92 * 16 + 2, 64, rate),
     }
     if not args.no_cpu_baseline:
         import oracle
@@ -683,10 +688,14 @@ def run_other_configs(args):
         sec = timed(lambda: pp.sweep(ianus.HEATBATH, bp, 100, 10), reps)
         upd = 256 * 2 * Lp ** dim * 100 * reps
         rate = upd / (sec * 1e9)
-        # per 4-sample word: Philox 19 (and 16 mad.wide); per bond 7 for the 4
-        # samples at once (target states by byte permutes, counts); table rows 8;
-        # per sample selection 6, pack 1
-        alu_word = 19 + 2 * dim * 7 + 8 + 4 * 7
+        # per 4-sample word: Philox 19 (and 16 mad.wide); per direction 15 for the 4
+        # samples at once: the forward target by two byte selects (8), its bits and
+        # their product (4), the backward target as one-hot fields (3); the row from
+        # their sums, 4 three-input adds, 4 for the fields' digits and 4 to take it
+        # apart (4D: 8 adds, 20 for two digits of 16 bits, 8); per sample selection 6,
+        # pack 1; the largest of the 4 random words tested (4).  32-bit multiply-adds
+        # issue elsewhere
+        alu_word = 19 + 15 * dim + (4 + 4 + 4 if dim == 3 else 8 + 20 + 8) + 4 * 7 + 4
         out[key] = {
             "updates_per_ns": rate, "ms_per_100_sweeps": sec * 1e3 / reps,
             "mode": f"4 samples per uint32 word, {dim}D, heat bath beta={bp}, E/Q every 10 sweeps",

@@ -531,7 +531,7 @@ ianus_status ianus_set_persistent_wait(ianus_lattice* lat, uint64_t timeout_ns, 
  * measured sweeps and tempering steps from graphs of whole cycles, captured
  * on a private stream when they are asked for again (by a later call, or by
  * several more replays in the same one) and dropped when the tables, the
- * variant or the launch shape change.  Captured kernels
+ * variant, the launch shape or the resident mode change.  Captured kernels
  * read the sweep index from device counters, so results are identical with
  * and without graphs.  enable = 0 launches every kernel directly. */
 ianus_status ianus_set_graphs(ianus_lattice* lat, int32_t enable);

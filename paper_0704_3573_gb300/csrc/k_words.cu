@@ -8,8 +8,11 @@
 // bytes for the run instead of several for every sweep.  Nothing is kept from
 // one run to the next, since a program may write either in the lattice's buffer.
 //
-// The sweep is the precompiled per-lane-plane kernel, which needs no run-time
-// compiler for a new temperature.  us per colour pass, 3D, heat bath (plain /
+// The sweep is the precompiled per-lane-plane kernel, so that a plain lattice never
+// waits for the run-time compiler (1.2 s for a geometry).  The lane-queue kernel
+// against per-lane planes (jit_sweep_lt.cuh) would also serve every temperature
+// once compiled, at 22 us for as many updates as the 38 us pass below (L=32, 64
+// samples x 2 x 32 temperatures, Metropolis).  us per colour pass, 3D, heat bath (plain /
 // words): L=64, 256 samples x 2 149 / 38; L=40, 100 x 2 33 / 8.7; L=100, 64 x 2
 // 288 / 39; L=16, 256 x 2 10.2 / 6.1; L=24, 20 samples 8.2 / 4.5.
 //
